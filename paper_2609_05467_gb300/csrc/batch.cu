@@ -16,7 +16,7 @@ namespace rc {
 
 rc_status point_order(rc_bvh h, const float* P, int64_t n, int32_t* order, cudaStream_t s);
 rc_status launch_batch(const BatchPart* d_parts, int n_parts, long long n_items, int ppi, const float4* tdirs,
-                       const rc_params* p, unsigned long long* work, cudaStream_t s);
+                       const rc_params* p, int64_t max_tris, unsigned long long* work, cudaStream_t s);
 rc_status prepare_batch_kernel(int n_dirs);
 rc_status device_dirs_for_cast(const rc_params* p, const float4** tdirs);
 rc_status check_params_public(const rc_params* p);
@@ -138,8 +138,10 @@ static rc_status prepare(rc_batch b, cudaStream_t s)
     const int ppi = b->p.points_per_item > 0 ? b->p.points_per_item : 1;
     std::vector<BatchPart> hp(np);
     long long first = 0;
+    int64_t max_tris = 0;
     for (int k = 0; k < np; ++k) {
         HostPart& q = b->parts[k];
+        max_tris = std::max(max_tris, q.h->T);
         if (b->p.point_order == 0 && !q.order && q.n > 1) {
             RC_CUDA(cudaMalloc(&q.order, sizeof(int32_t) * q.n));
             rc_status st = point_order(q.h, q.P, q.n, q.order, s);
@@ -213,7 +215,7 @@ static rc_status prepare(rc_batch b, cudaStream_t s)
     if (nbr > 0 && cudaEventRecord(b->fork_ev, cs) != cudaSuccess) lst = set_error(RC_E_CUDA, "fork");
     for (int j = 0; j < nbr && lst == RC_OK; ++j)
         if (cudaStreamWaitEvent(b->branch[j], b->fork_ev, 0) != cudaSuccess) lst = set_error(RC_E_CUDA, "fork");
-    if (lst == RC_OK) lst = launch_batch(b->d_parts, np, b->n_items, ppi, tdirs, &b->p, b->d_work, cs);
+    if (lst == RC_OK) lst = launch_batch(b->d_parts, np, b->n_items, ppi, tdirs, &b->p, max_tris, b->d_work, cs);
     if (lst == RC_OK && nbr > 0 && cudaEventRecord(b->cast_ev, cs) != cudaSuccess) lst = set_error(RC_E_CUDA, "cast");
     for (int pass = 0; pass < 2 && lst == RC_OK; ++pass)
     for (int k = 0; k < np && lst == RC_OK; ++k) {

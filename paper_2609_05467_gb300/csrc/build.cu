@@ -596,11 +596,11 @@ __device__ __forceinline__ int32_t encode_child(int32_t c, int64_t n_int, const 
 {
     if (c >= n_int) {
         const int32_t first = (int32_t)(c - n_int);
-        return -1 - (first * 8 + 0);
+        return leaf_code(first, 1);
     }
     const int32_t lo = range[2 * c], hi = range[2 * c + 1];
     const int32_t cnt = hi - lo + 1;
-    if (cnt <= kLeafMax) return -1 - (lo * 8 + (cnt - 1));
+    if (cnt <= kLeafMax) return leaf_code(lo, cnt);
     return c;
 }
 
@@ -682,17 +682,16 @@ __device__ __forceinline__ void wide_write(float4* wnodes, int32_t w, const floa
             ix[k] = -1;
         }
     }
-    float4* nd = wnodes + 8 * (int64_t)w;
-    nd[0] = make_float4(lo[0][0], lo[0][1], lo[0][2], lo[0][3]);
-    nd[1] = make_float4(hi[0][0], hi[0][1], hi[0][2], hi[0][3]);
-    nd[2] = make_float4(lo[1][0], lo[1][1], lo[1][2], lo[1][3]);
-    nd[3] = make_float4(hi[1][0], hi[1][1], hi[1][2], hi[1][3]);
-    nd[4] = make_float4(lo[2][0], lo[2][1], lo[2][2], lo[2][3]);
-    nd[5] = make_float4(hi[2][0], hi[2][1], hi[2][2], hi[2][3]);
-    nd[6] = make_float4(__int_as_float(ix[0]), __int_as_float(ix[1]), __int_as_float(ix[2]), __int_as_float(ix[3]));
+    wnodes[wide_at(w, 0)] = make_float4(lo[0][0], lo[0][1], lo[0][2], lo[0][3]);
+    wnodes[wide_at(w, 1)] = make_float4(hi[0][0], hi[0][1], hi[0][2], hi[0][3]);
+    wnodes[wide_at(w, 2)] = make_float4(lo[1][0], lo[1][1], lo[1][2], lo[1][3]);
+    wnodes[wide_at(w, 3)] = make_float4(hi[1][0], hi[1][1], hi[1][2], hi[1][3]);
+    wnodes[wide_at(w, 4)] = make_float4(lo[2][0], lo[2][1], lo[2][2], lo[2][3]);
+    wnodes[wide_at(w, 5)] = make_float4(hi[2][0], hi[2][1], hi[2][2], hi[2][3]);
+    wnodes[wide_at(w, 6)] = make_float4(__int_as_float(ix[0]), __int_as_float(ix[1]), __int_as_float(ix[2]), __int_as_float(ix[3]));
     // the binary nodes the children were made from (-1: empty slot), for
     // the boxes of the same tree in another coordinate frame
-    nd[7] = make_float4(__int_as_float(nch > 0 ? ch[0] : -1), __int_as_float(nch > 1 ? ch[1] : -1),
+    wnodes[wide_at(w, 7)] = make_float4(__int_as_float(nch > 0 ? ch[0] : -1), __int_as_float(nch > 1 ? ch[1] : -1),
                         __int_as_float(nch > 2 ? ch[2] : -1), __int_as_float(nch > 3 ? ch[3] : -1));
 }
 
@@ -791,7 +790,7 @@ __global__ void k_wide_small(int64_t T, const float* __restrict__ tbox, float4* 
     wnodes[3] = make_float4(hi[1], -I, -I, -I);
     wnodes[4] = make_float4(lo[2], I, I, I);
     wnodes[5] = make_float4(hi[2], -I, -I, -I);
-    wnodes[6] = make_float4(__int_as_float(-1 - (int)(T - 1)), __int_as_float(-1), __int_as_float(-1),
+    wnodes[6] = make_float4(__int_as_float(leaf_code(0, (int)T)), __int_as_float(-1), __int_as_float(-1),
                             __int_as_float(-1));
     wnodes[7] = make_float4(__int_as_float(kAllTris), __int_as_float(-1), __int_as_float(-1), __int_as_float(-1));
     sc->wide_depth = 1;
@@ -822,7 +821,7 @@ __global__ void k_pack_small(int64_t T, const float* __restrict__ tbox, float4* 
     nodes[0] = make_float4(lo[0], hi[0], lo[1], hi[1]);
     nodes[1] = make_float4(INFINITY, -INFINITY, INFINITY, -INFINITY);
     nodes[2] = make_float4(lo[2], hi[2], INFINITY, -INFINITY);
-    nodes[3] = make_float4(__int_as_float(-1 - (0 * 8 + (int)(T - 1))), __int_as_float(-1), 0.0f, 0.0f);
+    nodes[3] = make_float4(__int_as_float(leaf_code(0, (int)T)), __int_as_float(-1), 0.0f, 0.0f);
 }
 
 __global__ void k_tri_records(const float* __restrict__ V, int64_t nV, const int32_t* __restrict__ F,
@@ -1298,8 +1297,7 @@ __global__ void k_frame_pack(const float4* __restrict__ wnodes, int64_t n_int, i
 {
     const int64_t w = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (w >= sc->wide_nodes || w >= n_int) return;
-    const float4* nd = wnodes + 8 * w;
-    const float4 idv = nd[7];
+    const float4 idv = wnodes[wide_at(w, 7)];
     const int32_t ids[4] = {__float_as_int(idv.x), __float_as_int(idv.y), __float_as_int(idv.z), __float_as_int(idv.w)};
     float lo[3][4], hi[3][4];
     for (int k = 0; k < 4; ++k) {
@@ -1311,13 +1309,12 @@ __global__ void k_frame_pack(const float4* __restrict__ wnodes, int64_t n_int, i
             hi[a][k] = b ? b[3 + a] : -INFINITY;
         }
     }
-    float4* o = ftree + 8 * w;
     for (int a = 0; a < 3; ++a) {
-        o[2 * a] = make_float4(lo[a][0], lo[a][1], lo[a][2], lo[a][3]);
-        o[2 * a + 1] = make_float4(hi[a][0], hi[a][1], hi[a][2], hi[a][3]);
+        ftree[wide_at(w, 2 * a)] = make_float4(lo[a][0], lo[a][1], lo[a][2], lo[a][3]);
+        ftree[wide_at(w, 2 * a + 1)] = make_float4(hi[a][0], hi[a][1], hi[a][2], hi[a][3]);
     }
-    o[6] = nd[6];
-    o[7] = idv;
+    ftree[wide_at(w, 6)] = wnodes[wide_at(w, 6)];
+    ftree[wide_at(w, 7)] = idv;
 }
 
 // box of all leaf slots [0, T) of nbox_f (tiny parts: the one-leaf root)

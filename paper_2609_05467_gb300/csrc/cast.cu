@@ -16,7 +16,7 @@
 // distance by 1 + 2*gamma_3 (Ize, JCGT 2013).
 //
 // Kernels: k_hemisphere (the default cast: persistent warps, one point per
-// warp in tiles of 32 directions, the last points in parts),
+// warp, its rays' walks pooled in shared memory, the last points in parts),
 // k_hemisphere_update (re-cast after an edit), k_batch (many parts in one
 // launch), k_orthogonal_axis (one frame axis for 32 points per work item),
 // k_tool_cast_axis (the sampled ball-end tool), and the frame set-up
@@ -154,9 +154,10 @@ __device__ __forceinline__ int tri_test32(const Ray& r, const float4 v0, const f
 // sign decision (used for rays that only ambiguous pairs decide).
 struct Pair64 { int state; bool hit64; };
 
-__device__ __noinline__ Pair64 retest64(const Ray& r, const float4 v0, const float4 v1, const float4 v2)
+__device__ __noinline__ Pair64 retest64(float ox, float oy, float oz, float dx, float dy, float dz, const float4 v0,
+                                        const float4 v1, const float4 v2)
 {
-    const double o[3] = {r.ox, r.oy, r.oz}, d[3] = {r.dx, r.dy, r.dz};
+    const double o[3] = {ox, oy, oz}, d[3] = {dx, dy, dz};
     const double A[3] = {v0.x, v0.y, v0.z}, B[3] = {v1.x, v1.y, v1.z}, C[3] = {v2.x, v2.y, v2.z};
     double a[3], b[3], c[3], eab[3], ebc[3], eca[3];
     double R = 1.0;
@@ -211,6 +212,11 @@ __device__ __noinline__ Pair64 retest64(const Ray& r, const float4 v0, const flo
     return res;
 }
 
+__device__ __forceinline__ Pair64 retest64(const Ray& r, const float4 v0, const float4 v1, const float4 v2)
+{
+    return retest64(r.ox, r.oy, r.oz, r.dx, r.dy, r.dz, v0, v1, v2);
+}
+
 // Conservative slab test of both children of a packed node.
 __device__ __forceinline__ void box2(const Ray& r, const float4 n0, const float4 n1, const float4 n2,
                                      bool& h0, bool& h1, float& t0, float& t1)
@@ -238,7 +244,7 @@ __device__ __forceinline__ void box2(const Ray& r, const float4 n0, const float4
 // Per-warp-lane counters of a cast.
 struct CastAccFwd {
     int amb = 0, retests = 0, overflow = 0;
-    long long rays = 0, nvis = 0, ntri = 0;
+    long long rays = 0, nvis = 0, ntri = 0, nbox = 0;
 };
 
 // Result bits of trace(): bit 0 blocked, bit 1 decided by ambiguous pairs.
@@ -279,8 +285,7 @@ __device__ __forceinline__ TraceOut trace(const float4* __restrict__ nodes, cons
             if (h0) { cur = c0; continue; }
             if (h1) { cur = c1; continue; }
         } else {
-            const int v = -1 - cur;
-            const int first = v >> 3, cnt = (v & 7) + 1;
+            const int first = leaf_first(cur), cnt = leaf_count(cur);
             for (int k = 0; k < cnt; ++k) {
                 const float4* t = tris + 3 * (first + k);
                 const float4 v0 = __ldg(t), v1 = __ldg(t + 1), v2 = __ldg(t + 2);
@@ -342,23 +347,27 @@ __device__ __forceinline__ SlabRay make_slab_ray(const Ray& r, float M)
     return s;
 }
 
-// Slab test of the four children of wide node nd: d[k] = entry distance of a
-// hit child (else +inf), c[k] = child index; returns the number of hits.
-// kShared: nd is a frontier group in shared memory (the same layout).
-template <bool kShared = false>
-__device__ __forceinline__ float4 node_ld(const float4* p)
+// Where wide node w's float4s start to be read, and float4 c of it: trees are
+// allocated on 256-byte boundaries, so wide_at is one exclusive or on the
+// address.
+__device__ __forceinline__ const float4* wide_ptr(const float4* __restrict__ tree, int w)
 {
-    if (kShared) return *p;
-    return __ldg(p);
+    return (const float4*)((const char*)tree + (((size_t)(unsigned)w << 7) | (((unsigned)w & 7u) << 4)));
+}
+__device__ __forceinline__ float4 wide_ld(const float4* nd, int c)
+{
+    return __ldg((const float4*)((uintptr_t)nd ^ (uintptr_t)(c << 4)));
 }
 
-template <bool kShared = false>
-__device__ __forceinline__ int slab4(const float4* __restrict__ nd, const SlabRay& s, float d[4], int c[4])
+// Slab test of the four children of wide node w: d[k] = entry distance of a
+// hit child (else +inf), c[k] = child index; returns the number of hits.
+__device__ __forceinline__ int slab4(const float4* __restrict__ wnodes, int w, const SlabRay& s, float d[4], int c[4])
 {
-    const float4 nxv = node_ld<kShared>(nd + 0 + s.offx), fxv = node_ld<kShared>(nd + 1 - s.offx);
-    const float4 nyv = node_ld<kShared>(nd + 2 + s.offy), fyv = node_ld<kShared>(nd + 3 - s.offy);
-    const float4 nzv = node_ld<kShared>(nd + 4 + s.offz), fzv = node_ld<kShared>(nd + 5 - s.offz);
-    const float4 ci = node_ld<kShared>(nd + 6);
+    const float4* nd = wide_ptr(wnodes, w);
+    const float4 nxv = wide_ld(nd, s.offx), fxv = wide_ld(nd, 1 - s.offx);
+    const float4 nyv = wide_ld(nd, 2 + s.offy), fyv = wide_ld(nd, 3 - s.offy);
+    const float4 nzv = wide_ld(nd, 4 + s.offz), fzv = wide_ld(nd, 5 - s.offz);
+    const float4 ci = wide_ld(nd, 6);
     const float nx[4] = {nxv.x, nxv.y, nxv.z, nxv.w}, fx[4] = {fxv.x, fxv.y, fxv.z, fxv.w};
     const float ny[4] = {nyv.x, nyv.y, nyv.z, nyv.w}, fy[4] = {fyv.x, fyv.y, fyv.z, fyv.w};
     const float nz[4] = {nzv.x, nzv.y, nzv.z, nzv.w}, fz[4] = {fzv.x, fzv.y, fzv.z, fzv.w};
@@ -388,27 +397,32 @@ __device__ __forceinline__ int slab4(const float4* __restrict__ nd, const SlabRa
 // The warp finds that set once per point and keeps in shared memory what
 // each ray must still decide for itself: the triangles of the leaves whose
 // boxes contain o (local triangles), and the children of origin-set nodes
-// whose boxes do not contain o (the frontier, in the wide node's layout,
-// four entries per group).  A ray tests the local triangles, tests every
-// frontier box with its own slab test and walks the subtrees it enters:
-// exactly the triangles its walk from the root would test, so the same
-// decisions.  A local triangle wholly below the point's tangent plane is
-// dropped, because a hemisphere ray leaves that plane (d.n > 0 for every
-// direction of the set, N <= 65536, when n is of unit length to within the
-// rounding of an fp32 normal) and meets no point of it at t > 0; that
+// whose boxes do not contain o (the frontier).  A ray tests the local
+// triangles, tests the frontier boxes with its own slab test and walks the
+// subtrees it enters: the triangles its walk from the root would test, so
+// the same decisions.  A local triangle wholly below the point's tangent
+// plane is dropped, because a hemisphere ray leaves that plane (d.n > 0 for
+// every direction of the set, N <= 65536, when n is of unit length to within
+// the rounding of an fp32 normal) and meets no point of it at t > 0; that
 // exact FP64 test runs once per point.  For the same reason a frontier box
 // wholly below the plane is dropped, and so is a frontier leaf whose
-// triangles all lie below it (conservative fp32 tests).  A point whose frontier or local
-// triangles do not fit walks from the root instead.
+// triangles all lie below it (conservative fp32 tests).  Large boxes then
+// make way for their children's while there is room (see build_frontier),
+// and the boxes are sorted by distance.  What finds no room stays whole, as
+// a frontier box that every ray enters.
 // ---------------------------------------------------------------------------
-constexpr int kFrontGroups = 16;   // frontier entries, four per group
-constexpr int kFrontTris = 12;     // local triangles kept per point
-constexpr int kStackF = kStack4 + 4 * kFrontGroups;
+// 64 boxes: of the impeller's points 1 in 800 has more.  96 and 128 measured
+// within 2% of 64 (fewer walk steps, less L1 left beside the shared memory).
+constexpr int kFrontEntries = 64;                // frontier boxes kept per point
+constexpr int kFrontTris = 8;                    // local triangles kept per point
+constexpr int kFrontRounds = 8;                  // most rounds of growth, eight boxes each
+constexpr int kFrontWords = kFrontEntries / 32;  // boxes per lane
+static_assert(kFrontEntries % 32 == 0 && kFrontEntries <= 128, "a lane looks at whole words of boxes; a list of bytes");
 
 struct Frontier {
-    float4 grp[kFrontGroups * 7];  // per group: lo.x, hi.x, lo.y, hi.y, lo.z, hi.z of 4 entries, their codes
+    float4 box[2 * kFrontEntries]; // per entry: lo xyz and its code, hi xyz
     float4 tri[kFrontTris * 3];    // local triangle records
-    int ngroups, ntris, ok, nvis;
+    int nboxes, ntris, nvis;
 };
 
 // n . (v - o) < 0 for the three vertices, in FP64: the differences of fp32
@@ -447,134 +461,251 @@ __device__ __forceinline__ bool box_below_tangent(float lx, float hx, float ly, 
     return (mx + my) + mz < -8.0f * u * (fabsf(mx) + fabsf(my) + fabsf(mz));
 }
 
-// Lane 0 of the warp: the origin set of o (a walk over the boxes that
-// contain o), its frontier and local triangles into *f.
-__device__ __noinline__ void build_frontier(const float4* __restrict__ wnodes, const float4* __restrict__ tris,
-                                            int max_steps, float ox, float oy, float oz, float nx, float ny,
-                                            float nz, bool drop, Frontier* f)
+// Component c (0..5: lo.x, hi.x, lo.y, hi.y, lo.z, hi.z; 6: code) of child k
+// of a wide node.
+__device__ __forceinline__ float child_ld(const float4* __restrict__ wnodes, int w, int c, int k)
 {
-    int qs[kStack4];
-    int qsp = 0;
-    qs[qsp++] = 0;
-    int ne = 0, nt = 0, nvis = 0;
-    bool ok = true;
-    float* g = (float*)f->grp;
-    while (qsp > 0 && ok) {
-        if (++nvis > max_steps) { ok = false; break; }
-        const int cur = qs[--qsp];
-        const float4* nd = wnodes + 8 * (int64_t)cur;
-        const float4 lxv = __ldg(nd), hxv = __ldg(nd + 1), lyv = __ldg(nd + 2), hyv = __ldg(nd + 3);
-        const float4 lzv = __ldg(nd + 4), hzv = __ldg(nd + 5), civ = __ldg(nd + 6);
-        const float LX[4] = {lxv.x, lxv.y, lxv.z, lxv.w}, HX[4] = {hxv.x, hxv.y, hxv.z, hxv.w};
-        const float LY[4] = {lyv.x, lyv.y, lyv.z, lyv.w}, HY[4] = {hyv.x, hyv.y, hyv.z, hyv.w};
-        const float LZ[4] = {lzv.x, lzv.y, lzv.z, lzv.w}, HZ[4] = {hzv.x, hzv.y, hzv.z, hzv.w};
-        const int CI[4] = {__float_as_int(civ.x), __float_as_int(civ.y), __float_as_int(civ.z), __float_as_int(civ.w)};
-        for (int k = 0; k < 4 && ok; ++k) {
-            if (!(LX[k] <= HX[k])) continue;   // empty slot (its code -1 is also a leaf's)
-            const bool inside = LX[k] <= ox && ox <= HX[k] && LY[k] <= oy && oy <= HY[k] && LZ[k] <= oz &&
-                                oz <= HZ[k];
-            if (inside && CI[k] >= 0) {
-                if (qsp >= kStack4) { ok = false; break; }
-                qs[qsp++] = CI[k];
-            } else if (inside) {
-                const int v = -1 - CI[k], first = v >> 3, cnt = (v & 7) + 1;
-                for (int t = 0; t < cnt; ++t) {
-                    const float4* tp = tris + 3 * (int64_t)(first + t);
-                    const float4 v0 = __ldg(tp), v1 = __ldg(tp + 1), v2 = __ldg(tp + 2);
-                    if (drop && below_tangent(v0, ox, oy, oz, nx, ny, nz) &&
-                        below_tangent(v1, ox, oy, oz, nx, ny, nz) && below_tangent(v2, ox, oy, oz, nx, ny, nz))
-                        continue;
-                    if (nt >= kFrontTris) { ok = false; break; }
-                    f->tri[3 * nt] = v0;
-                    f->tri[3 * nt + 1] = v1;
-                    f->tri[3 * nt + 2] = v2;
-                    ++nt;
-                }
-            } else {
-                // a box below the tangent plane holds no hit of any ray of the
-                // point, and neither does a leaf whose triangles all lie below it
-                if (drop && box_below_tangent(LX[k], HX[k], LY[k], HY[k], LZ[k], HZ[k], ox, oy, oz, nx, ny, nz))
-                    continue;
-                if (drop && CI[k] < 0) {
-                    const int v = -1 - CI[k], first = v >> 3, cnt = (v & 7) + 1;
-                    bool below = true;
-                    for (int t = 0; t < cnt && below; ++t) {
-                        const float4* tp = tris + 3 * (int64_t)(first + t);
-                        for (int q = 0; q < 3 && below; ++q) {
-                            const float4 w = __ldg(tp + q);
-                            below = box_below_tangent(w.x, w.x, w.y, w.y, w.z, w.z, ox, oy, oz, nx, ny, nz);
-                        }
-                    }
-                    if (below) continue;
-                }
-                if (ne >= 4 * kFrontGroups) { ok = false; break; }
-                float* gp = g + 28 * (ne >> 2) + (ne & 3);
-                gp[0] = LX[k]; gp[4] = HX[k]; gp[8] = LY[k]; gp[12] = HY[k]; gp[16] = LZ[k]; gp[20] = HZ[k];
-                gp[24] = __int_as_float(CI[k]);
-                ++ne;
-            }
-        }
-    }
-    // the last group's unused slots: empty boxes, which no slab test enters
-    for (int e = ne; e < ((ne + 3) & ~3); ++e) {
-        float* gp = g + 28 * (e >> 2) + (e & 3);
-        gp[0] = INFINITY; gp[4] = -INFINITY; gp[8] = INFINITY; gp[12] = -INFINITY; gp[16] = INFINITY;
-        gp[20] = -INFINITY;
-        gp[24] = __int_as_float(-1);
-    }
-    f->ngroups = (ne + 3) >> 2;
-    f->ntris = nt;
-    f->ok = ok ? 1 : 0;
-    f->nvis = nvis;
+    return __ldg((const float*)(wnodes + wide_at(w, c)) + k);
 }
 
-template <bool kStats>
-__device__ __forceinline__ TraceOut trace4(const float4* __restrict__ wnodes, const float4* __restrict__ tris,
-                                           const Ray& r, int max_steps, const Frontier* front = nullptr)
+// the smallest and largest value over the warp
+__device__ __forceinline__ float warp_min(float x)
 {
-    TraceOut out = {0, 0, 0, 0, 0};
-    int stack[kStackF];
-    int sp = 0;
-    int cur = 0;
-    bool amb = false, ambhit = false;
-    const SlabRay sr = make_slab_ray(r, r.rs);
-    if (front) {
-        // the point's local triangles, then its frontier boxes: the entered
-        // ones go on the stack, the deepest (nearest the origin) on top
-        for (int t = 0; t < front->ntris; ++t) {
-            const float4 v0 = front->tri[3 * t], v1 = front->tri[3 * t + 1], v2 = front->tri[3 * t + 2];
-            if (kStats) ++out.tris;
-            const int st = tri_test32(r, v0, v1, v2);
-            if (st == kHit) { out.flags = 1; return out; }
-            if (st == kUnsure) {
-                ++out.retests;
-                const Pair64 p = retest64(r, v0, v1, v2);
-                if (p.state == kHit) { out.flags = 1; return out; }
-                if (p.state == kUnsure) { amb = true; ambhit |= p.hit64; }
+    float r;
+    asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float warp_max(float x)
+{
+    float r;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// The warp builds the point's frontier: the origin set of o (the nodes whose
+// boxes contain o) is walked level by level, up to eight nodes at a time, a
+// lane per child; `queue` (shared, kFrontQueue ints) holds the nodes visited
+// and to be visited.  A node or leaf for which there is no room stays whole:
+// a frontier box that every ray enters.
+constexpr int kFrontQueue = 256;
+
+__device__ __noinline__ void build_frontier(const float4* __restrict__ wnodes, const float4* __restrict__ tris,
+                                            float ox, float oy, float oz, float nx, float ny, float nz, bool drop,
+                                            float theta2, int rounds, Frontier* f, int* queue)
+{
+    constexpr unsigned kAll = 0xFFFFFFFFu;
+    const int lane = threadIdx.x & 31;
+    const unsigned below = (1u << lane) - 1u;
+    int head = 0, tail = 1, ne = 0, nt = 0;
+    if (lane == 0) queue[0] = 0;
+    __syncwarp();
+    while (head < tail && tail + 32 <= kFrontQueue) {
+        const int m = min(8, tail - head), k = lane & 3;
+        const bool on = (lane >> 2) < m;
+        const int nd = queue[on ? head + (lane >> 2) : head];
+        const float lx = child_ld(wnodes, nd, 0, k), hx = child_ld(wnodes, nd, 1, k), ly = child_ld(wnodes, nd, 2, k);
+        const float hy = child_ld(wnodes, nd, 3, k), lz = child_ld(wnodes, nd, 4, k), hz = child_ld(wnodes, nd, 5, k);
+        const int code = __float_as_int(child_ld(wnodes, nd, 6, k));
+        head += m;
+        const bool box = on && lx <= hx;   // an empty slot has an empty box (its code -1 is also a leaf's)
+        const bool in = box && lx <= ox && ox <= hx && ly <= oy && oy <= hy && lz <= oz && oz <= hz;
+        bool out = box && !in;
+        // a box below the tangent plane holds no hit of any ray of the point
+        if (out && drop && box_below_tangent(lx, hx, ly, hy, lz, hz, ox, oy, oz, nx, ny, nz)) out = false;
+        // leaves: a triangle of one that contains o becomes a local triangle
+        // unless it lies below the plane (FP64); one that does not is dropped
+        // when all its triangles do (fp32)
+        const int first = leaf_first(code), cnt = box && code < 0 && (in || (out && drop)) ? leaf_count(code) : 0;
+        bool above = !(out && drop && code < 0);
+        const int nt0 = nt;
+        for (int q = 0; __any_sync(kAll, q < cnt); ++q) {
+            bool keep = false;
+            float4 v0, v1, v2;
+            if (q < cnt) {
+                const float4* tp = tris + 3 * (int64_t)(first + q);
+                v0 = __ldg(tp);
+                v1 = __ldg(tp + 1);
+                v2 = __ldg(tp + 2);
+                if (in)
+                    keep = !(drop && below_tangent(v0, ox, oy, oz, nx, ny, nz) &&
+                             below_tangent(v1, ox, oy, oz, nx, ny, nz) && below_tangent(v2, ox, oy, oz, nx, ny, nz));
+                else
+                    above |= !(box_below_tangent(v0.x, v0.x, v0.y, v0.y, v0.z, v0.z, ox, oy, oz, nx, ny, nz) &&
+                               box_below_tangent(v1.x, v1.x, v1.y, v1.y, v1.z, v1.z, ox, oy, oz, nx, ny, nz) &&
+                               box_below_tangent(v2.x, v2.x, v2.y, v2.y, v2.z, v2.z, ox, oy, oz, nx, ny, nz));
+            }
+            const unsigned mt = __ballot_sync(kAll, keep);
+            if (keep && nt + __popc(mt & below) < kFrontTris) {
+                const int at = 3 * (nt + __popc(mt & below));
+                f->tri[at] = v0;
+                f->tri[at + 1] = v1;
+                f->tri[at + 2] = v2;
+            }
+            nt += __popc(mt);
+        }
+        // no room for their triangles: these leaves stay whole, as boxes
+        // that every ray enters
+        const bool whole_leaf = nt > kFrontTris && in && code < 0;
+        if (nt > kFrontTris) nt = nt0;
+        const unsigned mq = __ballot_sync(kAll, in && code >= 0);
+        const bool entry = (out && above) || whole_leaf;
+        const unsigned me = __ballot_sync(kAll, entry);
+        if (ne + __popc(me) + (tail - head) + __popc(mq) > kFrontEntries) {
+            // no room: these nodes stay whole, and so do those still queued
+            nt = nt0;
+            head -= m;
+            break;
+        }
+        if (in && code >= 0) queue[tail + __popc(mq & below)] = code;
+        tail += __popc(mq);
+        if (entry) {
+            const int at = 2 * (ne + __popc(me & below));
+            f->box[at] = make_float4(lx, ly, lz, __int_as_float(code));
+            f->box[at + 1] = make_float4(hx, hy, hz, 0.0f);
+        }
+        ne += __popc(me);
+        __syncwarp();
+    }
+    const int visited = head;
+    for (; head < tail; head += 32) {
+        if (lane < tail - head) {
+            const int at = 2 * (ne + lane);
+            f->box[at] = make_float4(-INFINITY, -INFINITY, -INFINITY, __int_as_float(queue[head + lane]));
+            f->box[at + 1] = make_float4(INFINITY, INFINITY, INFINITY, 0.0f);
+        }
+        ne += min(32, tail - head);
+    }
+    __syncwarp();
+    // Boxes that look large from o make way for their children's while there
+    // is room.  Testing a tile's rays against a box costs about as much as
+    // three (ray, node) pairs of the walk, and a tile first drops the boxes
+    // it cannot meet, so a box is worth it down to the angle at which each of
+    // its children is met by a few rays (theta2 = 20 / N steradian; the room
+    // runs out first nearly always).  A round costs a point about what a
+    // tenth of a tile does, hence the fewer rounds the fewer tiles.  Measured
+    // (100k points): impeller 35.4 -> 32.4 ms, housing 6.72 -> 6.11 ms at
+    // 2048 and 1024 directions; with 8 rounds at 150 directions 2.91 -> 3.31.
+    int grown = 0;
+    for (int round = 0; round < rounds && kFrontEntries - ne >= 3; ++round) {
+        float r[kFrontWords], most = 0.0f;
+#pragma unroll
+        for (int q = 0; q < kFrontWords; ++q) {
+            const int e = 32 * q + lane;
+            r[q] = 0.0f;
+            if (e < ne) {
+                const float4 lo = f->box[2 * e], hi = f->box[2 * e + 1];
+                const float dx = fmaxf(fmaxf(lo.x - ox, ox - hi.x), 0.0f), dy = fmaxf(fmaxf(lo.y - oy, oy - hi.y), 0.0f),
+                            dz = fmaxf(fmaxf(lo.z - oz, oz - hi.z), 0.0f);
+                const float ext = fmaxf(hi.x - lo.x, fmaxf(hi.y - lo.y, hi.z - lo.z));
+                if (__float_as_int(lo.w) >= 0 && ext > 0.0f && ext < INFINITY)
+                    r[q] = ext * ext / (dx * dx + dy * dy + dz * dz + 1e-30f);
+            }
+            most = fmaxf(most, r[q]);
+        }
+        most = warp_max(most);
+        const float least = fmaxf(theta2, 0.25f * most);
+        const int room = min(8, (kFrontEntries - ne) / 3);
+        int m = 0;
+#pragma unroll
+        for (int q = 0; q < kFrontWords; ++q) {
+            const unsigned b = __ballot_sync(kAll, r[q] > least);
+            const int at = m + __popc(b & below);
+            if (r[q] > least && at < room) queue[at] = 32 * q + lane;
+            m += __popc(b);
+        }
+        m = min(m, room);
+        if (m == 0) break;
+        __syncwarp();
+        const int k = lane & 3;
+        const bool on = (lane >> 2) < m;
+        const int nd = __float_as_int(f->box[2 * queue[on ? lane >> 2 : 0]].w);
+        const float lx = child_ld(wnodes, nd, 0, k), hx = child_ld(wnodes, nd, 1, k), ly = child_ld(wnodes, nd, 2, k);
+        const float hy = child_ld(wnodes, nd, 3, k), lz = child_ld(wnodes, nd, 4, k), hz = child_ld(wnodes, nd, 5, k);
+        const int code = __float_as_int(child_ld(wnodes, nd, 6, k));
+        const bool keep = on && lx <= hx &&
+                          !(drop && box_below_tangent(lx, hx, ly, hy, lz, hz, ox, oy, oz, nx, ny, nz));
+        const unsigned mk = __ballot_sync(kAll, keep);
+        __syncwarp();
+        // the children take their parents' places, then new ones; a place
+        // left over holds a box that no ray meets
+        const int rank = __popc(mk & below), at = rank < m ? queue[rank] : ne + rank - m;
+        const int spare = lane >= __popc(mk) && lane < m ? queue[lane] : -1;
+        __syncwarp();
+        if (keep) {
+            f->box[2 * at] = make_float4(lx, ly, lz, __int_as_float(code));
+            f->box[2 * at + 1] = make_float4(hx, hy, hz, 0.0f);
+        }
+        if (spare >= 0) {
+            f->box[2 * spare] = make_float4(1e30f, 1e30f, 1e30f, __int_as_float(-1));
+            f->box[2 * spare + 1] = make_float4(-1e30f, -1e30f, -1e30f, 0.0f);
+        }
+        ne += max(0, __popc(mk) - m);
+        grown += m;
+        __syncwarp();
+    }
+    if (grown) {
+        // nearest last: the boxes are tested from the end (in the order of
+        // growth the impeller took 40.1 ms instead of 32.4, farthest first 59)
+        float* key = (float*)queue;
+        float4 lo[kFrontWords], hi[kFrontWords];
+        float d[kFrontWords];
+        int at[kFrontWords];
+#pragma unroll
+        for (int q = 0; q < kFrontWords; ++q) {
+            const int e = 32 * q + lane;
+            at[q] = 0;
+            d[q] = 0.0f;
+            if (e < ne) {
+                lo[q] = f->box[2 * e];
+                hi[q] = f->box[2 * e + 1];
+                const float dx = fmaxf(fmaxf(lo[q].x - ox, ox - hi[q].x), 0.0f),
+                            dy = fmaxf(fmaxf(lo[q].y - oy, oy - hi[q].y), 0.0f),
+                            dz = fmaxf(fmaxf(lo[q].z - oz, oz - hi[q].z), 0.0f);
+                d[q] = dx * dx + dy * dy + dz * dz;
+                key[e] = d[q];
             }
         }
-        for (int gi = 0; gi < front->ngroups; ++gi) {
-            if (kStats) ++out.nodes;
-            float d[4];
-            int c[4];
-            slab4<true>(front->grp + 7 * gi, sr, d, c);
+        __syncwarp();
+        for (int e = 0; e < ne; ++e) {
+            const float k = key[e];
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-                if (d[k] != INFINITY) stack[sp++] = c[k];
+            for (int q = 0; q < kFrontWords; ++q) at[q] += k > d[q] || (k == d[q] && e < 32 * q + lane);
         }
-        if (sp == 0) {
-            out.flags = (ambhit ? 1 : 0) | (amb ? 2 : 0);
-            return out;
-        }
-        cur = stack[--sp];
+#pragma unroll
+        for (int q = 0; q < kFrontWords; ++q)
+            if (32 * q + lane < ne) {
+                f->box[2 * at[q]] = lo[q];
+                f->box[2 * at[q] + 1] = hi[q];
+            }
+        __syncwarp();
     }
+    if (lane == 0) {
+        f->nboxes = ne;
+        f->ntris = nt;
+        f->nvis = visited + grown;
+    }
+    __syncwarp();
+}
+
+// Any-hit walk of the subtree at wide node `start` (0: the whole tree) by one
+// lane, with its stack in local memory.
+template <bool kStats>
+__device__ __forceinline__ TraceOut trace4(const float4* __restrict__ wnodes, const float4* __restrict__ tris,
+                                           const Ray& r, int max_steps, int start = 0)
+{
+    TraceOut out = {0, 0, 0, 0, 0};
+    int stack[kStack4];
+    int sp = 0;
+    int cur = start;
+    bool amb = false, ambhit = false;
+    const SlabRay sr = make_slab_ray(r, r.rs);
     for (int steps = 0;; ++steps) {
         if (steps > max_steps) { out.overflow = 1; out.flags = 1; return out; }
         if (cur >= 0) {
             if (kStats) ++out.nodes;
             float d[4];
             int c[4];
-            const int nh = slab4(wnodes + 8 * cur, sr, d, c);
+            const int nh = slab4(wnodes, cur, sr, d, c);
             if (nh == 0) {
                 if (sp == 0) break;
                 cur = stack[--sp];
@@ -590,15 +721,14 @@ __device__ __forceinline__ TraceOut trace4(const float4* __restrict__ wnodes, co
             // than the full network, and no more nodes visited)
             RC_CSWAP(0, 1) RC_CSWAP(2, 3) RC_CSWAP(0, 2)
 #undef RC_CSWAP
-            if (sp + nh - 1 > kStackF) { out.overflow = 1; out.flags = 1; return out; }
+            if (sp + nh - 1 > kStack4) { out.overflow = 1; out.flags = 1; return out; }
             if (d[3] != INFINITY) stack[sp++] = c[3];
             if (d[2] != INFINITY) stack[sp++] = c[2];
             if (d[1] != INFINITY) stack[sp++] = c[1];
             cur = c[0];
             continue;
         } else {
-            const int v = -1 - cur;
-            const int first = v >> 3, cnt = (v & 7) + 1;
+            const int first = leaf_first(cur), cnt = leaf_count(cur);
             for (int k = 0; k < cnt; ++k) {
                 const float4* t = tris + 3 * (first + k);
                 const float4 v0 = __ldg(t), v1 = __ldg(t + 1), v2 = __ldg(t + 2);
@@ -622,9 +752,9 @@ __device__ __forceinline__ TraceOut trace4(const float4* __restrict__ wnodes, co
 
 template <bool kStats, bool kWide>
 __device__ __forceinline__ TraceOut trace_any(const float4* __restrict__ nodes, const float4* __restrict__ tris,
-                                              const Ray& r, int max_steps, const Frontier* front = nullptr)
+                                              const Ray& r, int max_steps)
 {
-    if (kWide) return trace4<kStats>(nodes, tris, r, max_steps, front);
+    if (kWide) return trace4<kStats>(nodes, tris, r, max_steps);
     return trace<kStats>(nodes, tris, r, max_steps);
 }
 
@@ -696,9 +826,11 @@ __device__ __forceinline__ TraceOut trace_axis(const float4* __restrict__ ftree,
         if (steps > max_steps) { out.overflow = 1; out.flags = 1; return out; }
         if (cur >= 0) {
             if (kStats) ++out.nodes;
-            const float4* nd = ftree + 8 * (int64_t)cur;
-            const float4 lxv = __ldg(nd), hxv = __ldg(nd + 1), lyv = __ldg(nd + 2), hyv = __ldg(nd + 3);
-            const float4 lzv = __ldg(nd + 4), hzv = __ldg(nd + 5), ci = __ldg(nd + 6), ev = __ldg(nd + near_off);
+            const float4* nd = wide_ptr(ftree, cur);
+            const float4 lxv = wide_ld(nd, 0), hxv = wide_ld(nd, 1);
+            const float4 lyv = wide_ld(nd, 2), hyv = wide_ld(nd, 3);
+            const float4 lzv = wide_ld(nd, 4), hzv = wide_ld(nd, 5);
+            const float4 ci = wide_ld(nd, 6), ev = wide_ld(nd, near_off);
             const float LX[4] = {lxv.x, lxv.y, lxv.z, lxv.w}, HX[4] = {hxv.x, hxv.y, hxv.z, hxv.w};
             const float LY[4] = {lyv.x, lyv.y, lyv.z, lyv.w}, HY[4] = {hyv.x, hyv.y, hyv.z, hyv.w};
             const float LZ[4] = {lzv.x, lzv.y, lzv.z, lzv.w}, HZ[4] = {hzv.x, hzv.y, hzv.z, hzv.w};
@@ -734,8 +866,7 @@ __device__ __forceinline__ TraceOut trace_axis(const float4* __restrict__ ftree,
             cur = c[0];
             continue;
         } else {
-            const int v = -1 - cur;
-            const int first = v >> 3, cnt = (v & 7) + 1;
+            const int first = leaf_first(cur), cnt = leaf_count(cur);
             for (int k = 0; k < cnt; ++k) {
                 const float4* t = tris + 3 * (first + k);
                 const float4 v0 = __ldg(t), v1 = __ldg(t + 1), v2 = __ldg(t + 2);
@@ -784,13 +915,23 @@ __device__ __forceinline__ void warp_add_counters(unsigned long long* counters, 
 // Section 3.1: hemispherical cast.  One warp per point (dynamic work
 // counter).  The warp casts the point's N directions in N/32 tiles of 32
 // spatially close directions (the table is stored in tile order, each entry
-// carrying its canonical index j), so that the lanes of a warp walk nearly
-// the same part of the tree.  Each visible direction sets bit j & 31 of word
-// j >> 5 in the warp's shared-memory row, which is written out in canonical
-// order once the point is done; the count is the sum of the tile ballots.
+// carrying its canonical index j), so that the rays of a warp walk nearly
+// the same part of the tree.  Direction j is bit j & 31 of word j >> 5 of the
+// warp's shared-memory row, which is written out in canonical order once the
+// point is done.
 // ---------------------------------------------------------------------------
+// 5 blocks of 4 warps: 96 registers without spills, and the 32 KB a block
+// keeps in shared memory leave L1 about 90 KB.  4 and 6 blocks measured 32.5
+// and 34.4 ms against 31.1 on the impeller (100k points x 2048), 5.99 and
+// 6.08 against 5.85 on the housing (100k x 1024).
 #ifndef RC_HEMI_MIN_BLOCKS
-#define RC_HEMI_MIN_BLOCKS 7
+#define RC_HEMI_MIN_BLOCKS 5
+#endif
+#ifndef RC_UPDATE_MIN_BLOCKS
+#define RC_UPDATE_MIN_BLOCKS 7
+#endif
+#ifndef RC_AXIS_MIN_BLOCKS
+#define RC_AXIS_MIN_BLOCKS 6
 #endif
 #ifndef RC_TAIL_SPLITS
 #define RC_TAIL_SPLITS 4
@@ -801,20 +942,511 @@ __device__ __forceinline__ void warp_add_counters(unsigned long long* counters, 
 
 using CastAcc = CastAccFwd;
 
-// The hemispherical cast of one point by one warp (see above).  `tdirs` is
-// the tile-ordered table, `row` the warp's shared-memory row of W words.
-// Tiles [t0, t1) are cast; a whole point (0, W) writes its bit row and count,
-// a part of a point ORs its bits into the (zeroed) row in memory and adds
-// its count.
-template <bool kStats, bool kWide>
-__device__ __forceinline__ void cast_point(const float4* __restrict__ nodes, const float4* __restrict__ tris,
-                                           int max_steps, float scene_maxabs, const float* __restrict__ P,
-                                           const float* __restrict__ Nrm, int64_t i,
-                                           const float4* __restrict__ tdirs, int W, double eps, uint32_t* row,
-                                           uint32_t* __restrict__ bits, int32_t* __restrict__ count, CastAcc& acc,
-                                           int t0 = 0, int t1 = -1, long long* relist = nullptr,
-                                           long long relist_cap = 0, unsigned long long* relist_ctr = nullptr,
-                                           Frontier* front = nullptr)
+// ---------------------------------------------------------------------------
+// Pooled walk of one point's rays by one warp (4-wide tree).  A tile of 32
+// walks, one per lane, keeps a warp at about 11 active lanes: walk lengths
+// are heavy-tailed, and lanes at a node wait for lanes at a leaf.  Here the
+// unit of work is a pair (ray, node) or (ray, leaf).  The warp keeps a stack
+// of such pairs in shared memory and takes up to 32 from its top at a time, a
+// pair per lane, whichever rays they belong to, so every box test and every
+// triangle test runs on (nearly) full warps.
+//   - Rays enter in tiles: a ray's direction and reciprocals live in a slot
+//     in shared memory; slots 32..63 hold the tile that entered last and
+//     slots 0..31 the rays of the pairs left over from earlier tiles (moved
+//     there when the next tile enters).
+//   - A tile first finds the frontier boxes it can meet at all (interval
+//     slab test on its directions, a lane per box: 5 of 25 on the impeller).
+//     Those are tested for its rays, nearest first, while fewer than 32 pairs
+//     wait, and the next tile enters when they are used up.  So the warp does
+//     not run dry before the point's last tile, and a tile whose rays are all
+//     blocked leaves its remaining boxes untested.  Testing boxes ahead (48
+//     or 64 pairs) fills the lanes better and still measured 11% and 22%
+//     slower: more pairs of rays that a nearer box would have blocked.
+//   - Pairs of a blocked ray are dropped when they are taken.  A leaf's pair
+//     waits in a queue of its own for a full step of triangle tests.
+//   - The nearest entered child of every lane's node is pushed last, so the
+//     walk stays depth-first and near-first per ray.
+// Every ray meets the same boxes and triangles as in a walk of its own, less
+// those that a hit found earlier makes unnecessary, so the bits are the same.
+// What bounds it: instruction issue (58% of cycles at 28 active lanes and 125
+// warp instructions per ray on the impeller, where a ray per lane took 73% at
+// 11 lanes and 191), then the L1 data path (48%).  A step at a node is about
+// 280 warp instructions, 60% of the time.
+// ---------------------------------------------------------------------------
+constexpr int kPoolPairs = 320;        // pairs (ray, node or leaf) on the stack
+constexpr int kPoolLeaves = 96;        // pairs (ray, leaf) that wait for a full step
+constexpr int kPoolFill = 28;          // lanes that are enough for a step
+// Room on the stack: a step takes n pairs and adds up to 4 n.  While more than
+// kPoolFull wait, steps take fewer, down to one pair at a time, whose subtree
+// needs at most 3 entries per level of a tree of depth (kStack4 - 1) / 3.
+constexpr int kPoolFull = kPoolPairs - kStack4 - 96;
+static_assert(kPoolFull >= 64, "a box's rays on top of what waits");
+
+// A pair: a code (node >= 0, leaf < 0) and the slot of its ray.  32 bits hold
+// codes of 26 bits, that is 2^25 nodes and 2^24 triangles; parts beyond that
+// use 64 (0.3 ms of 31 slower on the impeller, and half the stack more of L1).
+template <bool kBig>
+struct PairOf {
+    int v;
+    static __device__ __forceinline__ PairOf make(int code, int slot) { return {(code << 6) | slot}; }
+    __device__ __forceinline__ int code() const { return v >> 6; }
+    __device__ __forceinline__ int slot() const { return v & 63; }
+};
+template <>
+struct PairOf<true> {
+    int c, s;
+    static __device__ __forceinline__ PairOf make(int code, int slot) { return {code, slot}; }
+    __device__ __forceinline__ int code() const { return c; }
+    __device__ __forceinline__ int slot() const { return s; }
+};
+constexpr int64_t kPairTris = 1 << 24;     // most triangles of 32-bit pairs (leaves of 2, nodes fewer)
+static_assert(kLeafBits == 1, "a leaf code of 2^24 triangles has 26 bits with its sign");
+
+template <bool kBig>
+struct __align__(16) PoolOf {
+    Frontier front;
+    float4 onb[3];                 // basis t1, t2 and the normal: components x, y, z
+    float4 inv[64];                // reciprocals of the ray's direction, canonical index
+    float4 dir[64];                // direction, its largest |component|
+    PairOf<kBig> pair[kPoolPairs];
+    PairOf<kBig> leaf[kPoolLeaves];
+    uint8_t met[kFrontEntries];    // the frontier boxes that the current tile can meet
+};
+static_assert(kPoolPairs >= kFrontQueue, "the stack also serves as the frontier's queue");
+
+// bit rows of a warp: visible so far, met an ambiguous pair, met an ambiguous
+// pair that FP64 calls a hit, and (instrumented cast) re-tested in FP64
+__host__ __device__ __forceinline__ constexpr int pool_rows(bool stats) { return stats ? 4 : 3; }
+
+// FP32 decision of one pair by signed volumes (Moeller and Trumbore 1997),
+// with a forward error bound; kHit and kMiss only when certain, as
+// tri_test32.  With s = A - o, e1 = B - A, e2 = C - A, p = d x e2 and
+// q = s x e1 the hit point is A + (U/D) e1 + (V/D) e2 at t = T/D, where
+// U = s.p, V = d.q, D = -(e1.p), T = e2.q; the third edge is W = D - U - V.
+// Unlike the sheared form it needs no permutation of the coordinates by the
+// ray's largest component, and the bound needs only the largest |s_k| (S),
+// the triangle's largest edge component (e, stored in its record) and the
+// ray's largest |d_k| (m):
+//   inputs     s and e round once (u relative; e is a computed value)
+//   |p| <= 2me, error 5 u m e        |q| <= 2Se, error 7 u S e
+//   U: 15 (p) + 6 (s) + 12 (sum) = 33 u S m e;   V: 21 + 12 = 33 u S m e
+//   D: 15 + 6 + 12 = 33 u m e^2;     T: 21 + 6 + 12 = 39 u S e^2
+//   W: U + V + D and two roundings = u m e (84 S + 45 e)
+// each scaled by 1.0625 for second-order terms and the bound's own rounding;
+// 1e-36 covers products that leave the normal range.
+__device__ __forceinline__ int tri_test_mt(float ox, float oy, float oz, float dx, float dy, float dz, float m,
+                                           float rs, const float4 v0, const float4 v1, const float4 v2)
+{
+    const float u = 5.9604644775390625e-8f;
+    const float s0 = v0.x - ox, s1 = v0.y - oy, s2 = v0.z - oz;
+    const float a0 = v1.x - v0.x, a1 = v1.y - v0.y, a2 = v1.z - v0.z;
+    const float b0 = v2.x - v0.x, b1 = v2.y - v0.y, b2 = v2.z - v0.z;
+    const float p0 = fmaf(dy, b2, -(dz * b1)), p1 = fmaf(dz, b0, -(dx * b2)), p2 = fmaf(dx, b1, -(dy * b0));
+    const float q0 = fmaf(s1, a2, -(s2 * a1)), q1 = fmaf(s2, a0, -(s0 * a2)), q2 = fmaf(s0, a1, -(s1 * a0));
+    const float U = fmaf(s0, p0, fmaf(s1, p1, s2 * p2));
+    const float V = fmaf(dx, q0, fmaf(dy, q1, dz * q2));
+    const float D = -fmaf(a0, p0, fmaf(a1, p1, a2 * p2));
+    const float W = (D - U) - V;
+    const float S = fmaxf(fabsf(s0), fmaxf(fabsf(s1), fabsf(s2)));
+    const float e = v0.w;
+    const float ume = u * m * e;
+    const float eU = fmaf(35.1f * ume, S, 1e-36f);
+    const float eW = fmaf(89.3f * ume, S, fmaf(47.9f * ume, e, 1e-36f));
+    const bool pos = fmaxf(U, V) > eU || W > eW, neg = fminf(U, V) < -eU || W < -eW;
+    if (pos && neg) return kMiss;
+
+    const float T = fmaf(b0, q0, fmaf(b1, q1, b2 * q2));
+    const float eD = fmaf(35.1f * ume, e, 1e-36f);
+    const float eT = fmaf(41.5f * u * S, e * e, 1e-36f);
+    const bool tp_ok = fabsf(T) > eT;
+    if (fabsf(D) > eD && tp_ok && (T > 0.0f) != (D > 0.0f)) return kMiss;   // plane crossed behind the origin
+    // clear hit: every edge beyond its error and the tau band (|edge x d| <=
+    // 3 m e), hence all of one sign, which is D's; the crossing ahead and
+    // beyond tau R along the ray
+    const float tau_edge = 3.0f * 1e-9f * 1.01f * rs * m * e;
+    if (fminf(fabsf(U), fabsf(V)) > eU + tau_edge && fabsf(W) > eW + tau_edge && tp_ok &&
+        (T > 0.0f) == (U > 0.0f) && (fabsf(T) - eT) * m > 1.01e-9f * rs * (fabsf(D) + eD))
+        return kHit;
+    return kUnsure;
+}
+
+// One axis of the slab test on a tile's directions: their components span
+// [dl, dh], and a box spans [l, h] relative to the shared origin.  Some ray of
+// the tile can be inside the slab at t >= 0 only for t in [tn, tf]:
+// l <= t d with d <= dh gives t >= l / dh, and so on; a component that spans
+// zero (or nearly) bounds t from below only.  Roundings are covered by the
+// box's margin (ex, ey, ez) and the 1e-5 by which the caller widens tf.
+struct TileAxis {
+    float a, b, c, d, far;
+    __device__ __forceinline__ void clip(float l, float h, float& tn, float& tf) const
+    {
+        tn = fmaxf(tn, fmaxf(l * a, h * b));
+        tf = fminf(tf, fmaf(h, c, fmaf(l, d, far)));
+    }
+};
+
+__device__ __forceinline__ float rcp_approx(float x)   // within 2^-23 relative
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// a lane's share of a ray's reciprocals: one unit in the last place off at
+// most, zero components as in setup_ray
+__device__ __forceinline__ float ray_rcp(float d)
+{
+    const float i = rcp_approx(d);
+    return fabsf(i) <= 0x1p100f ? i : copysignf(0x1p100f, d);
+}
+
+__device__ __forceinline__ TileAxis tile_axis(float x)
+{
+    const float lo = warp_min(x), hi = warp_max(x);
+    constexpr float kSmall = 1e-4f;
+    TileAxis t;
+    const float rl = rcp_approx(lo), rh = rcp_approx(hi);
+    t.a = hi >= kSmall ? rh : (hi > 0.0f ? 1.0f / kSmall : 0.0f);
+    t.b = lo <= -kSmall ? rl : (lo < 0.0f ? -1.0f / kSmall : 0.0f);
+    t.c = lo >= kSmall ? rl : 0.0f;
+    t.d = hi <= -kSmall ? rh : 0.0f;
+    t.far = lo >= kSmall || hi <= -kSmall ? 0.0f : INFINITY;
+    return t;
+}
+
+// FP64 decision of the lanes' pairs (ray j in direction d, triangle record
+// tp) that FP32 left open; true for a clear hit.  Not inlined: it is rare.
+template <bool kStats>
+__device__ __noinline__ bool pool_retest(float ox, float oy, float oz, const float4 d, int j, const float4* tp,
+                                         uint32_t* rows, int W, int64_t i, long long* relist, long long relist_cap,
+                                         unsigned long long* relist_ctr)
+{
+    const Pair64 q = retest64(ox, oy, oz, d.x, d.y, d.z, tp[0], tp[1], tp[2]);
+    const uint32_t b = 1u << (j & 31);
+    if (kStats && relist && !(atomicOr(&rows[3 * W + (j >> 5)], b) & b)) {
+        const unsigned long long at = atomicAdd(relist_ctr, 1ULL);
+        if (at < (unsigned long long)relist_cap) relist[at] = (long long)i * 65536 + j;
+    }
+    if (q.state == kUnsure) {
+        atomicOr(&rows[W + (j >> 5)], b);
+        if (q.hit64) atomicOr(&rows[2 * W + (j >> 5)], b);
+    }
+    return q.state == kHit;
+}
+
+// cast_point on the 4-wide tree (same arguments; pool and rows: the warp's
+// shared memory)
+template <bool kStats, bool kBig>
+__device__ __forceinline__ void cast_point_pooled(const float4* __restrict__ wnodes, const float4* __restrict__ tris,
+                                                  int max_steps, float scene_maxabs, const float* __restrict__ P,
+                                                  const float* __restrict__ Nrm, int64_t i,
+                                                  const float4* __restrict__ tdirs, int W, double eps,
+                                                  PoolOf<kBig>* pool, uint32_t* rows, uint32_t* __restrict__ bits,
+                                                  int32_t* __restrict__ count, CastAcc& acc, int t0, int t1,
+                                                  long long* relist, long long relist_cap,
+                                                  unsigned long long* relist_ctr)
+{
+    using Pair = PairOf<kBig>;
+    constexpr unsigned kAll = 0xFFFFFFFFu;
+    const int lane = threadIdx.x & 31;
+    const unsigned below = (1u << lane) - 1u;
+    const bool whole = t1 < 0;
+    if (whole) t1 = W;
+    uint32_t* vis = rows;
+    for (int w = lane; w < pool_rows(kStats) * W; w += 32) rows[w] = 0u;
+    Frontier* f = &pool->front;
+    float ox, oy, oz;
+    {
+        const float nx = Nrm[3 * i], ny = Nrm[3 * i + 1], nz = Nrm[3 * i + 2];
+        ox = offset_coord(P[3 * i], nx, eps);
+        oy = offset_coord(P[3 * i + 1], ny, eps);
+        oz = offset_coord(P[3 * i + 2], nz, eps);
+        build_frontier(wnodes, tris, ox, oy, oz, nx, ny, nz, tangent_shortcuts_ok(nx, ny, nz, W),
+                       20.0f / (32.0f * W), min(kFrontRounds, W / 4), f, (int*)pool->pair);
+        if (lane == 0) {
+            const Onb b = make_onb(nx, ny, nz);
+            pool->onb[0] = make_float4(b.t1x, b.t2x, nx, 0.0f);
+            pool->onb[1] = make_float4(b.t1y, b.t2y, ny, 0.0f);
+            pool->onb[2] = make_float4(b.t1z, b.t2z, nz, 0.0f);
+        }
+        __syncwarp();
+    }
+    if (kStats && lane == 0) acc.nvis += f->nvis;
+    // M >= every coordinate, and the margin of a slab distance per unit of
+    // |reciprocal| (see SlabRay), here 6 u (M + |o|) <= 12 u M: a reciprocal
+    // off by 2 u, the products and sums of the constants 2 u, the final FMA u
+    const float rs = fmaxf(fmaxf(1.0f, scene_maxabs), fmaxf(fabsf(ox), fmaxf(fabsf(oy), fabsf(oz))));
+    const float em = 12.0f * 5.9604644775390625e-8f * rs;
+    int sp = 0, lsp = 0;                   // pairs on the stack, leaves that wait
+    unsigned live0 = 0, live1 = 0;         // slots 0..31 and 32..63 whose rays are not known to be blocked
+    int t = t0;                            // next tile
+    int boxes = 0;                         // of pool->met still to be tested
+    // on a well-formed tree a ray meets each node at most once; the cap only
+    // bounds a malformed one
+    int steps = (int)min64(0x7FFFFFFF, 2 * (int64_t)(t1 - t0 + 1) * max_steps);
+    for (;;) {
+        if (lsp < 32 && sp < 32 && boxes > 0) {
+            // the tile's rays against its frontier boxes, nearest first (the
+            // deepest), until a step's worth of pairs waits
+            if (live1 == 0) {
+                boxes = 0;
+                continue;
+            }
+            const bool on = (live1 >> lane) & 1u;
+            const float4 v = pool->inv[32 + lane];
+            const float x = ox * v.x, y = oy * v.y, z = oz * v.z;
+            const float mx = em * fabsf(v.x), my = em * fabsf(v.y), mz = em * fabsf(v.z);
+            const bool bx = signbit(v.x), by = signbit(v.y), bz = signbit(v.z);
+            do {
+                const int e = pool->met[--boxes];
+                const float4 lo = f->box[2 * e], hi = f->box[2 * e + 1];
+                const float tn = fmaxf(fmaxf(fmaf(bx ? hi.x : lo.x, v.x, -(x + mx)), fmaf(by ? hi.y : lo.y, v.y, -(y + my))),
+                                       fmaxf(fmaf(bz ? hi.z : lo.z, v.z, -(z + mz)), 0.0f));
+                const float tf = fminf(fminf(fmaf(bx ? lo.x : hi.x, v.x, mx - x), fmaf(by ? lo.y : hi.y, v.y, my - y)),
+                                       fmaf(bz ? lo.z : hi.z, v.z, mz - z));
+                const bool in = on && tn <= tf;
+                if (kStats) acc.nbox += on;
+                const unsigned m = __ballot_sync(kAll, in);
+                if (in) pool->pair[sp + __popc(m & below)] = Pair::make(__float_as_int(lo.w), 32 + lane);
+                sp += __popc(m);
+            } while (boxes > 0 && sp < 32);
+            __syncwarp();
+            continue;
+        }
+        if (lsp < 32 && (sp >= 32 || (sp > 0 && t >= t1))) {
+            // up to 32 live pairs with a node from the top of the stack, one
+            // per lane; pairs with a leaf move to the leaf queue, pairs of
+            // blocked rays are dropped, and lanes left without look again
+            if (--steps < 0) break;
+            bool have = false, idle = false;
+            if (sp > kPoolFull) idle = lane >= max(1, min(32, (kPoolPairs - kStack4 - sp) / 3));
+            int code = 0, slot = 0;
+            for (;;) {
+                const unsigned want = __ballot_sync(kAll, !(have || idle));
+                const int at = sp - 1 - __popc(want & below);
+                bool leaf = false;
+                if (!(have || idle) && at >= 0) {
+                    const Pair q = pool->pair[at];
+                    slot = q.slot();
+                    code = q.code();
+                    const bool live = ((slot & 32 ? live1 : live0) >> (slot & 31)) & 1u;
+                    have = live && code >= 0;
+                    leaf = live && code < 0;
+                }
+                const unsigned ml = __ballot_sync(kAll, leaf);
+                if (leaf) pool->leaf[lsp + __popc(ml & below)] = Pair::make(code, slot);
+                lsp += __popc(ml);
+                sp = max(0, sp - __popc(want));
+                if (sp == 0 || lsp > kPoolLeaves - 32 || __popc(__ballot_sync(kAll, have || idle)) >= kPoolFill) break;
+            }
+            float d[4] = {INFINITY, INFINITY, INFINITY, INFINITY};
+            int c[4] = {0, 0, 0, 0};
+            if (have) {
+                if (kStats) acc.nvis += 1;
+                const float4 v = pool->inv[slot];
+                const float x = ox * v.x, y = oy * v.y, z = oz * v.z;
+                const float mx = em * fabsf(v.x), my = em * fabsf(v.y), mz = em * fabsf(v.z);
+                // near and far planes by the sign of the direction (wide_at:
+                // float4 c lies at c ^ (node & 7))
+                const unsigned at = ((unsigned)code & 7u) << 4;
+                const unsigned qx = at ^ ((__float_as_uint(v.x) >> 27) & 16u),
+                               qy = at ^ ((__float_as_uint(v.y) >> 27) & 16u) ^ 32u,
+                               qz = at ^ ((__float_as_uint(v.z) >> 27) & 16u) ^ 64u;
+                const auto ld = [&](unsigned q) {
+                    if (kBig) return __ldg((const float4*)((const char*)wnodes + ((size_t)code << 7) + q));
+                    return __ldg((const float4*)((const char*)wnodes + (((unsigned)code << 7) | q)));
+                };
+                const float4 nx = ld(qx), fx = ld(qx ^ 16u), ny = ld(qy), fy = ld(qy ^ 16u), nz = ld(qz), fz = ld(qz ^ 16u);
+                const float4 ci = ld(at ^ 96u);
+                const auto entry = [&](float nxk, float nyk, float nzk, float fxk, float fyk, float fzk) {
+                    const float tn = fmaxf(fmaxf(fmaf(nxk, v.x, -(x + mx)), fmaf(nyk, v.y, -(y + my))),
+                                           fmaxf(fmaf(nzk, v.z, -(z + mz)), 0.0f));
+                    const float tf = fminf(fminf(fmaf(fxk, v.x, mx - x), fmaf(fyk, v.y, my - y)),
+                                           fmaf(fzk, v.z, mz - z));
+                    return tn <= tf ? tn : INFINITY;
+                };
+                d[0] = entry(nx.x, ny.x, nz.x, fx.x, fy.x, fz.x);
+                d[1] = entry(nx.y, ny.y, nz.y, fx.y, fy.y, fz.y);
+                d[2] = entry(nx.z, ny.z, nz.z, fx.z, fy.z, fz.z);
+                d[3] = entry(nx.w, ny.w, nz.w, fx.w, fy.w, fz.w);
+                c[0] = __float_as_int(ci.x);
+                c[1] = __float_as_int(ci.y);
+                c[2] = __float_as_int(ci.z);
+                c[3] = __float_as_int(ci.w);
+#define RC_CSWAP(a, b)                                              \
+    if (d[b] < d[a]) {                                              \
+        const float td = d[a]; d[a] = d[b]; d[b] = td;              \
+        const int tc = c[a]; c[a] = c[b]; c[b] = tc;                \
+    }
+                RC_CSWAP(0, 1) RC_CSWAP(2, 3) RC_CSWAP(0, 2)
+#undef RC_CSWAP
+            }
+            __syncwarp();
+            // push the entered children: the farther ones first (a lane's side
+            // by side, its count 0..3 summed over the lower lanes bit by bit),
+            // then the nearest of every lane
+            const bool i0 = d[0] != INFINITY, i1 = d[1] != INFINITY, i2 = d[2] != INFINITY, i3 = d[3] != INFINITY;
+            const unsigned b0 = __ballot_sync(kAll, i1 ^ i2 ^ i3), b1 = __ballot_sync(kAll, (i1 & i2) | (i3 & (i1 | i2))),
+                           bn = __ballot_sync(kAll, i0);
+            int at = sp + __popc(b0 & below) + 2 * __popc(b1 & below);
+            if (i3) pool->pair[at++] = Pair::make(c[3], slot);
+            if (i2) pool->pair[at++] = Pair::make(c[2], slot);
+            if (i1) pool->pair[at] = Pair::make(c[1], slot);
+            sp += __popc(b0) + 2 * __popc(b1);
+            if (i0) pool->pair[sp + __popc(bn & below)] = Pair::make(c[0], slot);
+            sp += __popc(bn);
+            __syncwarp();
+            continue;
+        }
+        if (lsp > 0) {
+            // up to 32 pairs with a leaf, one per lane
+            const int at = lsp - 1 - lane;
+            lsp = max(0, lsp - 32);
+            int ntri = 0, slot = 0;
+            float4 rd = make_float4(0, 0, 0, 0);
+            const float4* tp = tris;
+            if (at >= 0) {
+                const Pair q = pool->leaf[at];
+                slot = q.slot();
+                rd = pool->dir[slot];
+                tp = tris + 3 * (int64_t)leaf_first(q.code());
+                if (((slot & 32 ? live1 : live0) >> (slot & 31)) & 1u) ntri = leaf_count(q.code());
+            }
+            bool hit = false;
+            for (int k = 0; k < kLeafMax && __any_sync(kAll, k < ntri); ++k) {
+                int st = kMiss;
+                if (k < ntri) {
+                    if (kStats) acc.ntri += 1;
+                    st = tri_test_mt(ox, oy, oz, rd.x, rd.y, rd.z, rd.w, rs, __ldg(tp + 3 * k), __ldg(tp + 3 * k + 1),
+                                     __ldg(tp + 3 * k + 2));
+                    if (st == kUnsure) {
+                        acc.retests += 1;
+                        if (pool_retest<kStats>(ox, oy, oz, rd, __float_as_int(pool->inv[slot].w), tp + 3 * k, rows, W,
+                                                i, relist, relist_cap, relist_ctr))
+                            st = kHit;
+                    }
+                    if (st == kHit) {
+                        hit = true;
+                        ntri = 0;
+                    }
+                }
+            }
+            if (hit) {
+                const int j = __float_as_int(pool->inv[slot].w);
+                atomicAnd(&vis[j >> 5], ~(1u << (j & 31)));
+            }
+            const unsigned bit = hit ? 1u << (slot & 31) : 0u;
+            live0 &= ~__reduce_or_sync(kAll, slot & 32 ? 0u : bit);
+            live1 &= ~__reduce_or_sync(kAll, slot & 32 ? bit : 0u);
+            __syncwarp();
+            continue;
+        }
+        if (t >= t1) break;
+        // the next tile enters; the rays of the pairs left over move down
+        // (one slot per ray, the lowest pair's)
+        if (sp > 0) {
+            const bool mine = lane < sp;
+            Pair q = Pair::make(0, 0);
+            if (mine) q = pool->pair[lane];
+            const int from = q.slot();
+            const float4 li = pool->inv[from], ld = pool->dir[from];
+            const bool live = mine && (((from & 32 ? live1 : live0) >> (from & 31)) & 1u);
+            const int to = __ffs(__match_any_sync(kAll, live ? __float_as_int(li.w) : -1 - lane)) - 1;
+            live0 = __ballot_sync(kAll, live && to == lane);
+            if (live && to == lane) {
+                pool->inv[lane] = li;
+                pool->dir[lane] = ld;
+            }
+            if (mine) pool->pair[lane] = Pair::make(q.code(), to);    // a pair of a blocked ray: its own slot, not live
+            __syncwarp();
+        }
+        const float4 h = __ldg(&tdirs[32 * t + lane]);
+        const float4 cx = pool->onb[0], cy = pool->onb[1], cz = pool->onb[2];
+        const int jt = __float_as_int(h.w);    // -1: padding of the last tile
+        const Onb b = {cx.x, cy.x, cz.x, cx.y, cy.y, cz.y};
+        float4 rd;
+        local_to_world(b, cx.z, cy.z, cz.z, h.x, h.y, h.z, rd.x, rd.y, rd.z);
+        rd.w = fmaxf(fabsf(rd.x), fmaxf(fabsf(rd.y), fabsf(rd.z)));
+        pool->inv[32 + lane] = make_float4(ray_rcp(rd.x), ray_rcp(rd.y), ray_rcp(rd.z), h.w);
+        pool->dir[32 + lane] = rd;
+        ++t;
+        // the point's local triangles
+        bool open = jt >= 0;
+        for (int k = 0; k < f->ntris; ++k) {
+            if (!open) continue;
+            if (kStats) acc.ntri += 1;
+            int st = tri_test_mt(ox, oy, oz, rd.x, rd.y, rd.z, rd.w, rs, f->tri[3 * k], f->tri[3 * k + 1],
+                                 f->tri[3 * k + 2]);
+            if (st == kUnsure) {
+                acc.retests += 1;
+                if (pool_retest<kStats>(ox, oy, oz, rd, jt, &f->tri[3 * k], rows, W, i, relist, relist_cap, relist_ctr))
+                    st = kHit;
+            }
+            open = st != kHit;
+        }
+        if (open) atomicOr(&vis[jt >> 5], 1u << (jt & 31));
+        live1 = __ballot_sync(kAll, open);
+        // the frontier boxes that the tile can meet: the slab test on the
+        // intervals that its directions span, a lane per box
+        const int src = __ffs(__ballot_sync(kAll, jt >= 0)) - 1;
+        const float sx = __shfl_sync(kAll, rd.x, src), sy = __shfl_sync(kAll, rd.y, src),
+                    sz = __shfl_sync(kAll, rd.z, src);
+        const TileAxis ax = tile_axis(jt >= 0 ? rd.x : sx), ay = tile_axis(jt >= 0 ? rd.y : sy),
+                       az = tile_axis(jt >= 0 ? rd.z : sz);
+        for (int q = 0; q < f->nboxes; q += 32) {
+            const int k = q + lane;
+            bool in = k < f->nboxes;
+            if (in) {
+                const float4 lo = f->box[2 * k], hi = f->box[2 * k + 1];
+                float tn = 0.0f, tf = INFINITY;
+                ax.clip(lo.x - ox - em, hi.x - ox + em, tn, tf);
+                ay.clip(lo.y - oy - em, hi.y - oy + em, tn, tf);
+                az.clip(lo.z - oz - em, hi.z - oz + em, tn, tf);
+                in = tn <= tf * 1.00001f;
+            }
+            const unsigned m = __ballot_sync(kAll, in);
+            if (in) pool->met[boxes + __popc(m & below)] = (uint8_t)k;
+            boxes += __popc(m);
+        }
+        __syncwarp();
+    }
+    if (steps < 0) acc.overflow += lane == 0;
+    // visible, less the rays that only an FP64-ambiguous pair blocks
+    int cnt = 0;
+    for (int w = lane; w < W; w += 32) {
+        const uint32_t v = vis[w];
+        acc.amb += __popc(v & rows[W + w]);
+        const uint32_t r = v & ~rows[2 * W + w];
+        cnt += __popc(r);
+        if (whole)
+            bits[i * W + w] = r;
+        else if (r)
+            atomicOr(&bits[i * W + w], r);
+    }
+    for (int off = 16; off; off >>= 1) cnt += __shfl_xor_sync(kAll, cnt, off);
+    if (lane == 0) {
+        if (whole)
+            count[i] = cnt;
+        else
+            atomicAdd(&count[i], cnt);
+    }
+    __syncwarp();
+    acc.rays += (t1 - t0) - (t1 == W && __float_as_int(__ldg(&tdirs[32 * (W - 1) + lane]).w) < 0 ? 1 : 0);
+}
+
+// The hemispherical cast of one point by one warp on the binary tree (see
+// above), a ray per lane.  `tdirs` is the tile-ordered table, `row` the
+// warp's shared-memory row of W words.  Tiles [t0, t1) are cast; a whole
+// point (0, W) writes its bit row and count, a part of a point ORs its bits
+// into the (zeroed) row in memory and adds its count.
+template <bool kStats>
+__device__ __forceinline__ void cast_point_binary(const float4* __restrict__ nodes, const float4* __restrict__ tris,
+                                                  int max_steps, float scene_maxabs, const float* __restrict__ P,
+                                                  const float* __restrict__ Nrm, int64_t i,
+                                                  const float4* __restrict__ tdirs, int W, double eps, uint32_t* row,
+                                                  uint32_t* __restrict__ bits, int32_t* __restrict__ count,
+                                                  CastAcc& acc, int t0, int t1, long long* relist,
+                                                  long long relist_cap, unsigned long long* relist_ctr)
 {
     const int lane = threadIdx.x & 31;
     const bool whole = t1 < 0;
@@ -823,11 +1455,7 @@ __device__ __forceinline__ void cast_point(const float4* __restrict__ nodes, con
     const float px = P[3 * i], py = P[3 * i + 1], pz = P[3 * i + 2];
     const float nx = Nrm[3 * i], ny = Nrm[3 * i + 1], nz = Nrm[3 * i + 2];
     const float ox = offset_coord(px, nx, eps), oy = offset_coord(py, ny, eps), oz = offset_coord(pz, nz, eps);
-    if (kWide && front && lane == 0)
-        build_frontier(nodes, tris, max_steps, ox, oy, oz, nx, ny, nz, tangent_shortcuts_ok(nx, ny, nz, W), front);
     __syncwarp();
-    const Frontier* fr = kWide && front && front->ok ? front : nullptr;
-    if (kStats && front && lane == 0) acc.nvis += front->nvis;
     const Onb b = make_onb(nx, ny, nz);
     int cnt = 0;
     for (int t = t0; t < t1; ++t) {
@@ -840,7 +1468,7 @@ __device__ __forceinline__ void cast_point(const float4* __restrict__ nodes, con
         local_to_world(b, nx, ny, nz, h.x, h.y, h.z, dx, dy, dz);
         Ray r;
         setup_ray(r, ox, oy, oz, dx, dy, dz, scene_maxabs);
-        const TraceOut tr = trace_any<kStats, kWide>(nodes, tris, r, max_steps, fr);
+        const TraceOut tr = trace<kStats>(nodes, tris, r, max_steps);
         acc.retests += tr.retests;
         acc.overflow += tr.overflow;
         acc.amb += (j >= 0) & ((tr.flags >> 1) & 1);
@@ -872,18 +1500,46 @@ __device__ __forceinline__ void cast_point(const float4* __restrict__ nodes, con
     acc.rays += (t1 - t0) - (t1 == W && __float_as_int(__ldg(&tdirs[32 * (W - 1) + lane]).w) < 0 ? 1 : 0);
 }
 
-// Dynamic shared memory of the point casts: each warp's bit row of W words,
-// then (4-wide tree) each warp's frontier, 16-byte aligned.
-__host__ __device__ __forceinline__ size_t rows_bytes(int warps, int W)
+// One point by one warp, by the tree's kind: a ray per lane on the binary
+// tree, pooled on the 4-wide one (with 64-bit pairs on the largest parts).
+enum { kBinary = 0, kWide4 = 1, kWide4Big = 2 };
+
+// Dynamic shared memory of the point casts: each warp's pool (4-wide tree),
+// then each warp's bit rows of W words.
+__host__ __device__ __forceinline__ constexpr int cast_rows(int kind, bool stats)
 {
-    return ((size_t)warps * W * sizeof(uint32_t) + 15) & ~(size_t)15;
+    return kind == kBinary ? 1 : pool_rows(stats);
 }
-__host__ __device__ __forceinline__ size_t cast_smem(int warps, int W, bool wide)
+__host__ __device__ __forceinline__ constexpr size_t pool_bytes(int kind)
 {
-    return rows_bytes(warps, W) + (wide ? (size_t)warps * sizeof(Frontier) : 0);
+    return kind == kBinary ? 0 : kind == kWide4 ? sizeof(PoolOf<false>) : sizeof(PoolOf<true>);
+}
+__host__ __device__ __forceinline__ size_t cast_smem(int warps, int W, int kind, bool stats)
+{
+    return warps * pool_bytes(kind) + (size_t)warps * W * cast_rows(kind, stats) * sizeof(uint32_t);
 }
 
-template <bool kStats, bool kWide>
+template <bool kStats, int kKind>
+__device__ __forceinline__ void cast_point(const float4* __restrict__ nodes, const float4* __restrict__ tris,
+                                           int max_steps, float scene_maxabs, const float* __restrict__ P,
+                                           const float* __restrict__ Nrm, int64_t i,
+                                           const float4* __restrict__ tdirs, int W, double eps, unsigned char* smem,
+                                           uint32_t* __restrict__ bits, int32_t* __restrict__ count, CastAcc& acc,
+                                           int t0 = 0, int t1 = -1, long long* relist = nullptr,
+                                           long long relist_cap = 0, unsigned long long* relist_ctr = nullptr)
+{
+    const int warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    uint32_t* rows = (uint32_t*)(smem + warps * pool_bytes(kKind)) + warp * W * cast_rows(kKind, kStats);
+    if (kKind == kBinary)
+        cast_point_binary<kStats>(nodes, tris, max_steps, scene_maxabs, P, Nrm, i, tdirs, W, eps, rows, bits, count,
+                                  acc, t0, t1, relist, relist_cap, relist_ctr);
+    else
+        cast_point_pooled<kStats, kKind == kWide4Big>(nodes, tris, max_steps, scene_maxabs, P, Nrm, i, tdirs, W, eps,
+                                                      (PoolOf<kKind == kWide4Big>*)smem + warp, rows, bits, count, acc,
+                                                      t0, t1, relist, relist_cap, relist_ctr);
+}
+
+template <bool kStats, int kKind>
 __global__ void __launch_bounds__(128, RC_HEMI_MIN_BLOCKS)
 k_hemisphere(const float4* __restrict__ nodes, const float4* __restrict__ tris, int max_steps, float scene_maxabs,
              const float* __restrict__ P, const float* __restrict__ Nrm, int64_t n,
@@ -894,8 +1550,6 @@ k_hemisphere(const float4* __restrict__ nodes, const float4* __restrict__ tris, 
     extern __shared__ __align__(16) unsigned char s_dyn[];
     const int lane = threadIdx.x & 31;
     const int W = (n_dirs + 31) >> 5;
-    uint32_t* row = (uint32_t*)s_dyn + (threadIdx.x >> 5) * W;
-    Frontier* front = kWide ? (Frontier*)(s_dyn + rows_bytes(blockDim.x >> 5, W)) + (threadIdx.x >> 5) : nullptr;
     CastAcc acc;
     // With a work counter the warps take work until none is left: the first
     // n_whole points of the processing order whole, then the last n - n_whole
@@ -926,10 +1580,10 @@ k_hemisphere(const float4* __restrict__ nodes, const float4* __restrict__ tris, 
             if (t0 >= t1) continue;
         }
         const int64_t i = order ? (int64_t)__ldg(&order[r]) : r;
-        cast_point<kStats, kWide>(nodes, tris, max_steps, scene_maxabs, P, Nrm, i, tdirs, W, eps, row, bits, count,
-                                  acc, t0, t1, relist, relist_cap, counters ? counters + 6 : nullptr, front);
+        cast_point<kStats, kKind>(nodes, tris, max_steps, scene_maxabs, P, Nrm, i, tdirs, W, eps, s_dyn, bits, count, acc,
+                                  t0, t1, relist, relist_cap, counters ? counters + 6 : nullptr);
     }
-    warp_add_counters(counters, acc.rays, acc.amb, acc.retests, acc.overflow, acc.nvis, acc.ntri);
+    warp_add_counters(counters, acc.rays, acc.amb, acc.retests, acc.overflow, acc.nvis + (acc.nbox + 3) / 4, acc.ntri);
 }
 
 // zero the bit rows and counts of the points cast in parts (positions
@@ -988,7 +1642,7 @@ __device__ __forceinline__ bool box_in_front(const float4 lo, const float4 hi, f
 }
 
 template <bool kWide>
-__global__ void __launch_bounds__(128, RC_HEMI_MIN_BLOCKS)
+__global__ void __launch_bounds__(128, RC_UPDATE_MIN_BLOCKS)
 k_hemisphere_update(const float4* __restrict__ nodes, const float4* __restrict__ tris, int max_steps,
                     float scene_maxabs, const float* __restrict__ P, const float* __restrict__ Nrm, int64_t n,
                     const int32_t* __restrict__ order, const int32_t* __restrict__ face,
@@ -1060,10 +1714,10 @@ __device__ __forceinline__ void flush_part_counters(unsigned long long* c, CastA
 }
 
 #ifndef RC_BATCH_MIN_BLOCKS
-#define RC_BATCH_MIN_BLOCKS 6
+#define RC_BATCH_MIN_BLOCKS 5
 #endif
 
-template <bool kStats, bool kWide>
+template <bool kStats, int kKind>
 __global__ void __launch_bounds__(128, RC_BATCH_MIN_BLOCKS)
 k_batch(const BatchPart* __restrict__ parts, int n_parts, long long n_items, int ppi,
         const float4* __restrict__ tdirs, int n_dirs, double eps, unsigned long long* work)
@@ -1071,8 +1725,6 @@ k_batch(const BatchPart* __restrict__ parts, int n_parts, long long n_items, int
     extern __shared__ __align__(16) unsigned char s_dyn[];
     const int lane = threadIdx.x & 31;
     const int W = (n_dirs + 31) >> 5;
-    uint32_t* row = (uint32_t*)s_dyn + (threadIdx.x >> 5) * W;
-    Frontier* front = kWide ? (Frontier*)(s_dyn + rows_bytes(blockDim.x >> 5, W)) + (threadIdx.x >> 5) : nullptr;
     CastAcc acc;
     int cur = -1;
     for (;;) {
@@ -1094,8 +1746,8 @@ k_batch(const BatchPart* __restrict__ parts, int n_parts, long long n_items, int
         const long long q1 = q0 + ppi < bp.n ? q0 + ppi : bp.n;
         for (long long q = q0; q < q1; ++q) {
             const int64_t i = bp.order ? (int64_t)__ldg(&bp.order[q]) : (int64_t)q;
-            cast_point<kStats, kWide>(bp.nodes, bp.tris, bp.max_steps, bp.scene_maxabs, bp.P, bp.N, i, tdirs, W,
-                                      eps, row, bp.bits, bp.count, acc, 0, -1, nullptr, 0, nullptr, front);
+            cast_point<kStats, kKind>(bp.nodes, bp.tris, bp.max_steps, bp.scene_maxabs, bp.P, bp.N, i, tdirs, W, eps,
+                                      s_dyn, bp.bits, bp.count, acc);
         }
     }
     if (cur >= 0) flush_part_counters(parts[cur].counters, acc);
@@ -1113,7 +1765,7 @@ k_batch(const BatchPart* __restrict__ parts, int n_parts, long long n_items, int
 // mask[f n + i] afterwards.
 // ---------------------------------------------------------------------------
 template <bool kStats, bool kWide>
-__global__ void __launch_bounds__(128, RC_BATCH_MIN_BLOCKS)
+__global__ void __launch_bounds__(128, RC_AXIS_MIN_BLOCKS)
 k_orthogonal_axis(const float4* __restrict__ nodes, const float4* __restrict__ tris, int max_steps,
                   float scene_maxabs, const float* __restrict__ P, const float* __restrict__ Nrm, int64_t n,
                   const int32_t* __restrict__ order, const FrameDev* __restrict__ fds, int nf, double eps,
@@ -1200,7 +1852,7 @@ __global__ void k_mask_pack(const uint32_t* __restrict__ mbits, int64_t m, uint8
 // gather in mbits[i] (zeroed by the caller).
 // ---------------------------------------------------------------------------
 template <bool kWide>
-__global__ void __launch_bounds__(128, RC_BATCH_MIN_BLOCKS)
+__global__ void __launch_bounds__(128, RC_AXIS_MIN_BLOCKS)
 k_tool_cast_axis(const float4* __restrict__ nodes, const float4* __restrict__ tris, int max_steps,
                  float scene_maxabs, const float* __restrict__ P, const float* __restrict__ Nrm, int64_t n,
                  const int32_t* __restrict__ order, const FrameDev* __restrict__ fd, double eps, double par_tol,
@@ -1312,6 +1964,12 @@ static int max_steps(rc_bvh h) { return (int)(2 * (h->n_int + h->T) + 64); }
 // the 4-wide tree is the default; tree_width 2 selects the binary tree
 bool use_wide(const rc_params* p) { return p->tree_width != 2; }
 
+// the point casts' walk: 32-bit pairs wherever a code fits (see PairOf)
+static int cast_kind(const rc_params* p, int64_t max_tris)
+{
+    return !use_wide(p) ? kBinary : max_tris <= kPairTris ? kWide4 : kWide4Big;
+}
+
 static int g_sm_count = 0;
 
 static int sm_count()
@@ -1365,13 +2023,8 @@ rc_status launch_hemisphere(rc_bvh h, const float* P, const float* N, int64_t n,
     if (blocks > 0x7FFFFFFF) return set_error(RC_E_UNSUPPORTED, "too many points for one launch");
     if (p->launch_mode == 1) work = nullptr;
     const bool wide = use_wide(p);
-    const size_t smem = cast_smem(threads / 32, (p->n_dirs + 31) / 32, wide);
-    if (smem > 48 * 1024) {
-        RC_CUDA(cudaFuncSetAttribute(k_hemisphere<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        RC_CUDA(cudaFuncSetAttribute(k_hemisphere<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        RC_CUDA(cudaFuncSetAttribute(k_hemisphere<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        RC_CUDA(cudaFuncSetAttribute(k_hemisphere<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    }
+    const int kind = cast_kind(p, h->T);
+    const size_t smem = cast_smem(threads / 32, (p->n_dirs + 31) / 32, kind, stats);
     const float4* tree = wide ? h->wnodes : h->nodes;
     {
         // the last points (RC_TAIL_POINTS per resident warp) are cast in parts;
@@ -1391,16 +2044,19 @@ rc_status launch_hemisphere(rc_bvh h, const float* P, const float* N, int64_t n,
             k_zero_split<<<(unsigned)((n_split * W + 255) / 256), 256, 0, s>>>(order, n - n_split, n, W, bits, count);
             RC_LAUNCHED();
         }
-#define RC_HEMI(ST, WD)                                                                                    \
-    k_hemisphere<ST, WD><<<(unsigned)blocks, threads, smem, s>>>(tree, h->tris, max_steps(h), h->scene_maxabs, \
-                                                                 P, N, n, order, h->tdirs, p->n_dirs,         \
-                                                                 p->origin_offset, bits, count, counters, work, \
-                                                                 n - n_split, splits, relist, relist_cap)
-        if (stats && wide) RC_HEMI(true, true);
-        else if (stats) RC_HEMI(true, false);
-        else if (wide) RC_HEMI(false, true);
-        else RC_HEMI(false, false);
-#undef RC_HEMI
+        const auto run = [&](auto kernel) -> rc_status {
+            if (smem > 48 * 1024)
+                RC_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            kernel<<<(unsigned)blocks, threads, smem, s>>>(tree, h->tris, max_steps(h), h->scene_maxabs, P, N, n, order,
+                                                           h->tdirs, p->n_dirs, p->origin_offset, bits, count, counters,
+                                                           work, n - n_split, splits, relist, relist_cap);
+            return RC_OK;
+        };
+        rc_status st = RC_OK;
+        if (kind == kWide4) st = stats ? run(k_hemisphere<true, kWide4>) : run(k_hemisphere<false, kWide4>);
+        else if (kind == kBinary) st = stats ? run(k_hemisphere<true, kBinary>) : run(k_hemisphere<false, kBinary>);
+        else st = stats ? run(k_hemisphere<true, kWide4Big>) : run(k_hemisphere<false, kWide4Big>);
+        if (st != RC_OK) return st;
     }
     RC_LAUNCHED();
     return RC_OK;
@@ -1426,7 +2082,7 @@ rc_status launch_hemisphere_update(rc_bvh h, const float* P, const float* N, int
         if (st != RC_OK) return st;
     }
     const int threads = 128;
-    const int per_sm = p->blocks_per_sm > 0 ? p->blocks_per_sm : RC_HEMI_MIN_BLOCKS;
+    const int per_sm = p->blocks_per_sm > 0 ? p->blocks_per_sm : RC_UPDATE_MIN_BLOCKS;
     int64_t blocks = (int64_t)sm_count() * per_sm;
     const int64_t need = (n * 32 + threads - 1) / threads;
     if (blocks > need) blocks = need;
@@ -1545,7 +2201,7 @@ rc_status launch_orthogonal_frames_into(rc_bvh h, const float* P, const float* N
     RC_CUDA(cudaMemsetAsync(mbits, 0, sizeof(uint32_t) * (mw + 2), s));
     unsigned long long* work = (unsigned long long*)(mbits + mw);
     const int64_t items = (int64_t)nf * 6 * ((n + 31) / 32);
-    const int64_t cap = (int64_t)sm_count() * RC_BATCH_MIN_BLOCKS;
+    const int64_t cap = (int64_t)sm_count() * RC_AXIS_MIN_BLOCKS;
     int64_t blocks = (items + 3) / 4;
     if (blocks > cap && p->launch_mode == 0) blocks = cap;
     if (p->launch_mode == 1) work = nullptr;
@@ -1626,7 +2282,7 @@ rc_status launch_tool_cast(rc_bvh h, const float* P, const float* N, int64_t n, 
     if (st == RC_OK && order) st = point_order(h, P, n, order, s);
     if (st == RC_OK) {
         int64_t blocks = (6 * ((n + 31) / 32) + 3) / 4;
-        const int64_t cap = (int64_t)sm_count() * RC_BATCH_MIN_BLOCKS;
+        const int64_t cap = (int64_t)sm_count() * RC_AXIS_MIN_BLOCKS;
         if (blocks > cap) blocks = cap;
         unsigned long long* work = (unsigned long long*)(mbits + mw);
         if (use_wide(p))
@@ -1653,32 +2309,35 @@ rc_status launch_tool_cast(rc_bvh h, const float* P, const float* N, int64_t n, 
 }
 
 rc_status launch_batch(const BatchPart* d_parts, int n_parts, long long n_items, int ppi, const float4* tdirs,
-                       const rc_params* p, unsigned long long* work, cudaStream_t s)
+                       const rc_params* p, int64_t max_tris, unsigned long long* work, cudaStream_t s)
 {
     const int threads = 128;
-    const size_t smem = cast_smem(threads / 32, (p->n_dirs + 31) / 32, use_wide(p));
+    const int kind = cast_kind(p, max_tris);
+    const size_t smem = cast_smem(threads / 32, (p->n_dirs + 31) / 32, kind, false);
     const int per_sm = p->blocks_per_sm > 0 ? p->blocks_per_sm : RC_BATCH_MIN_BLOCKS;
     int64_t blocks = (int64_t)sm_count() * per_sm;
     const int64_t need = (n_items * 32 + threads - 1) / threads;
     if (blocks > need) blocks = need;
     if (blocks < 1) blocks = 1;
-    if (use_wide(p))
-        k_batch<false, true><<<(unsigned)blocks, threads, smem, s>>>(d_parts, n_parts, n_items, ppi, tdirs,
-                                                                    p->n_dirs, p->origin_offset, work);
-    else
-        k_batch<false, false><<<(unsigned)blocks, threads, smem, s>>>(d_parts, n_parts, n_items, ppi, tdirs,
-                                                                     p->n_dirs, p->origin_offset, work);
+    const auto kernel = kind == kWide4 ? k_batch<false, kWide4> : kind == kBinary ? k_batch<false, kBinary>
+                                                                                   : k_batch<false, kWide4Big>;
+    kernel<<<(unsigned)blocks, threads, smem, s>>>(d_parts, n_parts, n_items, ppi, tdirs, p->n_dirs, p->origin_offset,
+                                                   work);
     RC_LAUNCHED();
     return RC_OK;
 }
 
 rc_status prepare_batch_kernel(int n_dirs)
 {
-    const size_t smem = cast_smem(4, (n_dirs + 31) / 32, true);
-    if (smem > 48 * 1024) {
-        RC_CUDA(cudaFuncSetAttribute(k_batch<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        RC_CUDA(cudaFuncSetAttribute(k_batch<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    }
+    const int W = (n_dirs + 31) / 32;
+    const auto allow = [&](auto kernel, int kind) {
+        const size_t smem = cast_smem(4, W, kind, false);
+        return smem > 48 * 1024 ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
+                                : cudaSuccess;
+    };
+    RC_CUDA(allow(k_batch<false, kBinary>, kBinary));
+    RC_CUDA(allow(k_batch<false, kWide4>, kWide4));
+    RC_CUDA(allow(k_batch<false, kWide4Big>, kWide4Big));
     return RC_OK;
 }
 

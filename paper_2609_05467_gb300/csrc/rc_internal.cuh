@@ -39,6 +39,11 @@ void count_launch(int k = 1);
 #define RC_LEAF_MAX 2
 #endif
 constexpr int kLeafMax = RC_LEAF_MAX;   // triangles per packed leaf (1..8)
+constexpr int kLeafBits = kLeafMax <= 2 ? 1 : 3;   // leaf codes: -1 - (first << kLeafBits | count - 1)
+static_assert(kLeafMax <= 8, "a leaf code has at most three bits for its count");
+__host__ __device__ __forceinline__ int leaf_code(int first, int cnt) { return -1 - ((first << kLeafBits) | (cnt - 1)); }
+__host__ __device__ __forceinline__ int leaf_first(int code) { return (-1 - code) >> kLeafBits; }
+__host__ __device__ __forceinline__ int leaf_count(int code) { return ((-1 - code) & ((1 << kLeafBits) - 1)) + 1; }
 constexpr int kStack = 64;         // binary traversal stack entries (>= max tree depth)
 constexpr int kStack4 = 96;        // 4-wide traversal stack entries (>= 3 * wide depth + 1)
 constexpr double kTau = 1e-9;      // relative ambiguity band of the occlusion test
@@ -126,6 +131,13 @@ void fill_summary(const long long* sums, const double* wsum, int64_t n, int32_t 
 
 }  // namespace rc
 
+// Where float4 c (0..7) of 4-wide node w lies.  Lanes that read the same
+// float4 of 32 different 128-byte nodes would all meet in the same four of
+// L1's 32 banks; each node's float4s are therefore permuted by its number.
+namespace rc {
+__host__ __device__ __forceinline__ int64_t wide_at(int64_t w, int c) { return 8 * w + (c ^ (int)(w & 7)); }
+}  // namespace rc
+
 struct rc_bvh_s {
     int device = 0;
     int builder = 0;               // RC_BUILDER_KARRAS or RC_BUILDER_PLOC
@@ -134,7 +146,7 @@ struct rc_bvh_s {
     int32_t* F = nullptr;          // [T][3] copy of the faces
     float4* tris = nullptr;        // [T][3] triangle records in Morton order
     float4* nodes = nullptr;       // [n_int][4] packed BVH2 nodes
-    float4* wnodes = nullptr;      // [<= n_int][8] packed 4-wide nodes
+    float4* wnodes = nullptr;      // [<= n_int][8] packed 4-wide nodes (wide_at)
     int wide_depth = 0;
     int64_t n_int = 0;             // internal nodes (>= 1)
     int32_t* parent = nullptr;     // [n_int + T]: parent of internal i at i, of leaf k at n_int+k

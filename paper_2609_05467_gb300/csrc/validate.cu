@@ -22,8 +22,7 @@ struct CheckCounts {
 
 __device__ __forceinline__ bool leaf_ok(int32_t c, int64_t T)
 {
-    const int32_t v = -1 - c;
-    const int64_t first = v >> 3, cnt = (v & 7) + 1;
+    const int64_t first = leaf_first(c), cnt = leaf_count(c);
     return first >= 0 && first + cnt <= T;
 }
 
@@ -37,10 +36,9 @@ __global__ void k_check_wide_level(const float4* __restrict__ wnodes, int64_t n_
     if (t >= min(*qin_count, cap)) return;
     const int32_t w = qin[t];
     atomicAdd(&cc->nodes_seen, 1ULL);
-    const float4* nd = wnodes + 8 * (int64_t)w;
-    const float4 ci = nd[6];
+    const float4 ci = wnodes[wide_at(w, 6)];
     const int32_t c[4] = {__float_as_int(ci.x), __float_as_int(ci.y), __float_as_int(ci.z), __float_as_int(ci.w)};
-    const float4 lx = nd[0], hx = nd[1], ly = nd[2], hy = nd[3], lz = nd[4], hz = nd[5];
+    const float4 lx = wnodes[wide_at(w, 0)], hx = wnodes[wide_at(w, 1)], ly = wnodes[wide_at(w, 2)], hy = wnodes[wide_at(w, 3)], lz = wnodes[wide_at(w, 4)], hz = wnodes[wide_at(w, 5)];
     const float lo[3][4] = {{lx.x, lx.y, lx.z, lx.w}, {ly.x, ly.y, ly.z, ly.w}, {lz.x, lz.y, lz.z, lz.w}};
     const float hi[3][4] = {{hx.x, hx.y, hx.z, hx.w}, {hy.x, hy.y, hy.z, hy.w}, {hz.x, hz.y, hz.z, hz.w}};
     for (int k = 0; k < 4; ++k) {
