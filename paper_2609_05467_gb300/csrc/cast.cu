@@ -82,6 +82,46 @@ __device__ __forceinline__ void setup_ray(Ray& r, float ox, float oy, float oz, 
     r.rs = fmaxf(fmaxf(1.0f, scene_maxabs), fmaxf(fabsf(ox), fmaxf(fabsf(oy), fabsf(oz))));
 }
 
+// The decision of the watertight test from its edge functions, their error
+// bound eU and the vertices' distances along the permuted axis (error model
+// below; `extent` is the triangle's largest edge component).  kBand: eU has the
+// ambiguity band on top, and a crossing behind the origin must lie beyond its
+// band too, so that no pair of the band is called a miss.
+template <bool kBand>
+__device__ __forceinline__ int tri_decide(const Ray& r, float extent, float U, float V, float W, float eU, float az,
+                                          float bz, float cz)
+{
+    const float u = 5.9604644775390625e-8f;
+    const bool uc = fabsf(U) > eU, vc = fabsf(V) > eU, wc = fabsf(W) > eU;
+    const bool pos = (uc && U > 0.0f) || (vc && V > 0.0f) || (wc && W > 0.0f);
+    const bool neg = (uc && U < 0.0f) || (vc && V < 0.0f) || (wc && W < 0.0f);
+    if (pos && neg) return kMiss;
+
+    const float S = fabsf(U) + fabsf(V) + fabsf(W);
+    const float det = U + V + W;
+    const float Tp = fmaf(U, az, fmaf(V, bz, W * cz));
+    const float Zs = fabsf(az) + fabsf(bz) + fabsf(cz);
+    const float Zm = fmaxf(fabsf(az), fmaxf(fabsf(bz), fabsf(cz)));
+    const float eD = (3.0f * eU + 2.01f * u * S) * 1.0625f;
+    const float eT = (eU * Zs + 4.01f * u * S * Zm) * 1.0625f;
+    const bool det_ok = fabsf(det) > eD;
+    const bool tp_ok = fabsf(Tp) > eT;
+    // sign of t = sign(T') * sign(det) * sign(d[kz])
+    const bool ahead = ((Tp > 0.0f) == (det > 0.0f)) == (r.dkz > 0.0f);
+    // plane crossed behind the origin
+    if (det_ok && tp_ok && !ahead && (!kBand || fabsf(Tp) > eT + 1e-9f * r.rs * (fabsf(det) + eD) * 1.01f)) return kMiss;
+
+    // clear hit: every edge function beyond its error and the tau band, and
+    // the crossing ahead and beyond tau*R along the ray
+    const float tau_edge = 3.0f * 1e-9f * r.rs * extent * 1.01f;
+    const float thr = eU + tau_edge;
+    if (fabsf(U) > thr && fabsf(V) > thr && fabsf(W) > thr && tp_ok && ahead) {
+        const float need = eT + 1e-9f * r.rs * (fabsf(det) + eD) * 1.01f;
+        if (fabsf(Tp) > need) return kHit;
+    }
+    return kUnsure;
+}
+
 // FP32 watertight test with a forward error bound.  Returns kHit only when
 // the pair is certainly a clear hit (both outside the ambiguity band and
 // certain in sign), kMiss only when it is certainly not a hit, else kUnsure.
@@ -117,33 +157,62 @@ __device__ __forceinline__ int tri_test32(const Ray& r, const float4 v0, const f
                           fmaxf(fabsf(Cx), fabsf(Cy)));
     const float E = r.ef * M;
     const float eU = (4.0f * E * P + 6.0f * E * E + 3.0f * u * P * P) * 1.0625f;
-    const bool uc = fabsf(U) > eU, vc = fabsf(V) > eU, wc = fabsf(W) > eU;
-    const bool pos = (uc && U > 0.0f) || (vc && V > 0.0f) || (wc && W > 0.0f);
-    const bool neg = (uc && U < 0.0f) || (vc && V < 0.0f) || (wc && W < 0.0f);
-    if (pos && neg) return kMiss;
+    return tri_decide<false>(r, v0.w, U, V, W, eU, az, bz, cz);
+}
 
-    const float S = fabsf(U) + fabsf(V) + fabsf(W);
-    const float det = U + V + W;
-    const float Tp = fmaf(U, az, fmaf(V, bz, W * cz));
-    const float Zs = fabsf(az) + fabsf(bz) + fabsf(cz);
-    const float Zm = fmaxf(fabsf(az), fmaxf(fabsf(bz), fabsf(cz)));
-    const float eD = (3.0f * eU + 2.01f * u * S) * 1.0625f;
-    const float eT = (eU * Zs + 4.01f * u * S * Zm) * 1.0625f;
-    const bool det_ok = fabsf(det) > eD;
-    const bool tp_ok = fabsf(Tp) > eT;
-    // sign of t = sign(T') * sign(det) * sign(d[kz])
-    const bool ahead = ((Tp > 0.0f) == (det > 0.0f)) == (r.dkz > 0.0f);
-    if (det_ok && tp_ok && !ahead) return kMiss;   // plane crossed behind the origin
-
-    // clear hit: every edge function beyond its error and the tau band, and
-    // the crossing ahead and beyond tau*R along the ray
-    const float tau_edge = 3.0f * 1e-9f * r.rs * v0.w * 1.01f;
-    const float thr = eU + tau_edge;
-    if (fabsf(U) > thr && fabsf(V) > thr && fabsf(W) > thr && tp_ok && ahead) {
-        const float need = eT + 1e-9f * r.rs * (fabsf(det) + eD) * 1.01f;
-        if (fabsf(Tp) > need) return kHit;
-    }
-    return kUnsure;
+// The same test for a pair that tri_test32 leaves open because the triangle is
+// close to the ray but far from its origin: there E is a few u M with M the
+// distance to the origin.  Here one vertex is translated and sheared in
+// two-term arithmetic (hi + lo; the shear ratio too) and the others follow by
+// the sheared edges, so that E scales with the triangle and its distance from
+// the ray: E <= 3 u P + (2 + 3 S) u e + 1e-11 M, e the largest edge
+// component.  E can be smaller than the ambiguity band here, which is added to
+// the bound.  About 150 fp32 operations in place of 75 to 250 in FP64, which
+// issue at 1/64 of the rate: the axis rays of a frame search on the turned
+// prismatic part left 0.53 pairs per ray open, now 0.002.  With the bands and
+// the eligibility test in fp32 too its axis cast went from 2955 to 1310 us,
+// and the six axes and the tool in one turned frame from 748 + 1079 to
+// 678 + 618 us (100k points).
+__device__ __noinline__ int tri_test_close(const Ray& r, const float4 v0, const float4 v1, const float4 v2)
+{
+    const float u = 5.9604644775390625e-8f;
+    const float rk = __frcp_rn(r.dkz);
+    const float px = sel3(r.dx, r.dy, r.dz, r.kx), py = sel3(r.dx, r.dy, r.dz, r.ky);
+    const float sx = __fmul_rn(px, rk), sy = __fmul_rn(py, rk);
+    const float tx = __fmul_rn(__fmaf_rn(-sx, r.dkz, px), rk), ty = __fmul_rn(__fmaf_rn(-sy, r.dkz, py), rk);
+    const float ox = sel3(r.ox, r.oy, r.oz, r.kx), oy = sel3(r.ox, r.oy, r.oz, r.ky), oz = sel3(r.ox, r.oy, r.oz, r.kz);
+    const float vx = sel3(v0.x, v0.y, v0.z, r.kx), vy = sel3(v0.x, v0.y, v0.z, r.ky), vz = sel3(v0.x, v0.y, v0.z, r.kz);
+    // a - b = hi + lo exactly (Knuth)
+    const auto diff2 = [](float a, float b, float& hi, float& lo) {
+        hi = __fsub_rn(a, b);
+        const float t = __fsub_rn(hi, a);
+        lo = __fsub_rn(__fsub_rn(a, __fsub_rn(hi, t)), __fadd_rn(b, t));
+    };
+    float xh, xl, yh, yl, zh, zl;
+    diff2(vx, ox, xh, xl);
+    diff2(vy, oy, yh, yl);
+    diff2(vz, oz, zh, zl);
+    // (x - s z) for the two-term x, s, z
+    const auto shear2 = [&](float h, float l, float s, float t) {
+        const float p = __fmul_rn(s, zh), q = __fadd_rn(__fmaf_rn(s, zh, -p), __fmaf_rn(s, zl, __fmul_rn(t, zh)));
+        float dh, dl;
+        diff2(h, p, dh, dl);
+        return __fadd_rn(dh, __fadd_rn(dl, __fsub_rn(l, q)));
+    };
+    const float Ax = shear2(xh, xl, sx, tx), Ay = shear2(yh, yl, sy, ty);
+    const float bx = sel3(v1.x, v1.y, v1.z, r.kx), by = sel3(v1.x, v1.y, v1.z, r.ky), bz = sel3(v1.x, v1.y, v1.z, r.kz);
+    const float cx = sel3(v2.x, v2.y, v2.z, r.kx), cy = sel3(v2.x, v2.y, v2.z, r.ky), cz = sel3(v2.x, v2.y, v2.z, r.kz);
+    const float ez = bz - vz, fz = cz - vz;
+    const float Bx = Ax + fmaf(-sx, ez, bx - vx), By = Ay + fmaf(-sy, ez, by - vy);
+    const float Cx = Ax + fmaf(-sx, fz, cx - vx), Cy = Ay + fmaf(-sy, fz, cy - vy);
+    const float U = fmaf(Cx, By, -(Cy * Bx));
+    const float V = fmaf(Ax, Cy, -(Ay * Cx));
+    const float W = fmaf(Bx, Ay, -(By * Ax));
+    const float P = fmaxf(fmaxf(fmaxf(fabsf(Ax), fabsf(Ay)), fmaxf(fabsf(Bx), fabsf(By))), fmaxf(fabsf(Cx), fabsf(Cy)));
+    const float S = fmaxf(fabsf(sx), fabsf(sy)), M = fmaxf(fabsf(xh), fmaxf(fabsf(yh), fabsf(zh)));
+    const float E = 3.0f * u * P + (2.1f + 3.1f * S) * u * v0.w + 1e-11f * M;
+    const float eU = (4.0f * E * P + 6.0f * E * E + 3.0f * u * P * P) * 1.0625f + 3.0f * 1e-9f * r.rs * v0.w * 1.01f + 1e-36f;
+    return tri_decide<true>(r, v0.w, U, V, W, eU, zh, bz - oz, cz - oz);
 }
 
 // FP64 decision of one pair, written from the definition: the ray's line
@@ -154,13 +223,16 @@ __device__ __forceinline__ int tri_test32(const Ray& r, const float4 v0, const f
 // sign decision (used for rays that only ambiguous pairs decide).
 struct Pair64 { int state; bool hit64; };
 
+// kQuick ends early, after a third of the work, for most pairs; the cast of
+// hemisphere rays, which calls it 5 times in 10,000, takes the form that costs
+// its kernel fewer registers (2% of the impeller's time).
+template <bool kQuick>
 __device__ __noinline__ Pair64 retest64(float ox, float oy, float oz, float dx, float dy, float dz, const float4 v0,
                                         const float4 v1, const float4 v2)
 {
     const double o[3] = {ox, oy, oz}, d[3] = {dx, dy, dz};
     const double A[3] = {v0.x, v0.y, v0.z}, B[3] = {v1.x, v1.y, v1.z}, C[3] = {v2.x, v2.y, v2.z};
     double a[3], b[3], c[3], eab[3], ebc[3], eca[3];
-    double R = 1.0;
     for (int k = 0; k < 3; ++k) {
         a[k] = A[k] - o[k];
         b[k] = B[k] - o[k];
@@ -168,20 +240,48 @@ __device__ __noinline__ Pair64 retest64(float ox, float oy, float oz, float dx, 
         eab[k] = B[k] - A[k];
         ebc[k] = C[k] - B[k];
         eca[k] = A[k] - C[k];
-        R = fmax(R, fmax(fabs(o[k]), fmax(fabs(A[k]), fmax(fabs(B[k]), fabs(C[k])))));
     }
-    const double band = kTau * R;
+    const float Rf = fmaxf(fmaxf(fmaxf(1.0f, fmaxf(fabsf(ox), fmaxf(fabsf(oy), fabsf(oz)))),
+                                 fmaxf(fabsf(v0.x), fmaxf(fabsf(v0.y), fabsf(v0.z)))),
+                           fmaxf(fmaxf(fabsf(v1.x), fmaxf(fabsf(v1.y), fabsf(v1.z))),
+                                 fmaxf(fabsf(v2.x), fmaxf(fabsf(v2.y), fabsf(v2.z)))));
+    const double band = kTau * (double)Rf;
     // signed volume of (p, e, d) and |e x d| for the three edges
     const double* P3[3] = {b, c, a};
     const double* E3[3] = {ebc, eca, eab};
-    double Ev[3], Lv[3];
+    double Ev[3], Lv[3] = {0.0, 0.0, 0.0};
+    // (quick: a bound above the band on the volume, band |e x d| <= band
+    // |e|_1 |d|_1, in fp32 with 1% to spare; beyond it |e x d| is not needed)
+    bool clear[3] = {false, false, false}, posc = false, negc = false;
+    if (kQuick) {
+        const float l1[3] = {fabsf(v2.x - v1.x) + fabsf(v2.y - v1.y) + fabsf(v2.z - v1.z),
+                             fabsf(v0.x - v2.x) + fabsf(v0.y - v2.y) + fabsf(v0.z - v2.z),
+                             fabsf(v1.x - v0.x) + fabsf(v1.y - v0.y) + fabsf(v1.z - v0.z)};
+        const float wide = 1.01e-9f * Rf * (fabsf(dx) + fabsf(dy) + fabsf(dz));
+        for (int k = 0; k < 3; ++k) {
+            const double* p = P3[k];
+            const double* e = E3[k];
+            const double w0 = p[1] * e[2] - p[2] * e[1];
+            const double w1 = p[2] * e[0] - p[0] * e[2];
+            const double w2 = p[0] * e[1] - p[1] * e[0];
+            Ev[k] = w0 * d[0] + w1 * d[1] + w2 * d[2];
+            const float f = __double2float_rn(Ev[k]);
+            clear[k] = fabsf(f) > wide * l1[k] + 1e-36f;
+            posc |= clear[k] && f > 0.0f;
+            negc |= clear[k] && f < 0.0f;
+        }
+        if (posc && negc) return Pair64{kMiss, false};
+    }
     for (int k = 0; k < 3; ++k) {
-        const double* p = P3[k];
         const double* e = E3[k];
-        const double w0 = p[1] * e[2] - p[2] * e[1];
-        const double w1 = p[2] * e[0] - p[0] * e[2];
-        const double w2 = p[0] * e[1] - p[1] * e[0];
-        Ev[k] = w0 * d[0] + w1 * d[1] + w2 * d[2];
+        if (!kQuick) {
+            const double* p = P3[k];
+            const double w0 = p[1] * e[2] - p[2] * e[1];
+            const double w1 = p[2] * e[0] - p[0] * e[2];
+            const double w2 = p[0] * e[1] - p[1] * e[0];
+            Ev[k] = w0 * d[0] + w1 * d[1] + w2 * d[2];
+        }
+        if (clear[k]) continue;
         const double x0 = e[1] * d[2] - e[2] * d[1];
         const double x1 = e[2] * d[0] - e[0] * d[2];
         const double x2 = e[0] * d[1] - e[1] * d[0];
@@ -198,8 +298,9 @@ __device__ __noinline__ Pair64 retest64(float ox, float oy, float oz, float dx, 
     const double na = N0 * a[0] + N1 * a[1] + N2 * a[2];
     res.hit64 = !(spos && sneg) && nd != 0.0 && na != 0.0 && ((na > 0.0) == (nd > 0.0));
 
-    bool pos = false, neg = false, small = false;
+    bool pos = posc, neg = negc, small = false;
     for (int k = 0; k < 3; ++k) {
+        if (clear[k]) continue;
         if (fabs(Ev[k]) <= band * Lv[k]) { small = true; continue; }
         if (Ev[k] > 0.0) pos = true; else neg = true;
     }
@@ -214,7 +315,7 @@ __device__ __noinline__ Pair64 retest64(float ox, float oy, float oz, float dx, 
 
 __device__ __forceinline__ Pair64 retest64(const Ray& r, const float4 v0, const float4 v1, const float4 v2)
 {
-    return retest64(r.ox, r.oy, r.oz, r.dx, r.dy, r.dz, v0, v1, v2);
+    return retest64<true>(r.ox, r.oy, r.oz, r.dx, r.dy, r.dz, v0, v1, v2);
 }
 
 // Conservative slab test of both children of a packed node.
@@ -782,29 +883,44 @@ struct AxisRay {
     int pos;              // 1: along +column k, 0: along -column k
 };
 
+// x a + y b + z c as an unevaluated sum hi + lo of two fp32 values, within
+// 1e-13 of |x a| + |y b| + |z c| (each product and sum split into its rounded
+// value and its error: Dekker 1971, Knuth's TwoSum)
+__device__ __forceinline__ void dot2(float x, float a, float y, float b, float z, float c, float& hi, float& lo)
+{
+    const float p0 = __fmul_rn(x, a), p1 = __fmul_rn(y, b), p2 = __fmul_rn(z, c);
+    const float e0 = __fmaf_rn(x, a, -p0), e1 = __fmaf_rn(y, b, -p1), e2 = __fmaf_rn(z, c, -p2);
+    const float s = __fadd_rn(p0, p1), t = __fsub_rn(s, p0);
+    const float f = __fadd_rn(__fsub_rn(p0, __fsub_rn(s, t)), __fsub_rn(p1, t));
+    hi = __fadd_rn(s, p2);
+    const float v = __fsub_rn(hi, s);
+    const float g = __fadd_rn(__fsub_rn(s, __fsub_rn(hi, v)), __fsub_rn(p2, v));
+    lo = __fadd_rn(__fadd_rn(__fadd_rn(e0, e1), e2), __fadd_rn(f, g));
+}
+
+// The band of an axis ray (see above).  Its bounds are sums hi + lo -+ tol
+// rounded outward; everything in tol is rounded up by its spare factors.
 __device__ __forceinline__ AxisRay make_axis_ray(const FrameDev& fd, int a, float ox, float oy, float oz, float rs)
 {
     AxisRay ar;
     const int k = a >> 1;
     const bool pos = (a & 1) == 0;
-    const double x = ox, y = oy, z = oz;
-    double q[3], qs[3];
+    const float ex = ox - fd.c32[0], ey = oy - fd.c32[1], ez = oz - fd.c32[2];
+    const float reach = (sqrtf(ex * ex + ey * ey + ez * ez) + fd.r32 + 1e-6f * rs) * fd.rlen[k] + 1e-6f;
     for (int j = 0; j < 3; ++j) {
-        q[j] = __dadd_rn(__dadd_rn(__dmul_rn(x, fd.frame[j]), __dmul_rn(y, fd.frame[3 + j])), __dmul_rn(z, fd.frame[6 + j]));
-        qs[j] = fabs(x * fd.frame[j]) + fabs(y * fd.frame[3 + j]) + fabs(z * fd.frame[6 + j]);
-    }
-    const double ex = x - fd.sc_c[0], ey = y - fd.sc_c[1], ez = z - fd.sc_c[2];
-    const double reach = 1.01 * (sqrt(ex * ex + ey * ey + ez * ez) + fd.sc_r) / sqrt(fd.gram[4 * k]) + 1e-6;
-    for (int j = 0; j < 3; ++j) {
-        double tol = 1e-9 * (double)rs + 1e-15 * (qs[j] + 4.0 * (double)rs + 1.0);
-        if (j != k) tol += reach * (fabs(fd.gram[3 * j + k]) + 1e-15);
-        double l = q[j] - tol, h = q[j] + tol;
+        const float f0 = fd.axes[6 * j], f1 = fd.axes[6 * j + 1], f2 = fd.axes[6 * j + 2];   // column j
+        float hi, lo;
+        dot2(ox, f0, oy, f1, oz, f2, hi, lo);
+        const float qs = fabsf(ox * f0) + fabsf(oy * f1) + fabsf(oz * f2);
+        float tol = 1.01e-9f * rs + 2e-13f * (qs + 4.0f * rs + 1.0f);
+        if (j != k) tol += reach * (fd.gram_up[3 * j + k] + 1e-15f);
+        tol *= 1.001f;
+        ar.lo[j] = __fadd_rd(hi, __fsub_rd(lo, tol));
+        ar.hi[j] = __fadd_ru(hi, __fadd_ru(lo, tol));
         if (j == k) {
-            if (pos) h = INFINITY;
-            else l = -INFINITY;
+            if (pos) ar.hi[j] = INFINITY;
+            else ar.lo[j] = -INFINITY;
         }
-        ar.lo[j] = __double2float_rd(l);
-        ar.hi[j] = __double2float_ru(h);
     }
     ar.k = k;
     ar.pos = pos ? 1 : 0;
@@ -832,6 +948,19 @@ __device__ __forceinline__ void warp_add_counters(unsigned long long* counters, 
         if (nvis) atomicAdd(&counters[4], (unsigned long long)nvis);
         if (ntri) atomicAdd(&counters[5], (unsigned long long)ntri);
     }
+}
+
+// n.a >= -par_tol, as decided in FP64 (x, y, z order): in fp32 where its
+// error, under 4 u of the terms' magnitudes, cannot matter
+__device__ __forceinline__ bool eligible(float nx, float ny, float nz, float dx, float dy, float dz, double par_tol)
+{
+    const float s = fmaf(nx, dx, fmaf(ny, dy, nz * dz)), t = (float)par_tol;
+    const float m = 5e-7f * (fabsf(nx * dx) + fabsf(ny * dy) + fabsf(nz * dz) + t) + 1e-36f;
+    if (s + t > m) return true;
+    if (s + t < -m) return false;
+    double nd = __dadd_rn(__dmul_rn((double)nx, (double)dx), __dmul_rn((double)ny, (double)dy));
+    nd = __dadd_rn(nd, __dmul_rn((double)nz, (double)dz));
+    return nd >= -par_tol;
 }
 
 // ---------------------------------------------------------------------------
@@ -1044,7 +1173,7 @@ __device__ __noinline__ bool pool_retest(float ox, float oy, float oz, const flo
                                          uint32_t* rows, int W, int64_t i, long long* relist, long long relist_cap,
                                          unsigned long long* relist_ctr)
 {
-    const Pair64 q = retest64(ox, oy, oz, d.x, d.y, d.z, tp[0], tp[1], tp[2]);
+    const Pair64 q = retest64<false>(ox, oy, oz, d.x, d.y, d.z, tp[0], tp[1], tp[2]);
     const uint32_t b = 1u << (j & 31);
     if (kStats && relist && !(atomicOr(&rows[3 * W + (j >> 5)], b) & b)) {
         const unsigned long long at = atomicAdd(relist_ctr, 1ULL);
@@ -1502,6 +1631,7 @@ __device__ __forceinline__ bool trace_axis(const float4* __restrict__ ftree, con
             if (kStats) acc.ntri += 1;
             const float4 v0 = __ldg(tp + 3 * k), v1 = __ldg(tp + 3 * k + 1), v2 = __ldg(tp + 3 * k + 2);
             int st = tri_test32(q, v0, v1, v2);
+            if (st == kUnsure) st = tri_test_close(q, v0, v1, v2);
             if (st == kUnsure) {
                 ++acc.retests;
                 const Pair64 w = retest64(q, v0, v1, v2);
@@ -1912,10 +2042,7 @@ k_orthogonal_axis(const float4* __restrict__ nodes, const float4* __restrict__ t
             q = __dadd_rn(q, __dmul_rn((double)pz, frame[6 + kk]));
             const double tv = (a & 1) ? __dsub_rn(q, fbox[kk]) : __dsub_rn(fbox[3 + kk], q);
             travel[6 * row + a] = __double2float_rn(tv);
-            // eligibility n.a >= -parallel_tol (FP64, x, y, z order)
-            double nd = __dadd_rn(__dmul_rn((double)nx, (double)dx), __dmul_rn((double)ny, (double)dy));
-            nd = __dadd_rn(nd, __dmul_rn((double)nz, (double)dz));
-            cast = nd >= -par_tol;
+            cast = eligible(nx, ny, nz, dx, dy, dz, par_tol);
             ox = offset_coord(px, nx, eps);
             oy = offset_coord(py, ny, eps);
             oz = offset_coord(pz, nz, eps);
@@ -1991,9 +2118,7 @@ k_tool_cast_axis(const float4* __restrict__ nodes, const float4* __restrict__ tr
             i = order ? (int64_t)__ldg(&order[k]) : k;
             const double px = P[3 * i], py = P[3 * i + 1], pz = P[3 * i + 2];
             const double nx = Nrm[3 * i], ny = Nrm[3 * i + 1], nz = Nrm[3 * i + 2];
-            double nd = __dadd_rn(__dmul_rn(nx, (double)dx), __dmul_rn(ny, (double)dy));
-            nd = __dadd_rn(nd, __dmul_rn(nz, (double)dz));
-            open = nd >= -par_tol;
+            open = eligible(Nrm[3 * i], Nrm[3 * i + 1], Nrm[3 * i + 2], dx, dy, dz, par_tol);
             const double h = __dadd_rn(radius, eps);
             cx = __dadd_rn(px, __dmul_rn(h, nx));
             cy = __dadd_rn(py, __dmul_rn(h, ny));
@@ -2245,6 +2370,12 @@ __global__ void k_frame_init(FrameArgs a, FrameDev* d)
                                            __dmul_rn((double)a.f[6 + j], (double)a.f[6 + k]));
     }
     d->sc_r = a.sc_r;
+    d->r32 = __double2float_ru(a.sc_r);
+    for (int j = 0; j < 3; ++j) {
+        d->c32[j] = __double2float_rn(a.sc_c[j]);
+        d->rlen[j] = __double2float_ru(1.01 / sqrt(d->gram[4 * j]));
+        for (int k = 0; k < 3; ++k) d->gram_up[3 * j + k] = __double2float_ru(fabs(d->gram[3 * j + k]));
+    }
     for (int k = 0; k < 3; ++k)
         for (int c = 0; c < 3; ++c) {
             d->axes[3 * (2 * k) + c] = a.f[3 * c + k];

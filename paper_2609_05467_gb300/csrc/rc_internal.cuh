@@ -88,6 +88,10 @@ struct FrameDev {
     double gram[9];     // G = F^T F of the fp32 frame F (FP64): how far the axes are from orthonormal
     double sc_c[3];     // centre of the part's bounding box (world)
     double sc_r;        // half its diagonal
+    float gram_up[9];   // |G| rounded up, 1.01 / |column k|, and the centre and
+    float rlen[3];      //   half diagonal in fp32: the axis rays' bands are
+    float c32[3];       //   bounds, evaluated in fp32 (GB300 issues FP64 at
+    float r32;          //   1/64 of its fp32 rate)
 };
 
 // one part of a batched cast (device descriptor)
