@@ -45,12 +45,6 @@ __device__ __forceinline__ f2 pack2(float a, float b)
     return r;
 }
 __device__ __forceinline__ void unpack2(f2 v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
-__device__ __forceinline__ f2 mul2(f2 a, f2 b)
-{
-    f2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
 __device__ __forceinline__ f2 add2(f2 a, f2 b)
 {
     f2 r;
@@ -62,6 +56,14 @@ __device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c)
     f2 r;
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
     return r;
+}
+// The rounded product: a fused multiply-add of minus zero, whose value the
+// compiler must not know.  It joins mul.rn.f32x2 and add.rn.f32x2 into a fused
+// multiply-add (for scalars it does not), which moved the largest component of
+// a direction in 30 of 10^6 points x 2048 directions.
+__device__ __forceinline__ f2 mul2(f2 a, f2 b, f2 minus_zero)
+{
+    return fma2(a, b, minus_zero);
 }
 
 // The exact direction sums of one point, by one warp: M_k = sum over visible
@@ -143,6 +145,8 @@ k_variability(const uint32_t* __restrict__ bits, const float* __restrict__ Nrm,
     __shared__ double wsh[2][kVarThreads / 32];
     const int lane = threadIdx.x & 31;
     const int W = (n_dirs + 31) >> 5, np = (W + 1) >> 1;
+    const float nzero = __int_as_float((int)(0x80000000u | (unsigned)(n >> 63)));   // n >= 0: -0.0f
+    const f2 mz = pack2(nzero, nzero);
     if (threadIdx.x < S_N) blk[threadIdx.x] = 0;
     if (kTable)
         for (int k = threadIdx.x; k < 32 * np; k += kVarThreads) {
@@ -191,9 +195,9 @@ k_variability(const uint32_t* __restrict__ bits, const float* __restrict__ Nrm,
                         hz = pack2(h0.z, h1.z);
                     }
                     // local_to_world for both
-                    const f2 dx = add2(add2(mul2(ax, hx), mul2(bx, hy)), mul2(cx, hz));
-                    const f2 dy = add2(add2(mul2(ay, hx), mul2(by, hy)), mul2(cy, hz));
-                    const f2 dz = add2(add2(mul2(az, hx), mul2(bz, hy)), mul2(cz, hz));
+                    const f2 dx = add2(add2(mul2(ax, hx, mz), mul2(bx, hy, mz)), mul2(cx, hz, mz));
+                    const f2 dy = add2(add2(mul2(ay, hx, mz), mul2(by, hy, mz)), mul2(cy, hz, mz));
+                    const f2 dz = add2(add2(mul2(az, hx, mz), mul2(bz, hy, mz)), mul2(cz, hz, mz));
                     const bool v0 = (u0 >> lane) & 1u, v1 = (u1 >> lane) & 1u;
                     const f2 on = pack2(v0 ? 1.0f : 0.0f, v1 ? 1.0f : 0.0f);
                     sx = fma2(on, dx, sx);

@@ -82,3 +82,19 @@ def test_near_ties_take_the_exact_sums():
     s, acc, dom, conc, _ = _run(bits, N, dirs)
     M, _, odom, oconc, cnt = oracle.variability(bits, N, dirs)
     assert np.array_equal(dom, odom) and np.array_equal(conc, np.asarray(oconc, np.float64).astype(np.float32))
+
+
+@pytest.mark.parametrize("n,dirs", [(400_000, 1000), (40_000, 4000)])
+def test_largest_components_are_rounded_as_stated(n, dirs):
+    """Products and sums of a direction round one by one: a fused multiply-add in their place moves the largest component
+    of about 1 direction in 10^8, so many points are needed to see it.  Counts: no tolerance."""
+    rng = np.random.default_rng(dirs)
+    N = rng.normal(size=(n, 3))
+    N = (N / np.linalg.norm(N, axis=1, keepdims=True)).astype(np.float32)
+    row = _rows(rng, 1, dirs, np.ones(1))[1]
+    bits = np.repeat(row, n, axis=0)
+    s, _, dom, conc, _ = _run(bits, N, dirs)
+    _, ac, odom, oconc, _ = oracle.variability(bits, N, dirs, 0)
+    assert np.array_equal(dom, odom)
+    assert np.array_equal(conc, oconc.astype(np.float32))
+    assert s.conc_sum_q == int(np.rint(oconc * 2.0 ** 40).astype(np.int64).sum())
