@@ -40,16 +40,36 @@ struct BuildScratch {
 // ---------------------------------------------------------------------------
 // face preparation and validation
 // ---------------------------------------------------------------------------
-__global__ void k_face_prep(const float* __restrict__ V, int64_t nV, const int32_t* __restrict__ F,
-                            int64_t T, float* fnorm, double* farea, float* tbox, DevScalars* sc)
+// fl32(c / len) from the FP64 product q = c * inv, where inv is within 2^-44 of
+// 1 / len (0: unknown): the same fp32 value unless q lies within 2^-43 of a
+// midpoint of two fp32 values (2^-42 taken; 4 in 10^6), or outside the range
+// of normal fp32 values.  No FP64 division where three were.
+__device__ __forceinline__ float quotient32(double c, double len, double inv)
 {
-    const int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    // contributions to the scene bounds, reduced over the warp before the
-    // atomics (one set per warp instead of per face); neutral when absent
+    if ((__double_as_longlong(c) << 1) == 0) return __int_as_float(__double2hiint(c) & 0x80000000);
+    const double q = __dmul_rn(c, inv);
+    const unsigned e = ((unsigned)__double2hiint(q) >> 20) & 0x7FFu;
+    const int low = (__double2loint(q) & 0x1FFFFFFF) - 0x10000000;
+    if (e < 1023u - 120u || e > 1023u + 120u || abs(low) <= 2048) return __double2float_rn(__ddiv_rn(c, len));
+    return narrow(q);
+}
+
+// Bound by FP64, which issues at 1/64 of the fp32 rate (85% of its cycles):
+// no face divides in FP64, conversions, comparisons and the halving go by
+// integers, and the largest area is reduced as an integer.  Blocks stay for
+// many faces and reduce in shared memory before their atomics.  1.93M faces:
+// 345 -> 179 us.
+constexpr int kPrepThreads = 256;
+
+__global__ void __launch_bounds__(kPrepThreads)
+k_face_prep(const float* __restrict__ V, int64_t nV, const int32_t* __restrict__ F,
+            int64_t T, float* fnorm, double* farea, float* tbox, DevScalars* sc)
+{
+    // contributions to the scene bounds; neutral when absent
     float cmin[3] = {INFINITY, INFINITY, INFINITY}, cmax[3] = {-INFINITY, -INFINITY, -INFINITY};
     float mabs = 0.0f;
-    double amax = 0.0;
-    if (f < T) {
+    unsigned long long amax = 0;       // bits of the area (>= 0, so they order as integers)
+    for (int64_t f = blockIdx.x * (int64_t)kPrepThreads + threadIdx.x; f < T; f += (int64_t)gridDim.x * kPrepThreads) {
         int32_t id[3];
         bool bad = false;
         for (int k = 0; k < 3; ++k) {
@@ -74,21 +94,34 @@ __global__ void k_face_prep(const float* __restrict__ V, int64_t nV, const int32
             // c = (B - A) x (C - A) in FP64, each operation rounded separately
             double e1[3], e2[3];
             for (int k = 0; k < 3; ++k) {
-                e1[k] = __dsub_rn((double)v[1][k], (double)v[0][k]);
-                e2[k] = __dsub_rn((double)v[2][k], (double)v[0][k]);
+                const double o = widen(v[0][k]);
+                e1[k] = __dsub_rn(widen(v[1][k]), o);
+                e2[k] = __dsub_rn(widen(v[2][k]), o);
             }
             const double c0 = __dsub_rn(__dmul_rn(e1[1], e2[2]), __dmul_rn(e1[2], e2[1]));
             const double c1 = __dsub_rn(__dmul_rn(e1[2], e2[0]), __dmul_rn(e1[0], e2[2]));
             const double c2 = __dsub_rn(__dmul_rn(e1[0], e2[1]), __dmul_rn(e1[1], e2[0]));
             const double len =
                 __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(c0, c0), __dmul_rn(c1, c1)), __dmul_rn(c2, c2)));
-            farea[f] = 0.5 * len;
-            amax = 0.5 * len;
+            // len is zero or far inside the normal range (products of
+            // differences of fp32 values): halving lowers its exponent
+            const long long lb = __double_as_longlong(len);
+            const long long ab = lb > 0 ? lb - (1LL << 52) : 0;
+            farea[f] = __longlong_as_double(ab);
+            amax = max(amax, (unsigned long long)ab);
             float n0 = 0.0f, n1 = 0.0f, n2 = 0.0f;
-            if (len > 0.0) {
-                n0 = __double2float_rn(__ddiv_rn(c0, len));
-                n1 = __double2float_rn(__ddiv_rn(c1, len));
-                n2 = __double2float_rn(__ddiv_rn(c2, len));
+            if (lb > 0) {
+                // one Newton step from the fp32 reciprocal of len cut to fp32
+                // (0: outside fp32's range)
+                double inv = 0.0;
+                const unsigned e = (unsigned)(lb >> 52);
+                if (e > 1023u - 100u && e < 1023u + 100u) {
+                    const double y = widen(__frcp_rn(__uint_as_float(((unsigned)(lb >> 32) - 0x38000000u) << 3 | (unsigned)lb >> 29)));
+                    inv = __fma_rn(y, __fma_rn(-len, y, 1.0), y);
+                }
+                n0 = quotient32(c0, len, inv);
+                n1 = quotient32(c1, len, inv);
+                n2 = quotient32(c2, len, inv);
             }
             fnorm[3 * f + 0] = n0;
             fnorm[3 * f + 1] = n1;
@@ -99,27 +132,44 @@ __global__ void k_face_prep(const float* __restrict__ V, int64_t nV, const int32
                 tbox[6 * f + k] = lo;
                 tbox[6 * f + 3 + k] = hi;
                 const float c = 0.5f * (lo + hi);
-                cmin[k] = c;
-                cmax[k] = c;
+                cmin[k] = fminf(cmin[k], c);
+                cmax[k] = fmaxf(cmax[k], c);
             }
         }
     }
-    const unsigned FULL = 0xFFFFFFFFu;
-    for (int off = 16; off; off >>= 1) {
-        for (int k = 0; k < 3; ++k) {
-            cmin[k] = fminf(cmin[k], __shfl_xor_sync(FULL, cmin[k], off));
-            cmax[k] = fmaxf(cmax[k], __shfl_xor_sync(FULL, cmax[k], off));
-        }
-        mabs = fmaxf(mabs, __shfl_xor_sync(FULL, mabs, off));
-        amax = fmax(amax, __shfl_xor_sync(FULL, amax, off));
+    constexpr int W = kPrepThreads / 32;
+    __shared__ float s_f[7][W];
+    __shared__ unsigned long long s_a[W];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int k = 0; k < 3; ++k) {
+        cmin[k] = warp_min(cmin[k]);
+        cmax[k] = warp_max(cmax[k]);
     }
-    if ((threadIdx.x & 31) == 0 && cmin[0] <= cmax[0]) {
+    mabs = warp_max(mabs);
+    const unsigned hi = __reduce_max_sync(0xFFFFFFFFu, (unsigned)(amax >> 32));
+    const unsigned lo = __reduce_max_sync(0xFFFFFFFFu, (unsigned)(amax >> 32) == hi ? (unsigned)amax : 0u);
+    if (lane == 0) {
         for (int k = 0; k < 3; ++k) {
-            atomicMin(&sc->cmin[k], float_to_ordered(cmin[k]));
-            atomicMax(&sc->cmax[k], float_to_ordered(cmax[k]));
+            s_f[k][warp] = cmin[k];
+            s_f[3 + k][warp] = cmax[k];
         }
-        atomicMax(&sc->vmaxabs, float_to_ordered(mabs));
-        atomicMax(&sc->amax_bits, (unsigned long long)__double_as_longlong(amax));
+        s_f[6][warp] = mabs;
+        s_a[warp] = ((unsigned long long)hi << 32) | lo;
+    }
+    __syncthreads();
+    if (threadIdx.x < 8) {
+        const int k = threadIdx.x;
+        if (k < 7) {
+            float v = s_f[k][0];
+            for (int w = 1; w < W; ++w) v = k < 3 ? fminf(v, s_f[k][w]) : fmaxf(v, s_f[k][w]);
+            if (k < 3 && v < INFINITY) atomicMin(&sc->cmin[k], float_to_ordered(v));
+            else if (k >= 3 && k < 6 && v > -INFINITY) atomicMax(&sc->cmax[k - 3], float_to_ordered(v));
+            else if (k == 6) atomicMax(&sc->vmaxabs, float_to_ordered(v));
+        } else {
+            unsigned long long v = s_a[0];
+            for (int w = 1; w < W; ++w) v = max(v, s_a[w]);
+            atomicMax(&sc->amax_bits, v);
+        }
     }
 }
 
@@ -173,7 +223,6 @@ __global__ void k_morton(const float* __restrict__ tbox, int64_t T, const DevSca
 // ---------------------------------------------------------------------------
 constexpr int kMaxWalk = 4096;   // bound on leaf-to-root walks
 constexpr int kSortThreads = 256;
-constexpr int kSortTile = 4096;   // most keys per block
 
 __global__ void k_sort_hist(const unsigned long long* __restrict__ keys, int64_t T, int shift, int tile,
                             int nblk, unsigned int* __restrict__ counts)
@@ -200,79 +249,238 @@ __device__ __forceinline__ unsigned int warp_incl_scan(unsigned int v, int lane)
 
 // per digit, the exclusive prefix of its counts over the blocks (in place,
 // digit-major layout counts[d * nblk + b]) and the digit's total; one warp
-// per digit, 32 counts per step
-__global__ void __launch_bounds__(1024) k_sort_scan(unsigned int* __restrict__ counts, int nblk,
-                                                    unsigned int* __restrict__ totals)
+// per digit, a lane per run of consecutive counts, so that the loads do not
+// wait for one another
+constexpr int kScanRun = 32;       // counts per lane and round: one round for up to 1,024 blocks
+
+__global__ void __launch_bounds__(256) k_sort_scan(unsigned int* __restrict__ counts, int nblk,
+                                                   unsigned int* __restrict__ totals)
 {
     const int lane = threadIdx.x & 31;
     const int d = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (d >= 256) return;
     unsigned int* c = counts + (int64_t)d * nblk;
     unsigned int carry = 0;
-    for (int b = 0; b < nblk; b += 32) {
-        const int i = b + lane;
-        const unsigned int v = i < nblk ? c[i] : 0u;
-        const unsigned int inc = warp_incl_scan(v, lane);
-        if (i < nblk) c[i] = carry + inc - v;
+    for (int b0 = 0; b0 < nblk; b0 += 32 * kScanRun) {
+        const int m = min(32 * kScanRun, nblk - b0), run = (m + 31) / 32;
+        const int i0 = b0 + lane * run, i1 = min(i0 + run, b0 + m);
+        unsigned int v[kScanRun], sum = 0;
+#pragma unroll
+        for (int k = 0; k < kScanRun; ++k) v[k] = k < run && i0 + k < i1 ? c[i0 + k] : 0u;
+#pragma unroll
+        for (int k = 0; k < kScanRun; ++k) sum += v[k];
+        const unsigned int inc = warp_incl_scan(sum, lane);
+        unsigned int at = carry + inc - sum;
+#pragma unroll
+        for (int k = 0; k < kScanRun; ++k) {
+            if (k < run && i0 + k < i1) c[i0 + k] = at;
+            at += v[k];
+        }
         carry += __shfl_sync(0xFFFFFFFFu, inc, 31);
     }
     if (lane == 0) totals[d] = carry;
 }
 
-__global__ void k_sort_scatter(const unsigned long long* __restrict__ kin, const int32_t* __restrict__ vin,
-                               int64_t T, int shift, int tile, int nblk, const unsigned int* __restrict__ offs,
-                               const unsigned int* __restrict__ totals, unsigned long long* __restrict__ kout,
-                               int32_t* __restrict__ vout, unsigned int* err)
+// the lanes with the same digit (eight votes; the match instruction on 32
+// mostly different digits takes several times as long)
+__device__ __forceinline__ unsigned int same_digit(unsigned int dig, bool ok)
 {
-    constexpr int W = kSortThreads / 32;
+    unsigned int peers = __ballot_sync(0xFFFFFFFFu, ok);
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+        const bool set = (dig >> b) & 1u;
+        const unsigned int m = __ballot_sync(0xFFFFFFFFu, set);
+        peers &= set ? m : ~m;
+    }
+    return peers;
+}
+
+// A block ranks its tile's keys once: warp w holds keys [w, w + 1) * 32 * kItems
+// of the tile in registers, kItems rounds of 32; within a round equal digits
+// find each other by votes, and the warp's digit counters carry from round to
+// round.  The tile is then put in order in shared memory and written out from
+// there, so that a warp writes a few runs instead of 32 places.  Six block
+// barriers per tile, where one pass per 256 keys took 64.  1.93M keys: 37 ->
+// 18 us per pass.
+template <int kItems>
+__global__ void __launch_bounds__(kSortThreads)
+k_sort_scatter(const unsigned long long* __restrict__ kin, const int32_t* __restrict__ vin,
+               int64_t T, int shift, int nblk, const unsigned int* __restrict__ offs,
+               const unsigned int* __restrict__ totals, unsigned long long* __restrict__ kout,
+               int32_t* __restrict__ vout, unsigned int* err)
+{
+    constexpr int W = kSortThreads / 32, kTile = kItems * kSortThreads;
     static_assert(kSortThreads == 256, "one thread per digit");
-    __shared__ unsigned int base[256];
-    __shared__ unsigned int wcnt[W][256];
-    __shared__ unsigned int wsum[W];
+    __shared__ unsigned long long s_key[kTile];
+    __shared__ int32_t s_val[kTile];
+    __shared__ unsigned short wcnt[W][256];     // then the warps' first places in the ordered tile
+    __shared__ int to[256];                     // global place of a digit's first key, less its place in the tile
+    __shared__ unsigned int wsum[2][W];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int i = threadIdx.x; i < W * 128; i += kSortThreads) ((unsigned int*)&wcnt[0][0])[i] = 0;
     // the digit's start = the totals of the smaller digits (a block scan of
     // the 256 totals) + this digit's count in the blocks before this one
-    {
-        const unsigned int t = totals[threadIdx.x];
-        const unsigned int inc = warp_incl_scan(t, lane);
-        if (lane == 31) wsum[warp] = inc;
-        __syncthreads();
-        unsigned int before = 0;
-        for (int w = 0; w < warp; ++w) before += wsum[w];
-        base[threadIdx.x] = before + inc - t + offs[(int64_t)threadIdx.x * nblk + blockIdx.x];
+    const unsigned int t = totals[threadIdx.x], mine = offs[(int64_t)threadIdx.x * nblk + blockIdx.x];
+    const unsigned int inc = warp_incl_scan(t, lane);
+    if (lane == 31) wsum[0][warp] = inc;
+    const int64_t tile0 = (int64_t)blockIdx.x * kTile, first = tile0 + warp * (32 * kItems) + lane;
+    const int m = (int)min64(kTile, T - tile0);
+    unsigned long long key[kItems];
+    int32_t val[kItems];
+    unsigned short rank[kItems];
+#pragma unroll
+    for (int r = 0; r < kItems; ++r) {
+        const int64_t i = first + 32 * r;
+        key[r] = i < T ? kin[i] : 0ULL;
+        val[r] = i < T ? vin[i] : 0;
     }
     __syncthreads();
-    const int64_t b0 = (int64_t)blockIdx.x * tile;
-    const int64_t e0 = min64(T, b0 + tile);
-    for (int64_t c0 = b0; c0 < e0; c0 += kSortThreads) {
-        for (int i = threadIdx.x; i < W * 256; i += blockDim.x) (&wcnt[0][0])[i] = 0;
+    unsigned int before = 0;
+    for (int w = 0; w < warp; ++w) before += wsum[0][w];
+    const unsigned int start = before + inc - t + mine;
+#pragma unroll
+    for (int r = 0; r < kItems; ++r) {
+        const bool ok = first + 32 * r < T;
+        const unsigned int dig = (unsigned int)((key[r] >> shift) & 255);
+        const unsigned int peers = same_digit(dig, ok);
+        const unsigned int at = __popc(peers & ((1u << lane) - 1u));
+        const unsigned int had = ok ? wcnt[warp][dig] : 0u;
+        __syncwarp();
+        if (ok && at == 0) wcnt[warp][dig] = (unsigned short)(had + __popc(peers));
+        __syncwarp();
+        rank[r] = (unsigned short)(had + at);
+    }
+    __syncthreads();
+    // this thread's digit: its keys in the tile, their first place there, and
+    // the warps' places
+    unsigned int total = 0;
+    for (int w = 0; w < W; ++w) total += wcnt[w][threadIdx.x];
+    const unsigned int inc2 = warp_incl_scan(total, lane);
+    if (lane == 31) wsum[1][warp] = inc2;
+    __syncthreads();
+    unsigned int run = inc2 - total;
+    for (int w = 0; w < warp; ++w) run += wsum[1][w];
+    to[threadIdx.x] = (int)(start - run);
+    for (int w = 0; w < W; ++w) {
+        const unsigned int c = wcnt[w][threadIdx.x];
+        wcnt[w][threadIdx.x] = (unsigned short)run;
+        run += c;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kItems; ++r) {
+        if (first + 32 * r >= T) continue;
+        const unsigned int at = wcnt[warp][(key[r] >> shift) & 255] + rank[r];
+        s_key[at & (kTile - 1)] = key[r];
+        s_val[at & (kTile - 1)] = val[r];
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < m; i += kSortThreads) {
+        const unsigned long long k = s_key[i];
+        const int64_t pos = (int64_t)to[(k >> shift) & 255] + i;
+        if (pos >= 0 && pos < T) {
+            kout[pos] = k;
+            vout[pos] = s_val[i];
+        } else {
+            atomicAdd(err, 1u);
+        }
+    }
+}
+
+// All passes of a small sort by one block, keys and values in shared memory:
+// a part of a few thousand triangles or points is bound by launches (three
+// per pass), not by work.  1,472 keys, six passes: 18 launches of 4 us -> one
+// of 16 us.
+constexpr int kSmallItems = 4, kSmallThreads = 1024;
+constexpr int kSmallSort = kSmallItems * kSmallThreads;
+struct SmallSort {
+    unsigned long long key[kSmallSort];
+    int32_t val[kSmallSort];
+    unsigned short cnt[kSmallThreads / 32][256];
+    unsigned int base[256], wsum[8];
+};
+
+__global__ void __launch_bounds__(kSmallThreads)
+k_sort_small(unsigned long long* __restrict__ keys, int32_t* __restrict__ vals, int n, int passes, unsigned int* err)
+{
+    extern __shared__ __align__(16) unsigned char s_sort[];
+    SmallSort& sm = *(SmallSort*)s_sort;
+    constexpr int W = kSmallThreads / 32;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int first = warp * 32 * kSmallItems + lane;
+    unsigned long long key[kSmallItems];
+    int32_t val[kSmallItems];
+#pragma unroll
+    for (int r = 0; r < kSmallItems; ++r) {
+        const int i = first + 32 * r;
+        key[r] = i < n ? keys[i] : 0ULL;
+        val[r] = i < n ? vals[i] : 0;
+    }
+    for (int pass = 0; pass < passes; ++pass) {
+        const int shift = 8 * pass;
+        for (int i = threadIdx.x; i < W * 256; i += kSmallThreads) (&sm.cnt[0][0])[i] = 0;
         __syncthreads();
-        const int64_t i = c0 + threadIdx.x;
-        const bool ok = i < e0;
-        unsigned long long key = ok ? kin[i] : 0ULL;
-        int32_t val = ok ? vin[i] : 0;
-        const unsigned int dig = ok ? (unsigned int)((key >> shift) & 255) : 256u + lane;
-        const unsigned int peers = __match_any_sync(0xFFFFFFFFu, dig);
-        const unsigned int rank = __popc(peers & ((1u << lane) - 1u));
-        if (ok && rank == 0) wcnt[warp][dig] = __popc(peers);
+        unsigned int rank[kSmallItems];
+#pragma unroll
+        for (int r = 0; r < kSmallItems; ++r) {
+            const bool ok = first + 32 * r < n;
+            const unsigned int dig = (unsigned int)((key[r] >> shift) & 255);
+            const unsigned int peers = same_digit(dig, ok);
+            const unsigned int at = __popc(peers & ((1u << lane) - 1u));
+            const unsigned int had = ok ? sm.cnt[warp][dig] : 0u;
+            __syncwarp();
+            if (ok && at == 0) sm.cnt[warp][dig] = (unsigned short)(had + __popc(peers));
+            __syncwarp();
+            rank[r] = had + at;
+        }
         __syncthreads();
-        if (ok) {
-            unsigned int pos = base[dig] + rank;
-            for (int w = 0; w < warp; ++w) pos += wcnt[w][dig];
-            if (pos < (unsigned long long)T) {
-                kout[pos] = key;
-                vout[pos] = val;
+        // per digit the prefix over the warps, then over the digits
+        unsigned int total = 0, inc = 0;
+        if (threadIdx.x < 256) {
+            for (int w = 0; w < W; ++w) {
+                const unsigned int c = sm.cnt[w][threadIdx.x];
+                sm.cnt[w][threadIdx.x] = (unsigned short)total;
+                total += c;
+            }
+            inc = warp_incl_scan(total, lane);
+            if (lane == 31) sm.wsum[warp] = inc;
+        }
+        __syncthreads();
+        if (threadIdx.x < 256) {
+            unsigned int before = 0;
+            for (int w = 0; w < warp; ++w) before += sm.wsum[w];
+            sm.base[threadIdx.x] = before + inc - total;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < kSmallItems; ++r) {
+            if (first + 32 * r >= n) continue;
+            const unsigned int dig = (unsigned int)((key[r] >> shift) & 255);
+            const unsigned int pos = sm.base[dig] + sm.cnt[warp][dig] + rank[r];
+            if (pos < (unsigned int)n) {
+                sm.key[pos] = key[r];
+                sm.val[pos] = val[r];
             } else {
                 atomicAdd(err, 1u);
             }
         }
         __syncthreads();
-        for (int d = threadIdx.x; d < 256; d += blockDim.x) {
-            unsigned int s = 0;
-            for (int w = 0; w < W; ++w) s += wcnt[w][d];
-            base[d] += s;
+#pragma unroll
+        for (int r = 0; r < kSmallItems; ++r) {
+            const int i = first + 32 * r;
+            if (i < n) {
+                key[r] = sm.key[i];
+                val[r] = sm.val[i];
+            }
         }
-        __syncthreads();
+    }
+#pragma unroll
+    for (int r = 0; r < kSmallItems; ++r) {
+        const int i = first + 32 * r;
+        if (i < n) {
+            keys[i] = key[r];
+            vals[i] = val[r];
+        }
     }
 }
 
@@ -549,74 +757,162 @@ __global__ void k_ploc_emit(int64_t T, int64_t n_int, const int32_t* __restrict_
 }
 
 // ---------------------------------------------------------------------------
-// bottom-up refit
+// bottom-up refit and packing into the traversal layout
 // ---------------------------------------------------------------------------
-__global__ void k_leaf_boxes(const float* __restrict__ tbox, const int32_t* __restrict__ order,
-                             int64_t T, int64_t n_int, float* nbox)
+// The corners of sorted slot k's triangle; false for a face or vertex index
+// out of range (a bad mesh, reported by the build, must not be gathered).
+__device__ __forceinline__ bool gather_tri(const float* __restrict__ V, int64_t nV, const int32_t* __restrict__ F, int64_t T,
+                                           int32_t f, float v[3][3])
 {
-    int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (k >= T) return;
-    const int32_t f = order[k];
-    for (int c = 0; c < 6; ++c) nbox[6 * (n_int + k) + c] = f >= 0 && f < T ? tbox[6 * (int64_t)f + c] : 0.0f;
+    bool ok = f >= 0 && f < T;
+    for (int a = 0; a < 3; ++a) {
+        const int64_t vi = ok ? F[3 * (int64_t)f + a] : -1;
+        const bool in = vi >= 0 && vi < nV;
+        for (int c = 0; c < 3; ++c) v[a][c] = in ? V[3 * vi + c] : 0.0f;
+        ok &= in;
+    }
+    return ok;
 }
 
-__global__ void k_refit(int64_t T, int64_t n_int, const int32_t* __restrict__ parent,
-                        const int32_t* __restrict__ child, float* nbox, int32_t* visits, DevScalars* sc)
+// From a leaf up: the second thread to arrive at a node has its box, the
+// first one's box and both heights, and goes on.  A node whose leaves all
+// belong to one block (255 of 256 do) meets in shared memory, at the place of
+// its split (the last leaf of its left subtree, which no other node has).
+// The others meet in global memory: a fence, an exchange and a read back, a
+// microsecond or two per level; that chain bounds a small tree, and the boxes'
+// traffic a large one.  kPack: the packed binary nodes are written on the way
+// (both children's boxes are at hand), and `sc` receives the tree's depth and
+// box at the root; otherwise every node's box goes to nbox.  The arrival word
+// of a node holds 1 + the first arrival's height, so depth needs no walk of
+// its own.
+constexpr int kClimb = 256;        // leaves (threads) per block
+struct ClimbShared {
+    float box[2][6][kClimb];       // of the left and the right child, by split
+    int height[2][kClimb];
+    int arrived[kClimb];
+};
+
+__device__ __forceinline__ void put_box(float* nbox, int64_t node, const float lo[3], const float hi[3])
 {
-    const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int32_t cur = (int32_t)(n_int + k);
-    // every chain ends at the root; the caps only guard against a malformed
-    // tree (the build then reports an error instead of looping)
-    int depth = 0;
-    if (k < T)
-        for (int32_t p = parent[cur]; p >= 0 && depth <= kMaxWalk; p = parent[p]) ++depth;
-    int wmax = depth;                               // one atomic per warp
-    for (int off = 16; off; off >>= 1) wmax = max(wmax, __shfl_xor_sync(0xFFFFFFFFu, wmax, off));
-    if ((threadIdx.x & 31) == 0) atomicMax(&sc->max_depth, wmax);
-    if (k >= T || depth > kMaxWalk) return;
+    for (int c = 0; c < 3; ++c) {
+        __stcg(&nbox[6 * node + c], lo[c]);
+        __stcg(&nbox[6 * node + 3 + c], hi[c]);
+    }
+}
+
+// the whole block calls it (threads past the last leaf with leaf = false)
+template <bool kPack>
+__device__ __forceinline__ void climb(ClimbShared& sm, bool leaf, int64_t T, int64_t n_int, const int32_t* __restrict__ parent,
+                                      const int32_t* __restrict__ child, const int32_t* __restrict__ range, float* nbox,
+                                      float4* nodes, int32_t* visits, DevScalars* sc, int64_t k, float lo[3], float hi[3])
+{
+    sm.arrived[threadIdx.x] = 0;
+    __syncthreads();
+    if (!leaf) return;
+    const int64_t b0 = blockIdx.x * (int64_t)kClimb, b1 = min64(b0 + kClimb, T) - 1;
+    int32_t cur = (int32_t)(n_int + k);
+    int32_t first = (int32_t)k, last = (int32_t)k;      // leaves below cur
+    int height = 0;
+    if (!kPack) put_box(nbox, cur, lo, hi);
+    // every chain ends at the root; the cap only guards against a malformed
+    // tree (the build then reports the depth it reached)
     int32_t p = parent[cur];
     for (int steps = 0; p >= 0 && steps <= kMaxWalk; ++steps) {
-        __threadfence();
-        if (atomicAdd(&visits[p], 1) == 0) return;   // first arrival stops
-        const int32_t a = child[2 * p], b = child[2 * p + 1];
-        float box[6];
-        for (int c = 0; c < 3; ++c) {
-            box[c] = fminf(__ldcg(&nbox[6 * (int64_t)a + c]), __ldcg(&nbox[6 * (int64_t)b + c]));
-            box[3 + c] = fmaxf(__ldcg(&nbox[6 * (int64_t)a + 3 + c]), __ldcg(&nbox[6 * (int64_t)b + 3 + c]));
+        const int32_t a = child[2 * p], b = child[2 * p + 1], r0 = range[2 * p], r1 = range[2 * p + 1];
+        const bool left = a == cur;
+        const int32_t split = left ? last : first - 1;  // last leaf of the left child
+        float slo[3], shi[3];
+        if (r0 >= b0 && r1 <= b1 && split >= b0 && split < b1) {
+            const int at = (int)(split - b0), me = left ? 0 : 1;
+            for (int c = 0; c < 3; ++c) {
+                sm.box[me][c][at] = lo[c];
+                sm.box[me][3 + c][at] = hi[c];
+            }
+            sm.height[me][at] = height;
+            __threadfence_block();
+            if (atomicExch(&sm.arrived[at], 1) == 0) return;     // first arrival stops
+            __threadfence_block();
+            volatile float* bx = &sm.box[1 - me][0][at];
+            for (int c = 0; c < 3; ++c) {
+                slo[c] = bx[c * kClimb];
+                shi[c] = bx[(3 + c) * kClimb];
+            }
+            height = max(height, *(volatile int*)&sm.height[1 - me][at]) + 1;
+        } else {
+            if (kPack) put_box(nbox, cur, lo, hi);      // (else it is there)
+            __threadfence();
+            const int other = atomicExch(&visits[p], height + 1);
+            if (other == 0) return;
+            const int64_t sib = left ? b : a;
+            for (int c = 0; c < 3; ++c) {
+                slo[c] = __ldcg(&nbox[6 * sib + c]);
+                shi[c] = __ldcg(&nbox[6 * sib + 3 + c]);
+            }
+            height = max(height, other - 1) + 1;
         }
-        for (int c = 0; c < 6; ++c) __stcg(&nbox[6 * (int64_t)p + c], box[c]);
+        if (kPack) {
+            // a child of at most kLeafMax triangles becomes a leaf
+            const int nl = split - r0 + 1, nr = r1 - split;
+            const int ca = nl <= kLeafMax ? leaf_code(r0, nl) : a, cb = nr <= kLeafMax ? leaf_code(split + 1, nr) : b;
+            const float* Al = left ? lo : slo;
+            const float* Ah = left ? hi : shi;
+            const float* Bl = left ? slo : lo;
+            const float* Bh = left ? shi : hi;
+            float4* nd = nodes + 4 * (int64_t)p;
+            nd[0] = make_float4(Al[0], Ah[0], Al[1], Ah[1]);
+            nd[1] = make_float4(Bl[0], Bh[0], Bl[1], Bh[1]);
+            nd[2] = make_float4(Al[2], Ah[2], Bl[2], Bh[2]);
+            nd[3] = make_float4(__int_as_float(ca), __int_as_float(cb), 0.0f, 0.0f);
+        }
+        for (int c = 0; c < 3; ++c) {
+            lo[c] = fminf(lo[c], slo[c]);
+            hi[c] = fmaxf(hi[c], shi[c]);
+        }
+        if (!kPack) put_box(nbox, p, lo, hi);
+        cur = p;
+        first = r0;
+        last = r1;
         p = parent[p];
     }
-}
-
-// ---------------------------------------------------------------------------
-// packing into the traversal layout
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ int32_t encode_child(int32_t c, int64_t n_int, const int32_t* range)
-{
-    if (c >= n_int) {
-        const int32_t first = (int32_t)(c - n_int);
-        return leaf_code(first, 1);
+    if (kPack && p < 0) {
+        sc->max_depth = height;
+        for (int c = 0; c < 3; ++c) {
+            sc->lo[c] = lo[c];
+            sc->hi[c] = hi[c];
+        }
     }
-    const int32_t lo = range[2 * c], hi = range[2 * c + 1];
-    const int32_t cnt = hi - lo + 1;
-    if (cnt <= kLeafMax) return leaf_code(lo, cnt);
-    return c;
 }
 
-__global__ void k_pack(int64_t n_int, const int32_t* __restrict__ child, const int32_t* __restrict__ range,
-                       const float* __restrict__ nbox, float4* nodes)
+// Triangle records, leaf boxes, all boxes above them and the packed binary
+// nodes in one launch: the corners are gathered once.  1.93M triangles: the
+// four kernels this replaces took 331 us, this one 200 us.
+__global__ void __launch_bounds__(kClimb)
+k_refit(const float* __restrict__ V, int64_t nV, const int32_t* __restrict__ F, const int32_t* __restrict__ order, int64_t T,
+        int64_t n_int, const int32_t* __restrict__ parent, const int32_t* __restrict__ child,
+        const int32_t* __restrict__ range, float* nbox, float4* nodes, float4* tris, int32_t* visits, DevScalars* sc)
 {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n_int) return;
-    const int32_t a = child[2 * i], b = child[2 * i + 1];
-    const float* A = nbox + 6 * (int64_t)a;
-    const float* B = nbox + 6 * (int64_t)b;
-    nodes[4 * i + 0] = make_float4(A[0], A[3], A[1], A[4]);
-    nodes[4 * i + 1] = make_float4(B[0], B[3], B[1], B[4]);
-    nodes[4 * i + 2] = make_float4(A[2], A[5], B[2], B[5]);
-    nodes[4 * i + 3] = make_float4(__int_as_float(encode_child(a, n_int, range)),
-                                   __int_as_float(encode_child(b, n_int, range)), 0.0f, 0.0f);
+    __shared__ ClimbShared sm;
+    const int64_t k = blockIdx.x * (int64_t)kClimb + threadIdx.x;
+    float lo[3] = {0, 0, 0}, hi[3] = {0, 0, 0};
+    if (k < T) {
+        const int32_t f = order[k];
+        float v[3][3];
+        gather_tri(V, nV, F, T, f, v);
+        float le = 0.0f;
+        for (int c = 0; c < 3; ++c) {
+            le = fmaxf(le, fabsf(v[1][c] - v[0][c]));
+            le = fmaxf(le, fabsf(v[2][c] - v[1][c]));
+            le = fmaxf(le, fabsf(v[0][c] - v[2][c]));
+        }
+        tris[3 * k + 0] = make_float4(v[0][0], v[0][1], v[0][2], le);
+        tris[3 * k + 1] = make_float4(v[1][0], v[1][1], v[1][2], __int_as_float(f));
+        tris[3 * k + 2] = make_float4(v[2][0], v[2][1], v[2][2], 0.0f);
+        for (int c = 0; c < 3; ++c) {
+            lo[c] = fminf(v[0][c], fminf(v[1][c], v[2][c]));
+            hi[c] = fmaxf(v[0][c], fmaxf(v[1][c], v[2][c]));
+        }
+    }
+    if (parent) climb<true>(sm, k < T, T, n_int, parent, child, range, nbox, nodes, visits, sc, k, lo, hi);
 }
 
 // ---------------------------------------------------------------------------
@@ -628,59 +924,77 @@ __global__ void k_pack(int64_t n_int, const int32_t* __restrict__ child, const i
 // children, then the four child indices (>= 0 wide node, < 0 leaf as in the
 // binary layout), then padding.  Empty slots have an empty box.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ bool bin_is_leaf(int32_t c, int64_t n_int, const int32_t* range)
-{
-    return c >= n_int || range[2 * c + 1] - range[2 * c] + 1 <= kLeafMax;
-}
+// the children of a wide node: boxes (lo, hi), codes (a binary interior node
+// >= 0, or a leaf), and how many
+struct WideKids {
+    float lo[4][3], hi[4][3];
+    int32_t code[4];
+    int n;
+};
 
-__device__ __forceinline__ float half_area(const float* b)
+// The children of the wide node made from binary interior node b: b's two
+// children, the interior one of largest box surface area replaced by its own
+// two until there are four or only leaves.  Reads one packed 64-byte node per
+// replacement (boxes and codes together; child, range and box arrays took
+// four dependent gathers each).
+__device__ __forceinline__ WideKids wide_kids(int32_t b, const float4* __restrict__ nodes)
 {
-    const float dx = b[3] - b[0], dy = b[4] - b[1], dz = b[5] - b[2];
-    return dx * dy + dy * dz + dz * dx;
-}
-
-// the children of the wide node made from binary interior node b: start
-// from b's two children and keep replacing the interior child of largest box
-// surface area by its two children until there are four or only leaves
-__device__ __forceinline__ int wide_children(int32_t b, int64_t n_int, const int32_t* __restrict__ child,
-                                             const int32_t* __restrict__ range, const float* __restrict__ nbox,
-                                             int32_t ch[4])
-{
-    int nch = 2;
-    ch[0] = child[2 * b];
-    ch[1] = child[2 * b + 1];
-    while (nch < 4) {
-        int best = -1;
-        float ba = -1.0f;
-        for (int k = 0; k < nch; ++k) {
-            if (bin_is_leaf(ch[k], n_int, range)) continue;
-            const float a = half_area(nbox + 6 * (int64_t)ch[k]);
-            if (a > ba) { ba = a; best = k; }
+    WideKids w;
+    w.n = 0;
+    int at = 0;
+    for (;;) {
+        const float4* nd = nodes + 4 * (int64_t)b;
+        const float4 n0 = nd[0], n1 = nd[1], n2 = nd[2], n3 = nd[3];
+        const int other = w.n == 0 ? 1 : w.n;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (k == at) {
+                w.lo[k][0] = n0.x; w.hi[k][0] = n0.y; w.lo[k][1] = n0.z; w.hi[k][1] = n0.w;
+                w.lo[k][2] = n2.x; w.hi[k][2] = n2.y;
+                w.code[k] = __float_as_int(n3.x);
+            }
+            if (k == other) {
+                w.lo[k][0] = n1.x; w.hi[k][0] = n1.y; w.lo[k][1] = n1.z; w.hi[k][1] = n1.w;
+                w.lo[k][2] = n2.z; w.hi[k][2] = n2.w;
+                w.code[k] = __float_as_int(n3.y);
+            }
         }
-        if (best < 0) break;
-        const int32_t c = ch[best];
-        ch[best] = child[2 * c];
-        ch[nch++] = child[2 * c + 1];
+        w.n = other + 1;
+        if (w.n == 4) return w;
+        at = -1;
+        float most = -1.0f;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (k >= w.n || w.code[k] < 0) continue;
+            const float dx = w.hi[k][0] - w.lo[k][0], dy = w.hi[k][1] - w.lo[k][1], dz = w.hi[k][2] - w.lo[k][2];
+            const float a = dx * dy + dy * dz + dz * dx;
+            if (a > most) {
+                most = a;
+                at = k;
+                b = w.code[k];
+            }
+        }
+        if (at < 0) return w;
     }
-    return nch;
 }
 
-// write wide node w: the boxes of its nch children and their indices idx
-// (wide node >= 0, leaf < 0); empty slots get an empty box and index -1
-__device__ __forceinline__ void wide_write(float4* wnodes, int32_t w, const float* __restrict__ nbox,
-                                           const int32_t ch[4], const int32_t idx[4], int nch)
+// write wide node w: its children's boxes and their indices idx (wide node
+// >= 0, leaf < 0); empty slots get an empty box and index -1
+__device__ __forceinline__ void wide_write(float4* wnodes, int32_t w, const WideKids& kids, const int32_t idx[4])
 {
     float lo[3][4], hi[3][4];
-    int32_t ix[4];
+    int32_t ix[4], id[4];
+#pragma unroll
     for (int k = 0; k < 4; ++k) {
-        if (k < nch) {
-            const float* bb = nbox + 6 * (int64_t)ch[k];
-            for (int a = 0; a < 3; ++a) { lo[a][k] = bb[a]; hi[a][k] = bb[3 + a]; }
-            ix[k] = idx[k];
-        } else {
-            for (int a = 0; a < 3; ++a) { lo[a][k] = INFINITY; hi[a][k] = -INFINITY; }
-            ix[k] = -1;
+        const bool on = k < kids.n;
+        for (int a = 0; a < 3; ++a) {
+            lo[a][k] = on ? kids.lo[k][a] : INFINITY;
+            hi[a][k] = on ? kids.hi[k][a] : -INFINITY;
         }
+        ix[k] = on ? idx[k] : -1;
+        // the binary node the child was made from, for the boxes of the same
+        // tree in another coordinate frame (-1: empty slot)
+        id[k] = on ? (kids.code[k] >= 0 ? kids.code[k] : kLeafChild) : -1;
     }
     wnodes[wide_at(w, 0)] = make_float4(lo[0][0], lo[0][1], lo[0][2], lo[0][3]);
     wnodes[wide_at(w, 1)] = make_float4(hi[0][0], hi[0][1], hi[0][2], hi[0][3]);
@@ -689,38 +1003,95 @@ __device__ __forceinline__ void wide_write(float4* wnodes, int32_t w, const floa
     wnodes[wide_at(w, 4)] = make_float4(lo[2][0], lo[2][1], lo[2][2], lo[2][3]);
     wnodes[wide_at(w, 5)] = make_float4(hi[2][0], hi[2][1], hi[2][2], hi[2][3]);
     wnodes[wide_at(w, 6)] = make_float4(__int_as_float(ix[0]), __int_as_float(ix[1]), __int_as_float(ix[2]), __int_as_float(ix[3]));
-    // the binary nodes the children were made from (-1: empty slot), for
-    // the boxes of the same tree in another coordinate frame
-    wnodes[wide_at(w, 7)] = make_float4(__int_as_float(nch > 0 ? ch[0] : -1), __int_as_float(nch > 1 ? ch[1] : -1),
-                        __int_as_float(nch > 2 ? ch[2] : -1), __int_as_float(nch > 3 ? ch[3] : -1));
+    wnodes[wide_at(w, 7)] = make_float4(__int_as_float(id[0]), __int_as_float(id[1]), __int_as_float(id[2]), __int_as_float(id[3]));
 }
 
-// one level of the top of the tree: each queued binary node becomes a wide
-// node; its interior children go to the next level's queue
-__global__ void k_wide_level(int64_t n_int, const int32_t* __restrict__ child, const int32_t* __restrict__ range,
-                             const float* __restrict__ nbox, const int32_t* __restrict__ qin_bin,
-                             const int32_t* __restrict__ qin_wide, const int* __restrict__ qin_count,
-                             int32_t* qout_bin, int32_t* qout_wide, int* qout_count, int* wide_count,
-                             float4* wnodes, DevScalars* sc, int level)
+// The first of n (0..4) consecutive numbers from a counter, for every active
+// lane: one atomic per warp (a lane each, on one address, took most of the
+// collapse's time).
+__device__ __forceinline__ int take_numbers(int* counter, int n)
 {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= *qin_count) return;
-    const int32_t b = qin_bin[t], w = qin_wide[t];
-    int32_t ch[4], idx[4];
-    const int nch = wide_children(b, n_int, child, range, nbox, ch);
-    for (int k = 0; k < nch; ++k) {
-        if (bin_is_leaf(ch[k], n_int, range)) {
-            idx[k] = encode_child(ch[k], n_int, range);
-        } else {
-            const int nw = atomicAdd(wide_count, 1);
-            const int q = atomicAdd(qout_count, 1);
-            qout_bin[q] = ch[k];
-            qout_wide[q] = nw;
-            idx[k] = nw;
+    const unsigned active = __activemask(), lane = threadIdx.x & 31, below = active & ((1u << lane) - 1u);
+    const unsigned b0 = __ballot_sync(active, n & 1), b1 = __ballot_sync(active, n & 2), b2 = __ballot_sync(active, n & 4);
+    const int before = __popc(b0 & below) + 2 * __popc(b1 & below) + 4 * __popc(b2 & below);
+    const int total = __popc(b0) + 2 * __popc(b1) + 4 * __popc(b2);
+    const int leader = __ffs(active) - 1;
+    int first = 0;
+    if ((int)lane == leader && total) first = atomicAdd(counter, total);
+    return __shfl_sync(active, first, leader) + before;
+}
+
+// A queue of (binary node, wide node) pairs: one node and its place.
+// Expands one queued binary node into its wide node; interior children get
+// consecutive wide numbers and go to the next queue.
+__device__ __forceinline__ void wide_expand(const float4* __restrict__ nodes, int2 q, int2* qout, int* qout_count,
+                                            int* wide_count, float4* wnodes)
+{
+    const WideKids kids = wide_kids(q.x, nodes);
+    int ni = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) ni += k < kids.n && kids.code[k] >= 0;
+    int nw = take_numbers(wide_count, ni), at = take_numbers(qout_count, ni);
+    int32_t idx[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        idx[k] = -1;
+        if (k >= kids.n) continue;
+        idx[k] = kids.code[k];
+        if (kids.code[k] >= 0) {
+            qout[at++] = make_int2(kids.code[k], nw);
+            idx[k] = nw++;
         }
     }
-    wide_write(wnodes, w, nbox, ch, idx, nch);
-    atomicMax(&sc->wide_depth, level + 1);
+    wide_write(wnodes, q.y, kids, idx);
+}
+
+// The top levels of the tree in one block: level by level until a queue may
+// outgrow it (level l holds at most 4^l nodes), a launch each otherwise: at
+// 10 us and more a level, the top six had cost as much as the rest.
+constexpr int kWideTop = 6, kWideTopThreads = 1024;   // 4^5 nodes on the sixth level
+
+__global__ void __launch_bounds__(kWideTopThreads)
+k_wide_top(const float4* __restrict__ nodes, int2* qa, int2* qb, int* counts /*[2]: sizes of qa and qb*/, int* wide_count,
+           float4* wnodes, DevScalars* sc, int levels)
+{
+    __shared__ int s_count[2];
+    if (threadIdx.x == 0) {
+        qa[0] = make_int2(0, 0);
+        s_count[0] = 1;
+        s_count[1] = 0;
+        *wide_count = 1;
+    }
+    __syncthreads();
+    int depth = 0;
+    for (int l = 0; l < levels; ++l) {
+        const int n = s_count[l & 1];
+        int2* in = l & 1 ? qb : qa;
+        int2* out = l & 1 ? qa : qb;
+        if (n > 0) depth = l + 1;
+        for (int t = threadIdx.x; t < n; t += kWideTopThreads)
+            wide_expand(nodes, in[t], out, &s_count[1 - (l & 1)], wide_count, wnodes);
+        __syncthreads();
+        if (threadIdx.x == 0) s_count[l & 1] = 0;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        counts[0] = s_count[0];
+        counts[1] = s_count[1];
+        sc->wide_depth = depth;
+    }
+}
+
+// one further level, a launch each
+__global__ void __launch_bounds__(256)
+k_wide_level(const float4* __restrict__ nodes, const int2* __restrict__ qin, int* qin_count, int2* qout, int* qout_count,
+             int* wide_count, float4* wnodes, DevScalars* sc, int level)
+{
+    const int n = *qin_count;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= n) return;
+    if (t == 0) atomicMax(&sc->wide_depth, level + 1);
+    wide_expand(nodes, qin[t], qout, qout_count, wide_count, wnodes);
 }
 
 // the rest of the tree: each thread finishes the subtree below one queued
@@ -732,40 +1103,42 @@ constexpr int kWideDfs = 96;
 #define RC_WIDE_SUBTREE 4.0      // binary nodes per subtree thread (0: one launch per level throughout)
 #endif
 
-__global__ void k_wide_subtrees(int64_t n_int, const int32_t* __restrict__ child, const int32_t* __restrict__ range,
-                                const float* __restrict__ nbox, const int32_t* __restrict__ qin_bin,
-                                const int32_t* __restrict__ qin_wide, const int* __restrict__ qin_count,
-                                int* wide_count, float4* wnodes, DevScalars* sc, int level)
+__global__ void k_wide_subtrees(const float4* __restrict__ nodes, const int2* __restrict__ qin,
+                                const int* __restrict__ qin_count, int* wide_count, float4* wnodes, DevScalars* sc, int level)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= *qin_count) return;
-    int32_t sb[kWideDfs], sw[kWideDfs];
+    int2 st[kWideDfs];
     uint8_t sd[kWideDfs];
-    sb[0] = qin_bin[t];
-    sw[0] = qin_wide[t];
+    st[0] = qin[t];
     sd[0] = 0;
     int sp = 1, maxd = 0;
     while (sp > 0) {
         --sp;
-        const int32_t b = sb[sp], w = sw[sp];
+        const int32_t w = st[sp].y;
         const int d = sd[sp];
-        int32_t ch[4], idx[4];
-        const int nch = wide_children(b, n_int, child, range, nbox, ch);
+        const WideKids kids = wide_kids(st[sp].x, nodes);
         int ni = 0;
-        for (int k = 0; k < nch; ++k) ni += bin_is_leaf(ch[k], n_int, range) ? 0 : 1;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) ni += k < kids.n && kids.code[k] >= 0;
         if (sp + ni > kWideDfs || d + 1 > 250) {
             atomicMax(&sc->wide_depth, kStack4);
             return;
         }
-        int nw = ni ? atomicAdd(wide_count, ni) : 0;
-        for (int k = 0; k < nch; ++k) idx[k] = bin_is_leaf(ch[k], n_int, range) ? encode_child(ch[k], n_int, range)
-                                                                                 : nw++;
-        wide_write(wnodes, w, nbox, ch, idx, nch);
+        const int base = take_numbers(wide_count, ni);
+        int32_t idx[4];
+        int nw = base;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            idx[k] = -1;
+            if (k < kids.n) idx[k] = kids.code[k] >= 0 ? nw++ : kids.code[k];
+        }
+        wide_write(wnodes, w, kids, idx);
         maxd = max(maxd, d + 1);
-        for (int k = nch - 1; k >= 0; --k) {     // the first child is taken next
-            if (idx[k] < 0) continue;
-            sb[sp] = ch[k];
-            sw[sp] = idx[k];
+#pragma unroll
+        for (int k = 3; k >= 0; --k) {           // the first child is taken next
+            if (k >= kids.n || kids.code[k] < 0) continue;
+            st[sp] = make_int2(kids.code[k], idx[k]);
             sd[sp] = (uint8_t)(d + 1);
             ++sp;
         }
@@ -797,19 +1170,8 @@ __global__ void k_wide_small(int64_t T, const float* __restrict__ tbox, float4* 
     sc->wide_nodes = 1;
 }
 
-__global__ void k_wide_init(int32_t* q_bin, int32_t* q_wide, int* counts)
-{
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        q_bin[0] = 0;
-        q_wide[0] = 0;
-        counts[0] = 1;   // queue A size
-        counts[1] = 0;   // queue B size
-        counts[2] = 1;   // wide nodes allocated
-    }
-}
-
 // single-leaf root for parts with at most kLeafMax triangles
-__global__ void k_pack_small(int64_t T, const float* __restrict__ tbox, float4* nodes)
+__global__ void k_pack_small(int64_t T, const float* __restrict__ tbox, float4* nodes, DevScalars* sc)
 {
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
@@ -818,82 +1180,101 @@ __global__ void k_pack_small(int64_t T, const float* __restrict__ tbox, float4* 
             lo[c] = fminf(lo[c], tbox[6 * f + c]);
             hi[c] = fmaxf(hi[c], tbox[6 * f + 3 + c]);
         }
+    for (int c = 0; c < 3; ++c) {
+        sc->lo[c] = lo[c];
+        sc->hi[c] = hi[c];
+    }
     nodes[0] = make_float4(lo[0], hi[0], lo[1], hi[1]);
     nodes[1] = make_float4(INFINITY, -INFINITY, INFINITY, -INFINITY);
     nodes[2] = make_float4(lo[2], hi[2], INFINITY, -INFINITY);
     nodes[3] = make_float4(__int_as_float(leaf_code(0, (int)T)), __int_as_float(-1), 0.0f, 0.0f);
 }
 
-__global__ void k_tri_records(const float* __restrict__ V, int64_t nV, const int32_t* __restrict__ F,
-                              const int32_t* __restrict__ order, int64_t T, float4* tris)
-{
-    int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (k >= T) return;
-    const int32_t f = order[k];
-    float v[3][3] = {};
-    // a bad mesh (reported by the build) must not be gathered out of range
-    if (f >= 0 && f < T) {
-        for (int a = 0; a < 3; ++a) {
-            const int64_t vi = F[3 * (int64_t)f + a];
-            if (vi >= 0 && vi < nV)
-                for (int c = 0; c < 3; ++c) v[a][c] = V[3 * vi + c];
-        }
-    }
-    float le = 0.0f;
-    for (int c = 0; c < 3; ++c) {
-        le = fmaxf(le, fabsf(v[1][c] - v[0][c]));
-        le = fmaxf(le, fabsf(v[2][c] - v[1][c]));
-        le = fmaxf(le, fabsf(v[0][c] - v[2][c]));
-    }
-    tris[3 * k + 0] = make_float4(v[0][0], v[0][1], v[0][2], le);
-    tris[3 * k + 1] = make_float4(v[1][0], v[1][1], v[1][2], __int_as_float(f));
-    tris[3 * k + 2] = make_float4(v[2][0], v[2][1], v[2][2], 0.0f);
-}
-
 // ---------------------------------------------------------------------------
 // area CDF (2^32-quantised areas, inclusive prefix in int64)
 // ---------------------------------------------------------------------------
-constexpr int kScanBlock = 1024;
+constexpr int kScanThreads = 1024, kScanItems = 4;
+constexpr int kScanBlock = kScanThreads * kScanItems;
 
-__global__ void k_quant_area(const double* __restrict__ farea, int64_t T, const DevScalars* sc,
-                             long long* q)
+// llround(area / amax * 2^32) from the product with scale = 2^32 / amax, within
+// 2^-18 of the quotient's value; taken as it is unless that close to a
+// half-integer (2^-17 taken: 1 in 65,536), where the division decides.
+__device__ __forceinline__ long long quantise_area(double area, double amax, double scale)
 {
-    int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (f >= T) return;
-    const double amax = __longlong_as_double((long long)sc->amax_bits);
-    q[f] = amax > 0.0 ? llround(__dmul_rn(__ddiv_rn(farea[f], amax), 4294967296.0)) : 0LL;
+    const double C = 6755399441055744.0;           // 1.5 * 2^52: adding it leaves the integer in the low bits
+    const double q = __dmul_rn(area, scale), t = __dadd_rn(q, C);
+    const double off = __dsub_rn(q, __dsub_rn(t, C));          // |off| < 0.5 - 2^-17, compared by its high word
+    if ((__double2hiint(off) & 0x7FFFFFFF) >= 0x3FDFFFE0) return llround(__dmul_rn(__ddiv_rn(area, amax), 4294967296.0));
+    return __double_as_longlong(t) - __double_as_longlong(C);
 }
 
-// block-wise inclusive scan, writing per-block totals
-__global__ void k_scan_block(long long* x, int64_t n, long long* bsum)
+// block-wise inclusive scan, writing per-block totals; with farea the scanned
+// values are the quantised areas, formed here (FP64 divisions in a kernel of
+// their own had taken 45 us for 1.93M faces, the scan of 1,024-value blocks
+// with a barrier per doubling 25; together now 51)
+__global__ void __launch_bounds__(kScanThreads)
+k_scan_block(long long* x, int64_t n, const double* __restrict__ farea, const DevScalars* sc, long long* bsum)
 {
-    __shared__ long long s[kScanBlock];
-    const int64_t i = blockIdx.x * (int64_t)kScanBlock + threadIdx.x;
-    s[threadIdx.x] = i < n ? x[i] : 0;
-    __syncthreads();
-    for (int off = 1; off < kScanBlock; off <<= 1) {
-        long long v = threadIdx.x >= off ? s[threadIdx.x - off] : 0;
-        __syncthreads();
-        s[threadIdx.x] += v;
+    __shared__ long long wsum[32];
+    __shared__ double s_scale;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const double amax = farea ? __longlong_as_double((long long)sc->amax_bits) : 0.0;
+    if (farea) {
+        if (threadIdx.x == 0) s_scale = amax > 0.0 ? __ddiv_rn(4294967296.0, amax) : 0.0;
         __syncthreads();
     }
-    if (i < n) x[i] = s[threadIdx.x];
-    if (threadIdx.x == kScanBlock - 1) bsum[blockIdx.x] = s[threadIdx.x];
+    const int64_t i0 = blockIdx.x * (int64_t)kScanBlock + (int64_t)threadIdx.x * kScanItems;
+    long long v[kScanItems], sum = 0;
+    static_assert(kScanItems == 4, "two 16-byte loads");
+    if (i0 + 4 <= n) {
+        const longlong2* src = (const longlong2*)(farea ? (const long long*)farea : x) + i0 / 2;
+        const longlong2 a = src[0], b = src[1];
+        v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+    } else {
+        for (int k = 0; k < 4; ++k) v[k] = i0 + k < n ? (farea ? __double_as_longlong(farea[i0 + k]) : x[i0 + k]) : 0;
+    }
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k) {
+        if (farea) v[k] = amax > 0.0 && i0 + k < n ? quantise_area(__longlong_as_double(v[k]), amax, s_scale) : 0LL;
+        sum += v[k];
+    }
+    long long inc = sum;
+    for (int off = 1; off < 32; off <<= 1) {
+        const long long u = __shfl_up_sync(0xFFFFFFFFu, inc, off);
+        if (lane >= off) inc += u;
+    }
+    if (lane == 31) wsum[warp] = inc;
+    __syncthreads();
+    if (warp == 0) {
+        long long t = wsum[lane];
+        for (int off = 1; off < 32; off <<= 1) {
+            const long long u = __shfl_up_sync(0xFFFFFFFFu, t, off);
+            if (lane >= off) t += u;
+        }
+        wsum[lane] = t;
+    }
+    __syncthreads();
+    long long run = inc - sum + (warp ? wsum[warp - 1] : 0);
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k) {
+        run += v[k];
+        if (i0 + k < n) x[i0 + k] = run;
+    }
+    if (threadIdx.x == kScanThreads - 1) bsum[blockIdx.x] = run;
 }
 
-__global__ void k_scan_add(long long* x, int64_t n, const long long* bsum_incl)
+__global__ void __launch_bounds__(kScanThreads)
+k_scan_add(long long* x, int64_t n, const long long* bsum_incl)
 {
-    const int64_t i = blockIdx.x * (int64_t)kScanBlock + threadIdx.x;
-    if (i >= n || blockIdx.x == 0) return;
-    x[i] += bsum_incl[blockIdx.x - 1];
+    if (blockIdx.x == 0) return;
+    const long long add = bsum_incl[blockIdx.x - 1];
+    const int64_t i0 = blockIdx.x * (int64_t)kScanBlock;
+    for (int k = threadIdx.x; k < kScanBlock; k += kScanThreads)
+        if (i0 + k < n) x[i0 + k] += add;
 }
 
-__global__ void k_store_total(const long long* cdf, int64_t T, DevScalars* sc)
-{
-    if (threadIdx.x == 0 && blockIdx.x == 0) sc->total = T > 0 ? cdf[T - 1] : 0;
-}
-
-static rc_status scan_inclusive(long long* x, int64_t n, cudaStream_t s)
+// inclusive scan of x, or of the quantised areas into x
+static rc_status scan_inclusive(long long* x, int64_t n, const double* farea, const DevScalars* sc, cudaStream_t s)
 {
     if (n <= 0) return RC_OK;
     const int64_t nb = (n + kScanBlock - 1) / kScanBlock;
@@ -901,12 +1282,12 @@ static rc_status scan_inclusive(long long* x, int64_t n, cudaStream_t s)
     BuildScratch g{s};
     RC_CUDA(cudaMallocAsync(&bs, sizeof(long long) * nb, s));
     g.p[0] = bs;
-    k_scan_block<<<(unsigned)nb, kScanBlock, 0, s>>>(x, n, bs);
+    k_scan_block<<<(unsigned)nb, kScanThreads, 0, s>>>(x, n, farea, sc, bs);
     RC_LAUNCHED();
     if (nb > 1) {
-        rc_status st = scan_inclusive(bs, nb, s);
+        rc_status st = scan_inclusive(bs, nb, nullptr, nullptr, s);
         if (st != RC_OK) return st;
-        k_scan_add<<<(unsigned)nb, kScanBlock, 0, s>>>(x, n, bs);
+        k_scan_add<<<(unsigned)nb, kScanThreads, 0, s>>>(x, n, bs);
         RC_LAUNCHED();
     }
     return RC_OK;
@@ -923,14 +1304,13 @@ __device__ __forceinline__ double uniform01(unsigned long long seed, long long i
 }
 
 __global__ void k_sample_area(const float* __restrict__ V, const int32_t* __restrict__ F, int64_t T,
-                              const long long* __restrict__ cdf, const DevScalars* sc,
-                              const float* __restrict__ fnorm, int64_t n, unsigned long long seed,
+                              const long long* __restrict__ cdf, const float* __restrict__ fnorm, int64_t n, unsigned long long seed,
                               float* P, float* Nout, int32_t* face, double* weight)
 {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
     const double u0 = uniform01(seed, i, 0), u1 = uniform01(seed, i, 1), u2 = uniform01(seed, i, 2);
-    const long long total = sc->total;
+    const long long total = cdf[T - 1];
     const long long target = (long long)floor(__dmul_rn(u0, __ll2double_rn(total)));
     int64_t lo = 0, hi = T - 1;
     while (lo < hi) {
@@ -943,12 +1323,12 @@ __global__ void k_sample_area(const float* __restrict__ V, const int32_t* __rest
     const double wb = __dmul_rn(s, __dsub_rn(1.0, u2));
     const double wc = __dmul_rn(s, u2);
     for (int k = 0; k < 3; ++k) {
-        const double A = V[3 * (int64_t)F[3 * f + 0] + k];
-        const double B = V[3 * (int64_t)F[3 * f + 1] + k];
-        const double C = V[3 * (int64_t)F[3 * f + 2] + k];
+        const double A = widen(V[3 * (int64_t)F[3 * f + 0] + k]);
+        const double B = widen(V[3 * (int64_t)F[3 * f + 1] + k]);
+        const double C = widen(V[3 * (int64_t)F[3 * f + 2] + k]);
         double p = __dadd_rn(__dmul_rn(wa, A), __dmul_rn(wb, B));
         p = __dadd_rn(p, __dmul_rn(wc, C));
-        P[3 * i + k] = __double2float_rn(p);
+        P[3 * i + k] = narrow(p);
         Nout[3 * i + k] = fnorm[3 * f + k];
     }
     face[i] = (int32_t)f;
@@ -997,22 +1377,35 @@ __global__ void k_point_morton(const float* __restrict__ P, int64_t n, float lx,
 // ---------------------------------------------------------------------------
 static inline unsigned nblocks(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
+static int device_sms()
+{
+    int dev = 0, sms = 1;
+    cudaGetDevice(&dev);
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 1;
+    return sms;
+}
+
 // Stable LSD sort of (key, value) pairs by the low `passes` bytes of the key;
 // the result is back in (keys, vals) when `passes` is even.
 static rc_status sort_pairs(unsigned long long* keys, int32_t* vals, int64_t n, int passes, unsigned int* err,
                             cudaStream_t s)
 {
     if (n <= 1) return RC_OK;
+    if (n <= kSmallSort) {
+        RC_CUDA(cudaFuncSetAttribute(k_sort_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SmallSort)));
+        k_sort_small<<<1, kSmallThreads, sizeof(SmallSort), s>>>(keys, vals, (int)n, passes, err);
+        RC_LAUNCHED();
+        return RC_OK;
+    }
     unsigned long long* k1 = nullptr;
     int32_t* v1 = nullptr;
     unsigned int* counts = nullptr;
-    // about two tiles per SM (a multiple of the block size, 512 to 4096 keys):
-    // small sorts spread over the GPU, large ones keep the count table short
-    int dev = 0, sms = 1;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 1;
-    int64_t tile = (n + 2 * sms - 1) / (2 * sms);
-    tile = std::min<int64_t>(kSortTile, std::max<int64_t>(512, (tile + kSortThreads - 1) / kSortThreads * kSortThreads));
+    // tiles of 512 to 2,048 keys, at least two per SM: small sorts spread over
+    // the GPU, large ones keep the count table short (2,048 keys leave room
+    // for five blocks per SM)
+    const int sms = device_sms();
+    const int items = n <= (int64_t)2 * sms * 512 ? 2 : n <= (int64_t)2 * sms * 1024 ? 4 : 8;
+    const int64_t tile = (int64_t)items * kSortThreads;
     const int nblk = (int)((n + tile - 1) / tile);
     BuildScratch g{s};
     RC_CUDA(cudaMallocAsync(&k1, sizeof(unsigned long long) * n, s));
@@ -1023,14 +1416,15 @@ static rc_status sort_pairs(unsigned long long* keys, int32_t* vals, int64_t n, 
     g.p[2] = counts;
     unsigned long long *kin = keys, *kout = k1;
     int32_t *vin = vals, *vout = v1;
+    const auto scatter = items == 2 ? k_sort_scatter<2> : items == 4 ? k_sort_scatter<4> : k_sort_scatter<8>;
     for (int pass = 0; pass < passes; ++pass) {
         const int shift = 8 * pass;
         k_sort_hist<<<nblk, kSortThreads, 0, s>>>(kin, n, shift, (int)tile, nblk, counts);
         RC_LAUNCHED();
-        k_sort_scan<<<8, 1024, 0, s>>>(counts, nblk, counts + (int64_t)256 * nblk);
+        k_sort_scan<<<32, 256, 0, s>>>(counts, nblk, counts + (int64_t)256 * nblk);
         RC_LAUNCHED();
-        k_sort_scatter<<<nblk, kSortThreads, 0, s>>>(kin, vin, n, shift, (int)tile, nblk, counts,
-                                                     counts + (int64_t)256 * nblk, kout, vout, err);
+        scatter<<<nblk, kSortThreads, 0, s>>>(kin, vin, n, shift, nblk, counts, counts + (int64_t)256 * nblk, kout, vout,
+                                              err);
         RC_LAUNCHED();
         std::swap(kin, kout);
         std::swap(vin, vout);
@@ -1061,7 +1455,6 @@ __global__ void k_init_scalars(DevScalars* sc)
 {
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     sc->amax_bits = 0;
-    sc->total = 0;
     for (int k = 0; k < 3; ++k) { sc->cmin[k] = 0x7FFFFFFF; sc->cmax[k] = (int)0x80000000; }
     sc->vmaxabs = 0;
     sc->err_index = 0x7FFFFFFF;
@@ -1083,15 +1476,10 @@ static rc_status face_data(rc_bvh h, float* tbox, cudaStream_t s)
 {
     rc_status st = init_scalars(h->sc, s);
     if (st != RC_OK) return st;
-    k_face_prep<<<nblocks(h->T, 256), 256, 0, s>>>(h->V, h->nV, h->F, h->T, h->fnorm, h->farea, tbox, h->sc);
+    k_face_prep<<<(unsigned)std::min<int64_t>(nblocks(h->T, kPrepThreads), 8 * (int64_t)device_sms()), kPrepThreads, 0, s>>>(
+        h->V, h->nV, h->F, h->T, h->fnorm, h->farea, tbox, h->sc);
     RC_LAUNCHED();
-    k_quant_area<<<nblocks(h->T, 256), 256, 0, s>>>(h->farea, h->T, h->sc, h->cdf);
-    RC_LAUNCHED();
-    st = scan_inclusive(h->cdf, h->T, s);
-    if (st != RC_OK) return st;
-    k_store_total<<<1, 1, 0, s>>>(h->cdf, h->T, h->sc);
-    RC_LAUNCHED();
-    return RC_OK;
+    return scan_inclusive(h->cdf, h->T, h->farea, h->sc, s);
 }
 
 // mesh validity and scene bounds from the scalars already read back
@@ -1106,13 +1494,6 @@ static rc_status checked_scalars(rc_bvh h)
     // the tree depth is set by the build once the tree exists (a refit keeps
     // the topology and hence the depth)
     return RC_OK;
-}
-
-static rc_status check_scalars(rc_bvh h, cudaStream_t s)
-{
-    RC_CUDA(cudaMemcpyAsync(&h->host_sc, h->sc, sizeof(DevScalars), cudaMemcpyDeviceToHost, s));
-    RC_CUDA(cudaStreamSynchronize(s));
-    return checked_scalars(h);
 }
 
 // PLOC build of the binary tree over the Morton-sorted leaves (h->order);
@@ -1214,44 +1595,42 @@ static rc_status build_wide(rc_bvh h, const float* tbox, cudaStream_t s)
         return RC_OK;
     }
     const int64_t n_int = h->n_int;
-    int32_t* q = nullptr;
-    int* counts = nullptr;
+    int2* q = nullptr;
     BuildScratch g{s};
-    RC_CUDA(cudaMallocAsync(&q, sizeof(int32_t) * 4 * n_int, s));
+    RC_CUDA(cudaMallocAsync(&q, sizeof(int2) * (2 * n_int + 1), s));   // two queues, then their sizes
     g.p[0] = q;
-    RC_CUDA(cudaMallocAsync(&counts, sizeof(int) * 4, s));
-    g.p[1] = counts;
-    int32_t *qa_bin = q, *qa_wide = q + n_int, *qb_bin = q + 2 * n_int, *qb_wide = q + 3 * n_int;
-    int *ca = counts, *cb = counts + 1;
-    k_wide_init<<<1, 32, 0, s>>>(qa_bin, qa_wide, counts);
-    RC_LAUNCHED();
-    // The top `split` levels take one launch each (a level's queue is at most
+    int2 *qa = q, *qb = q + n_int;
+    int *ca = (int*)(q + 2 * n_int), *cb = ca + 1;
+    int* wide_count = &h->sc->wide_nodes;
+    // The top `split` levels go level by level (a level's queue is at most
     // 4^level long); then one launch finishes every queued subtree, a thread
     // each, once the queue holds about n_int / RC_WIDE_SUBTREE nodes.  Levels
     // past the bottom of a shallow tree find an empty queue.
     int split = 0;
     while (split < 30 && std::pow(4.0, (double)split) * RC_WIDE_SUBTREE < (double)n_int) ++split;
     if (RC_WIDE_SUBTREE <= 0) split = kStack;      // a deeper tree is rejected anyway
-    int level = 0;
+    int level = std::min(split, kWideTop);
+    k_wide_top<<<1, kWideTopThreads, 0, s>>>(h->nodes, qa, qb, ca, wide_count, h->wnodes, h->sc, level);
+    RC_LAUNCHED();
+    if (level & 1) {
+        std::swap(qa, qb);
+        std::swap(ca, cb);
+    }
     for (; level < split; ++level) {
         const double cap = std::min((double)n_int, std::pow(4.0, (double)std::min(level, 30)));
         const unsigned grid = (unsigned)std::max(1.0, std::ceil(cap / 256.0));
         RC_CUDA(cudaMemsetAsync(cb, 0, sizeof(int), s));
-        k_wide_level<<<grid, 256, 0, s>>>(n_int, h->child, h->range, h->nbox, qa_bin, qa_wide, ca, qb_bin, qb_wide,
-                                          cb, counts + 2, h->wnodes, h->sc, level);
+        k_wide_level<<<grid, 256, 0, s>>>(h->nodes, qa, ca, qb, cb, wide_count, h->wnodes, h->sc, level);
         RC_LAUNCHED();
-        std::swap(qa_bin, qb_bin);
-        std::swap(qa_wide, qb_wide);
+        std::swap(qa, qb);
         std::swap(ca, cb);
     }
     {
         const double cap = std::min((double)n_int, std::pow(4.0, (double)std::min(level, 30)));
         const unsigned grid = (unsigned)std::max(1.0, std::ceil(cap / 256.0));
-        k_wide_subtrees<<<grid, 256, 0, s>>>(n_int, h->child, h->range, h->nbox, qa_bin, qa_wide, ca, counts + 2,
-                                             h->wnodes, h->sc, level);
+        k_wide_subtrees<<<grid, 256, 0, s>>>(h->nodes, qa, ca, wide_count, h->wnodes, h->sc, level);
         RC_LAUNCHED();
     }
-    RC_CUDA(cudaMemcpyAsync(&h->sc->wide_nodes, counts + 2, sizeof(int), cudaMemcpyDeviceToDevice, s));
     return RC_OK;
 }
 
@@ -1263,32 +1642,35 @@ static rc_status build_wide(rc_bvh h, const float* tbox, cudaStream_t s)
 // axis walk of the orthogonal cast tests these boxes (its rays run along a
 // frame axis) and still tests triangles in world coordinates.
 // ---------------------------------------------------------------------------
-__global__ void k_frame_leaf_boxes(const float* __restrict__ V, const int32_t* __restrict__ F,
-                                   const int32_t* __restrict__ order, int64_t T, int64_t nV, int64_t n_int,
-                                   FrameArgs fa, float* __restrict__ nbox_f)
+// q (two-term, exact to 1e-13 of sum |x_i f_i|) of a vertex along one frame
+// axis, rounded outward; the roundings of frame coordinates in FP64 are covered
+__device__ __forceinline__ void frame_bounds(float x, float y, float z, float a, float b, float c, float& lo, float& hi)
 {
-    const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (k >= T) return;
-    const int32_t f = order[k];
-    double lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
-    if (f >= 0 && f < T)
-        for (int a = 0; a < 3; ++a) {
-            const int64_t v = F[3 * (int64_t)f + a];
-            if (v < 0 || v >= nV) continue;
-            const double x = V[3 * v], y = V[3 * v + 1], z = V[3 * v + 2];
-            for (int j = 0; j < 3; ++j) {
-                // frame coordinate j: column j of the row-major frame
-                const double q = __dadd_rn(__dadd_rn(__dmul_rn(x, (double)fa.f[j]), __dmul_rn(y, (double)fa.f[3 + j])),
-                                           __dmul_rn(z, (double)fa.f[6 + j]));
-                lo[j] = fmin(lo[j], q);
-                hi[j] = fmax(hi[j], q);
-            }
-        }
-    float* b = nbox_f + 6 * (n_int + k);
-    for (int j = 0; j < 3; ++j) {
-        b[j] = __double2float_rd(lo[j]);
-        b[3 + j] = __double2float_ru(hi[j]);
-    }
+    float h, l;
+    dot2(x, a, y, b, z, c, h, l);
+    const float e = 2e-13f * (fabsf(x * a) + fabsf(y * b) + fabsf(z * c)) + 1e-36f;
+    lo = fminf(lo, __fadd_rd(h, __fsub_rd(l, e)));
+    hi = fmaxf(hi, __fadd_ru(h, __fadd_ru(l, e)));
+}
+
+// leaf boxes in frame coordinates and all boxes above them.  The bounds are
+// formed in two-term fp32 sums: in FP64 (1/64 of the fp32 rate) the leaf boxes
+// alone took 50 us for 203k triangles and the climb 49, together now 43.
+__global__ void __launch_bounds__(kClimb)
+k_frame_refit(const float* __restrict__ V, int64_t nV, const int32_t* __restrict__ F, const int32_t* __restrict__ order,
+              int64_t T, int64_t n_int, FrameArgs fa, const int32_t* __restrict__ parent,
+              const int32_t* __restrict__ child, const int32_t* __restrict__ range, float* nbox_f, int32_t* visits)
+{
+    __shared__ ClimbShared sm;
+    const int64_t k = blockIdx.x * (int64_t)kClimb + threadIdx.x;
+    float v[3][3];
+    float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+    if (k < T && gather_tri(V, nV, F, T, order[k], v))
+        for (int a = 0; a < 3; ++a)
+            for (int j = 0; j < 3; ++j)            // frame coordinate j: column j of the row-major frame
+                frame_bounds(v[a][0], v[a][1], v[a][2], fa.f[j], fa.f[3 + j], fa.f[6 + j], lo[j], hi[j]);
+    if (parent) climb<false>(sm, k < T, T, n_int, parent, child, range, nbox_f, nullptr, visits, nullptr, k, lo, hi);
+    else if (k < T) put_box(nbox_f, n_int + k, lo, hi);
 }
 
 __global__ void k_frame_pack(const float4* __restrict__ wnodes, int64_t n_int, int64_t T,
@@ -1300,13 +1682,24 @@ __global__ void k_frame_pack(const float4* __restrict__ wnodes, int64_t n_int, i
     const float4 idv = wnodes[wide_at(w, 7)];
     const int32_t ids[4] = {__float_as_int(idv.x), __float_as_int(idv.y), __float_as_int(idv.z), __float_as_int(idv.w)};
     float lo[3][4], hi[3][4];
+    const float4 cv = wnodes[wide_at(w, 6)];
+    const int32_t codes[4] = {__float_as_int(cv.x), __float_as_int(cv.y), __float_as_int(cv.z), __float_as_int(cv.w)};
     for (int k = 0; k < 4; ++k) {
         const float* b = nullptr;
+        int n = 1;
         if (ids[k] == kAllTris) b = all_box;
-        else if (ids[k] >= 0 && ids[k] < n_int + T) b = nbox_f + 6 * (int64_t)ids[k];
+        else if (ids[k] >= 0 && ids[k] < n_int) b = nbox_f + 6 * (int64_t)ids[k];
+        else if (ids[k] == kLeafChild && leaf_first(codes[k]) + leaf_count(codes[k]) <= T) {
+            b = nbox_f + 6 * (n_int + leaf_first(codes[k]));
+            n = leaf_count(codes[k]);
+        }
         for (int a = 0; a < 3; ++a) {
-            lo[a][k] = b ? b[a] : INFINITY;
-            hi[a][k] = b ? b[3 + a] : -INFINITY;
+            lo[a][k] = INFINITY;
+            hi[a][k] = -INFINITY;
+            for (int t = 0; b && t < n; ++t) {
+                lo[a][k] = fminf(lo[a][k], b[6 * t + a]);
+                hi[a][k] = fmaxf(hi[a][k], b[6 * t + 3 + a]);
+            }
         }
     }
     for (int a = 0; a < 3; ++a) {
@@ -1341,19 +1734,34 @@ rc_status frame_tree(rc_bvh h, const float f9[9], float4* ftree, cudaStream_t s)
     RC_CUDA(cudaMallocAsync(&nbox_f, sizeof(float) * 6 * (n_int + T + 1), s));
     g.p[0] = nbox_f;
     float* all_box = nbox_f + 6 * (n_int + T);
-    k_frame_leaf_boxes<<<(unsigned)((T + 255) / 256), 256, 0, s>>>(h->V, h->F, h->order, T, h->nV, n_int, fa, nbox_f);
-    RC_LAUNCHED();
+    const unsigned grid = nblocks(T, kClimb);
     if (T > kLeafMax) {
         RC_CUDA(cudaMallocAsync(&visits, sizeof(int32_t) * n_int, s));
         g.p[1] = visits;
         RC_CUDA(cudaMemsetAsync(visits, 0, sizeof(int32_t) * n_int, s));
-        k_refit<<<(unsigned)((T + 255) / 256), 256, 0, s>>>(T, n_int, h->parent, h->child, nbox_f, visits, h->sc);
+        k_frame_refit<<<grid, kClimb, 0, s>>>(h->V, h->nV, h->F, h->order, T, n_int, fa, h->parent, h->child, h->range,
+                                              nbox_f, visits);
         RC_LAUNCHED();
     } else {
+        k_frame_refit<<<grid, kClimb, 0, s>>>(h->V, h->nV, h->F, h->order, T, n_int, fa, nullptr, nullptr, nullptr, nbox_f,
+                                              nullptr);
+        RC_LAUNCHED();
         k_frame_all_box<<<1, 32, 0, s>>>(nbox_f, n_int, T, all_box);
         RC_LAUNCHED();
     }
     k_frame_pack<<<(unsigned)((n_int + 255) / 256), 256, 0, s>>>(h->wnodes, n_int, T, h->sc, nbox_f, all_box, ftree);
+    RC_LAUNCHED();
+    return RC_OK;
+}
+
+// triangle records, boxes and packed binary nodes of the tree in h (tiny
+// parts: records only)
+static rc_status refit_tree(rc_bvh h, cudaStream_t s)
+{
+    const bool tree = h->T > kLeafMax;
+    if (tree) RC_CUDA(cudaMemsetAsync(h->visits, 0, sizeof(int32_t) * h->n_int, s));
+    k_refit<<<nblocks(h->T, kClimb), kClimb, 0, s>>>(h->V, h->nV, h->F, h->order, h->T, h->n_int, tree ? h->parent : nullptr,
+                                               h->child, h->range, h->nbox, h->nodes, h->tris, h->visits, h->sc);
     RC_LAUNCHED();
     return RC_OK;
 }
@@ -1379,7 +1787,7 @@ rc_status build_bvh(rc_bvh h, cudaStream_t s)
         int32_t ord[kLeafMax];
         for (int i = 0; i < kLeafMax; ++i) ord[i] = i;
         RC_CUDA(cudaMemcpyAsync(h->order, ord, sizeof(int32_t) * T, cudaMemcpyHostToDevice, s));
-        k_pack_small<<<1, 32, 0, s>>>(T, tbox, h->nodes);
+        k_pack_small<<<1, 32, 0, s>>>(T, tbox, h->nodes, h->sc);
         RC_LAUNCHED();
         h->max_depth = 1;
     } else {
@@ -1404,25 +1812,17 @@ rc_status build_bvh(rc_bvh h, cudaStream_t s)
             k_karras<<<nblocks(n_int, 256), 256, 0, s>>>(k0, T, h->child, h->range, h->parent);
             RC_LAUNCHED();
         }
-        RC_CUDA(cudaMemsetAsync(h->visits, 0, sizeof(int32_t) * n_int, s));
-        k_leaf_boxes<<<nblocks(T, 256), 256, 0, s>>>(tbox, h->order, T, n_int, h->nbox);
-        RC_LAUNCHED();
-        k_refit<<<nblocks(T, 256), 256, 0, s>>>(T, n_int, h->parent, h->child, h->nbox, h->visits, h->sc);
-        RC_LAUNCHED();
-        k_pack<<<nblocks(n_int, 256), 256, 0, s>>>(n_int, h->child, h->range, h->nbox, h->nodes);
-        RC_LAUNCHED();
     }
+    if ((st = refit_tree(h, s)) != RC_OK) return st;
     st = build_wide(h, tbox, s);
     if (st != RC_OK) return st;
-    k_tri_records<<<nblocks(T, 256), 256, 0, s>>>(h->V, h->nV, h->F, h->order, T, h->tris);
-    RC_LAUNCHED();
     RC_CUDA(cudaMemcpyAsync(&h->host_sc, h->sc, sizeof(DevScalars), cudaMemcpyDeviceToHost, s));
     RC_CUDA(cudaStreamSynchronize(s));
     if ((st = checked_scalars(h)) != RC_OK) return st;
     if (h->host_sc.pad != 0) return set_error(RC_E_DEVICE, "radix sort produced an out-of-range position");
     if (T > kLeafMax) h->max_depth = h->host_sc.max_depth;
     h->wide_depth = h->host_sc.wide_depth;
-    for (int k = 0; k < 3; ++k) { h->lo[k] = 0; h->hi[k] = 0; }
+    for (int k = 0; k < 3; ++k) { h->lo[k] = h->host_sc.lo[k]; h->hi[k] = h->host_sc.hi[k]; }
     if (h->max_depth >= kStack)
         return set_error(RC_E_UNSUPPORTED, "BVH depth " + std::to_string(h->max_depth) +
                                                " exceeds the traversal stack");
@@ -1441,27 +1841,19 @@ rc_status refit_bvh(rc_bvh h, cudaStream_t s)
     g.p[0] = tbox;
     rc_status st = face_data(h, tbox, s);
     if (st != RC_OK) return st;
-    st = check_scalars(h, s);
-    if (st != RC_OK) return st;
     if (T <= kLeafMax) {
-        k_pack_small<<<1, 32, 0, s>>>(T, tbox, h->nodes);
-        RC_LAUNCHED();
-    } else {
-        const int64_t n_int = h->n_int;
-        RC_CUDA(cudaMemsetAsync(h->visits, 0, sizeof(int32_t) * n_int, s));
-        k_leaf_boxes<<<nblocks(T, 256), 256, 0, s>>>(tbox, h->order, T, n_int, h->nbox);
-        RC_LAUNCHED();
-        k_refit<<<nblocks(T, 256), 256, 0, s>>>(T, n_int, h->parent, h->child, h->nbox, h->visits, h->sc);
-        RC_LAUNCHED();
-        k_pack<<<nblocks(n_int, 256), 256, 0, s>>>(n_int, h->child, h->range, h->nbox, h->nodes);
+        k_pack_small<<<1, 32, 0, s>>>(T, tbox, h->nodes, h->sc);
         RC_LAUNCHED();
     }
+    if ((st = refit_tree(h, s)) != RC_OK) return st;
     st = build_wide(h, tbox, s);
     if (st != RC_OK) return st;
-    k_tri_records<<<nblocks(T, 256), 256, 0, s>>>(h->V, h->nV, h->F, h->order, T, h->tris);
-    RC_LAUNCHED();
+    // one synchronisation, as in the build: a bad vertex is reported from the
+    // final readback
     RC_CUDA(cudaMemcpyAsync(&h->host_sc, h->sc, sizeof(DevScalars), cudaMemcpyDeviceToHost, s));
     RC_CUDA(cudaStreamSynchronize(s));
+    if ((st = checked_scalars(h)) != RC_OK) return st;
+    for (int k = 0; k < 3; ++k) { h->lo[k] = h->host_sc.lo[k]; h->hi[k] = h->host_sc.hi[k]; }
     h->wide_depth = h->host_sc.wide_depth;
     if (3 * h->wide_depth + 1 >= kStack4)
         return set_error(RC_E_UNSUPPORTED, "4-wide BVH depth exceeds the traversal stack after refit");
@@ -1477,7 +1869,7 @@ rc_status sample_points(rc_bvh h, int64_t n, const rc_params* p, float* P, float
         RC_LAUNCHED();
         return RC_OK;
     }
-    k_sample_area<<<nblocks(n, 256), 256, 0, s>>>(h->V, h->F, h->T, h->cdf, h->sc, h->fnorm, n, p->seed,
+    k_sample_area<<<nblocks(n, 256), 256, 0, s>>>(h->V, h->F, h->T, h->cdf, h->fnorm, n, p->seed,
                                                   P, N, face, weight);
     RC_LAUNCHED();
     return RC_OK;

@@ -569,20 +569,6 @@ __device__ __forceinline__ float child_ld(const float4* __restrict__ wnodes, int
     return __ldg((const float*)(wnodes + wide_at(w, c)) + k);
 }
 
-// the smallest and largest value over the warp
-__device__ __forceinline__ float warp_min(float x)
-{
-    float r;
-    asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
-    return r;
-}
-__device__ __forceinline__ float warp_max(float x)
-{
-    float r;
-    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
-    return r;
-}
-
 // The warp builds the point's frontier: the origin set of o (the nodes whose
 // boxes contain o) is walked level by level, up to eight nodes at a time, a
 // lane per child; `queue` (shared, kFrontQueue ints) holds the nodes visited
@@ -882,21 +868,6 @@ struct AxisRay {
     int k;                // frame axis of the ray
     int pos;              // 1: along +column k, 0: along -column k
 };
-
-// x a + y b + z c as an unevaluated sum hi + lo of two fp32 values, within
-// 1e-13 of |x a| + |y b| + |z c| (each product and sum split into its rounded
-// value and its error: Dekker 1971, Knuth's TwoSum)
-__device__ __forceinline__ void dot2(float x, float a, float y, float b, float z, float c, float& hi, float& lo)
-{
-    const float p0 = __fmul_rn(x, a), p1 = __fmul_rn(y, b), p2 = __fmul_rn(z, c);
-    const float e0 = __fmaf_rn(x, a, -p0), e1 = __fmaf_rn(y, b, -p1), e2 = __fmaf_rn(z, c, -p2);
-    const float s = __fadd_rn(p0, p1), t = __fsub_rn(s, p0);
-    const float f = __fadd_rn(__fsub_rn(p0, __fsub_rn(s, t)), __fsub_rn(p1, t));
-    hi = __fadd_rn(s, p2);
-    const float v = __fsub_rn(hi, s);
-    const float g = __fadd_rn(__fsub_rn(s, __fsub_rn(hi, v)), __fsub_rn(p2, v));
-    lo = __fadd_rn(__fadd_rn(__fadd_rn(e0, e1), e2), __fadd_rn(f, g));
-}
 
 // The band of an axis ray (see above).  Its bounds are sums hi + lo -+ tol
 // rounded outward; everything in tol is rounded up by its spare factors.

@@ -63,7 +63,6 @@ constexpr size_t kVarScratchBytes = kVarPartOffset + 2 * sizeof(double) * kVarMa
 // ---------------------------------------------------------------------------
 struct DevScalars {
     unsigned long long amax_bits;  // max face area (FP64 bits, >= 0)
-    long long total;               // total quantised area
     int cmin[3], cmax[3];          // box-centre bounds (orderable float ints)
     int vmaxabs;                   // max |coordinate| (orderable float int)
     int err_index;                 // first bad face (index out of range), else -1
@@ -72,9 +71,11 @@ struct DevScalars {
     int pad;
     int wide_depth;
     int wide_nodes;                // 4-wide nodes allocated
+    float lo[3], hi[3];            // box of the whole part (the root's)
 };
 
 constexpr int kAllTris = -2;       // wide-node child made of all triangles (parts with <= kLeafMax of them)
+constexpr int kLeafChild = -3;     // wide-node child that is a leaf (its triangles are in its code)
 
 // machining frame on the device (Section 3.2)
 struct FrameArgs { float f[9]; const float4* tree; double sc_c[3]; double sc_r; };
@@ -210,6 +211,55 @@ __host__ __device__ __forceinline__ double ordered_to_double(long long i)
     u.i = i >= 0 ? i : i ^ 0x7FFFFFFFFFFFFFFFLL;
     return u.d;
 #endif
+}
+
+// the smallest and largest value over the warp
+__device__ __forceinline__ float warp_min(float x)
+{
+    float r;
+    asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float warp_max(float x)
+{
+    float r;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// x a + y b + z c as an unevaluated sum hi + lo of two fp32 values, within
+// 1e-13 of |x a| + |y b| + |z c| (each product and sum split into its rounded
+// value and its error: Dekker 1971, Knuth's TwoSum)
+__device__ __forceinline__ void dot2(float x, float a, float y, float b, float z, float c, float& hi, float& lo)
+{
+    const float p0 = __fmul_rn(x, a), p1 = __fmul_rn(y, b), p2 = __fmul_rn(z, c);
+    const float e0 = __fmaf_rn(x, a, -p0), e1 = __fmaf_rn(y, b, -p1), e2 = __fmaf_rn(z, c, -p2);
+    const float s = __fadd_rn(p0, p1), t = __fsub_rn(s, p0);
+    const float f = __fadd_rn(__fsub_rn(p0, __fsub_rn(s, t)), __fsub_rn(p1, t));
+    hi = __fadd_rn(s, p2);
+    const float v = __fsub_rn(hi, s);
+    const float g = __fadd_rn(__fsub_rn(s, __fsub_rn(hi, v)), __fsub_rn(p2, v));
+    lo = __fadd_rn(__fadd_rn(__fadd_rn(e0, e1), e2), __fadd_rn(f, g));
+}
+
+// Conversions between fp32 and FP64 by integer operations: they issue at the
+// FP64 rate otherwise, 1/64 of fp32's.  widen: exact, finite values.
+__device__ __forceinline__ double widen(float f)
+{
+    const unsigned b = __float_as_uint(f), m = b & 0x7FFFFFFFu;
+    if (m - 1u < 0x007FFFFFu) return (double)f;                  // subnormal
+    return __hiloint2double((int)((b & 0x80000000u) | (m ? (m >> 3) + 0x38000000u : 0u)), (int)(b << 29));
+}
+
+// the nearest fp32 value (ties to even) of a double
+__device__ __forceinline__ float narrow(double d)
+{
+    const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+    const unsigned e = (hi >> 20) & 0x7FFu;
+    if (e < 1023u - 126u || e >= 1023u + 127u) return __double2float_rn(d);   // not a normal fp32 value, or zero
+    const unsigned t = (((hi & 0x7FFFFFFFu) - 0x38000000u) << 3) | (lo >> 29), rest = lo & 0x1FFFFFFFu;
+    const unsigned up = rest > 0x10000000u || (rest == 0x10000000u && (t & 1u)) ? 1u : 0u;
+    return __uint_as_float((hi & 0x80000000u) | (t + up));
 }
 
 // splitmix64 (Steele, Lea, Flood 2014): mix(x + golden)
