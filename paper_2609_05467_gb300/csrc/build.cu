@@ -1377,7 +1377,7 @@ __global__ void k_point_morton(const float* __restrict__ P, int64_t n, float lx,
 // ---------------------------------------------------------------------------
 static inline unsigned nblocks(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
-static int device_sms()
+int device_sms()
 {
     int dev = 0, sms = 1;
     cudaGetDevice(&dev);
@@ -1668,7 +1668,7 @@ k_frame_refit(const float* __restrict__ V, int64_t nV, const int32_t* __restrict
     if (k < T && gather_tri(V, nV, F, T, order[k], v))
         for (int a = 0; a < 3; ++a)
             for (int j = 0; j < 3; ++j)            // frame coordinate j: column j of the row-major frame
-                frame_bounds(v[a][0], v[a][1], v[a][2], fa.f[j], fa.f[3 + j], fa.f[6 + j], lo[j], hi[j]);
+                frame_bounds(v[a][0], v[a][1], v[a][2], fa.f[0][j], fa.f[0][3 + j], fa.f[0][6 + j], lo[j], hi[j]);
     if (parent) climb<false>(sm, k < T, T, n_int, parent, child, range, nbox_f, nullptr, visits, nullptr, k, lo, hi);
     else if (k < T) put_box(nbox_f, n_int + k, lo, hi);
 }
@@ -1726,8 +1726,8 @@ __global__ void k_frame_all_box(const float* __restrict__ nbox_f, int64_t n_int,
 rc_status frame_tree(rc_bvh h, const float f9[9], float4* ftree, cudaStream_t s)
 {
     const int64_t T = h->T, n_int = h->n_int;
-    FrameArgs fa;
-    for (int k = 0; k < 9; ++k) fa.f[k] = f9[k];
+    FrameArgs fa = {};
+    for (int k = 0; k < 9; ++k) fa.f[0][k] = f9[k];
     float* nbox_f = nullptr;
     int32_t* visits = nullptr;
     BuildScratch g{s};

@@ -58,7 +58,7 @@ k_moments(const float* __restrict__ V, const int32_t* __restrict__ F, const doub
         double v[3][3];
         for (int c = 0; c < 3; ++c) {
             const int64_t vi = F[3 * f + c];
-            for (int k = 0; k < 3; ++k) v[c][k] = __dsub_rn((double)V[3 * vi + k], r[k]);
+            for (int k = 0; k < 3; ++k) v[c][k] = __dsub_rn(widen(V[3 * vi + k]), r[k]);
         }
         double sv[3];
         for (int k = 0; k < 3; ++k) sv[k] = __dadd_rn(__dadd_rn(v[0][k], v[1][k]), v[2][k]);
@@ -91,6 +91,7 @@ __global__ void k_moments_final(const double* __restrict__ partial, int blocks, 
 {
     if (threadIdx.x >= 10) return;
     double s = 0.0;
+#pragma unroll 32
     for (int b = 0; b < blocks; ++b) s = __dadd_rn(s, partial[10 * b + threadIdx.x]);
     out[threadIdx.x] = s;
 }
@@ -102,142 +103,314 @@ __global__ void k_moments_final(const double* __restrict__ partial, int blocks, 
 // H[cell] += quantised area; rep[cell] = max of (qa << 31 | (2^31-1 - face)),
 // i.e. the largest face, lowest id on ties.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ int cell_index(double u)
+__device__ __forceinline__ int cell_index(float a, float m)   // u = a / m, |a| <= m
 {
-    int i = (int)floor(__dmul_rn(__dadd_rn(u, 1.0), (double)(kCells / 2)));
+    // in fp32 where (u + 1) kCells / 2 is clear of a whole number by more
+    // than its rounding (three operations of 2^-23, values up to 32)
+    if (a == 0.0f) return kCells / 2;
+    if (a == m) return kCells - 1;
+    if (a == -m) return 0;
+    const float t = (__fdividef(a, m) + 1.0f) * (float)(kCells / 2), n = rintf(t);
+    int i = (int)floorf(t);
+    if (!(fabsf(t - n) > 1e-4f) || m < 1e-30f)
+        i = (int)floor(__dmul_rn(__dadd_rn(__ddiv_rn((double)a, (double)m), 1.0), (double)(kCells / 2)));
     return i < 0 ? 0 : (i > kCells - 1 ? kCells - 1 : i);
 }
 
+// The faces of a warp that share a cell add and compare among themselves
+// first (quantised areas are below 2^33): a flat side puts most of a part's
+// faces into one cell, and the atomics on it were what bound this kernel,
+// before the FP64 quotients.  203k faces: 69 -> 8 us.
 __global__ void k_normal_cells(const float* __restrict__ fnorm, const long long* __restrict__ cdf, int64_t T,
                                unsigned long long* __restrict__ H, unsigned long long* __restrict__ rep)
 {
+    constexpr unsigned kAll = 0xFFFFFFFFu;
     const int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (f >= T) return;
-    const long long qa = cdf[f] - (f ? cdf[f - 1] : 0LL);
-    if (qa <= 0) return;
-    const double n[3] = {(double)fnorm[3 * f], (double)fnorm[3 * f + 1], (double)fnorm[3 * f + 2]};
-    int k = 0;
-    if (fabs(n[1]) > fabs(n[k])) k = 1;
-    if (fabs(n[2]) > fabs(n[k])) k = 2;
-    const double sg = n[k] < 0.0 ? -1.0 : 1.0;
-    const double m = fabs(n[k]);
-    const double u = __ddiv_rn(__dmul_rn(n[(k + 1) % 3], sg), m);
-    const double v = __ddiv_rn(__dmul_rn(n[(k + 2) % 3], sg), m);
-    const int cell = (k * kCells + cell_index(u)) * kCells + cell_index(v);
-    atomicAdd(&H[cell], (unsigned long long)qa);
-    atomicMax(&rep[cell], ((unsigned long long)qa << 31) | (unsigned long long)(0x7FFFFFFFLL - f));
+    unsigned long long qa = 0;
+    int cell = -1;
+    if (f < T) {
+        const long long d = cdf[f] - (f ? cdf[f - 1] : 0LL);
+        if (d > 0) {
+            qa = (unsigned long long)d;
+            const float n[3] = {fnorm[3 * f], fnorm[3 * f + 1], fnorm[3 * f + 2]};
+            const int k = fabsf(n[2]) > fmaxf(fabsf(n[0]), fabsf(n[1])) ? 2 : fabsf(n[1]) > fabsf(n[0]) ? 1 : 0;
+            const float nk = k == 0 ? n[0] : k == 1 ? n[1] : n[2], na = k == 0 ? n[1] : k == 1 ? n[2] : n[0],
+                        nb = k == 0 ? n[2] : k == 1 ? n[0] : n[1];
+            const float sg = nk < 0.0f ? -1.0f : 1.0f;
+            cell = (k * kCells + cell_index(na * sg, fabsf(nk))) * kCells + cell_index(nb * sg, fabsf(nk));
+        }
+    }
+    const unsigned long long key = (qa << 31) | (unsigned long long)(0x7FFFFFFFLL - f);
+    for (unsigned left = __ballot_sync(kAll, cell >= 0); left;) {
+        const int c = __shfl_sync(kAll, cell, __ffs(left) - 1);
+        const bool in = cell == c;
+        const unsigned m = __ballot_sync(kAll, in);
+        left &= ~m;
+        if (!in) continue;
+        const unsigned long long sum = ((unsigned long long)__reduce_add_sync(m, (unsigned)(qa >> 16)) << 16) +
+                                       __reduce_add_sync(m, (unsigned)qa & 0xFFFFu);
+        const unsigned hi = __reduce_max_sync(m, (unsigned)(key >> 32));
+        const unsigned lo = __reduce_max_sync(m, (unsigned)(key >> 32) == hi ? (unsigned)key : 0u);
+        if ((threadIdx.x & 31) == __ffs(m) - 1) {
+            atomicAdd(&H[c], sum);
+            atomicMax(&rep[c], (unsigned long long)hi << 32 | lo);
+        }
+    }
 }
 
 // ---------------------------------------------------------------------------
 // device: bounding boxes of the vertices in many FP64 frames G (columns).
 // The defined coordinate is Q64 = fl64((x G0k + y G1k) + z G2k), its min and
-// max over the vertices exact.  FP64 is slow on this part, so two passes:
-//   A (fp32): Q32 with the fp32-rounded frame, per column its min and max
-//     and the largest S32 = |x||g0k| + |y||g1k| + |z||g2k|;
-//   B: vertices whose Q32 lies within W = 2^-19 max S32 of an fp32 extreme
-//     get Q64, and only those enter the FP64 min / max.
-// |Q32 - Q64| <= e = 4.1 * 2^-24 * S32 (rounding of the frame to fp32, two
-// three-term dot products), so the vertex holding the FP64 extreme has Q32
-// within 2 max e of the fp32 extreme; W = 2^-19 max S32 covers that twice,
-// including the rounding of the threshold itself.  The result is exactly the
-// one-pass FP64 result.  Block (x, g) handles a chunk of vertices for frame g;
-// per block and column one atomic on order-preserving integers.
+// max over the vertices exact.  FP64 issues at 1/64 of the fp32 rate, so:
+//   ranges (fp32): a block holds 2,048 vertices in registers and writes their
+//     least and largest Q32 for a slice of the frames, and their |x| maxima;
+//   exact: a block per frame finds the extremes over all chunks, and of the
+//     chunks that come within W of one it takes the vertices that do; only
+//     those get Q64 and enter the FP64 min / max.
+// |Q32 - Q64| <= e = 4.1 * 2^-24 * S (rounding of the frame to fp32, two
+// three-term dot products), S = sum of max |x_i| |g_ik| over the part, so the
+// vertex holding the FP64 extreme has Q32 within 2 e of the fp32 extreme;
+// W = 2^-19 S covers that twice, including the rounding of the threshold
+// itself.  The result is exactly the one-pass FP64 result.  (Reading every
+// vertex for every frame in both passes was bound by L2 and the warps' FP64
+// reductions: 101k vertices x 1,152 frames 216 + 407 us; now 71 + 72 us.)
 // ---------------------------------------------------------------------------
-constexpr int kBoxThreads = 256;
-constexpr int kBoxChunk = 8192;
-
-__global__ void k_box_init(long long* box, int* box32, int nf)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < nf * 6) box[i] = (i % 6) < 3 ? 0x7FFFFFFFFFFFFFFFLL : (long long)0x8000000000000000ULL;
-    if (i < nf * 9) {
-        const int c = i % 9;   // lo xyz, hi xyz, max S xyz
-        box32[i] = c < 3 ? 0x7FFFFFFF : (c < 6 ? (int)0x80000000 : 0);
-    }
-}
+constexpr int kBoxThreads = 256, kBoxWarps = kBoxThreads / 32, kBoxPer = 8;
+constexpr int kBoxChunk = kBoxThreads * kBoxPer;   // vertices of a block
+constexpr int kBoxRun = 32 * kBoxPer;              // consecutive vertices of a warp
+constexpr int64_t kBoxFine = 1 << 20;              // vertices up to which ranges are kept per warp: 113 MB
+constexpr int kBoxBatch = 32;                      // frames between two block reductions
 
 __device__ __forceinline__ float dot32(float x, float y, float z, float g0, float g1, float g2)
 {
-    return __fadd_rn(__fadd_rn(__fmul_rn(x, g0), __fmul_rn(y, g1)), __fmul_rn(z, g2));
+    return fmaf(x, g0, fmaf(y, g1, z * g2));
 }
 
 __global__ void __launch_bounds__(kBoxThreads)
-k_box_pass32(const float* __restrict__ V, int64_t nV, const double* __restrict__ G /*[nf][9]*/,
-             int* __restrict__ box32 /*[nf][9]*/)
+k_box_ranges(const float* __restrict__ V, int64_t nV, const double* __restrict__ G /*[nf][9]*/, int nf, int slice,
+             int per_warp, float* __restrict__ range /*[nf][groups][6]*/, float* __restrict__ amax /*[chunks][3]*/)
 {
-    const int g = blockIdx.y;
-    float gm[9];
-    for (int k = 0; k < 9; ++k) gm[k] = __double2float_rn(G[9 * g + k]);
-    float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY}, sm[3] = {0, 0, 0};
-    const int64_t v0 = (int64_t)blockIdx.x * kBoxChunk;
-    const int64_t v1 = min64(v0 + kBoxChunk, nV);
-    for (int64_t v = v0 + threadIdx.x; v < v1; v += blockDim.x) {
-        const float x = V[3 * v], y = V[3 * v + 1], z = V[3 * v + 2];
+    __shared__ float4 s_g[kBoxBatch][3];                   // columns
+    __shared__ float s_r[kBoxBatch][6][kBoxWarps];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t chunk = blockIdx.x, chunks = gridDim.x;
+    float x[kBoxPer], y[kBoxPer], z[kBoxPer], a[3] = {0.0f, 0.0f, 0.0f};
+#pragma unroll
+    for (int r = 0; r < kBoxPer; ++r) {
+        const int64_t v = min64(chunk * kBoxChunk + warp * kBoxRun + r * 32 + lane, nV - 1);
+        x[r] = V[3 * v], y[r] = V[3 * v + 1], z[r] = V[3 * v + 2];
+        a[0] = fmaxf(a[0], fabsf(x[r])), a[1] = fmaxf(a[1], fabsf(y[r])), a[2] = fmaxf(a[2], fabsf(z[r]));
+    }
+    if (blockIdx.y == 0) {
         for (int k = 0; k < 3; ++k) {
-            const float q = dot32(x, y, z, gm[k], gm[3 + k], gm[6 + k]);
-            lo[k] = fminf(lo[k], q);
-            hi[k] = fmaxf(hi[k], q);
-            sm[k] = fmaxf(sm[k], dot32(fabsf(x), fabsf(y), fabsf(z), fabsf(gm[k]), fabsf(gm[3 + k]),
-                                       fabsf(gm[6 + k])));
+            const float w = warp_max(a[k]);
+            if (lane == 0) s_r[0][k][warp] = w;
+        }
+        __syncthreads();
+        if (threadIdx.x < 3) {
+            float w = 0.0f;
+            for (int q = 0; q < kBoxWarps; ++q) w = fmaxf(w, s_r[0][threadIdx.x][q]);
+            amax[3 * chunk + threadIdx.x] = w;
         }
     }
-    for (int off = 16; off; off >>= 1)
-        for (int k = 0; k < 3; ++k) {
-            lo[k] = fminf(lo[k], __shfl_xor_sync(0xFFFFFFFFu, lo[k], off));
-            hi[k] = fmaxf(hi[k], __shfl_xor_sync(0xFFFFFFFFu, hi[k], off));
-            sm[k] = fmaxf(sm[k], __shfl_xor_sync(0xFFFFFFFFu, sm[k], off));
+    const int g_end = min(nf, (int)(blockIdx.y + 1) * slice);
+    for (int g0 = blockIdx.y * slice; g0 < g_end; g0 += kBoxBatch) {
+        const int m = min(kBoxBatch, g_end - g0);
+        __syncthreads();
+        for (int t = threadIdx.x; t < 9 * m; t += kBoxThreads) {
+            const int g = t / 9, e = t % 9;
+            ((float*)&s_g[g][e % 3])[e / 3] = __double2float_rn(G[9 * (int64_t)(g0 + g) + e]);
         }
-    if ((threadIdx.x & 31) == 0)
-        for (int k = 0; k < 3; ++k)
-            if (lo[k] <= hi[k]) {
-                atomicMin(&box32[9 * g + k], float_to_ordered(lo[k]));
-                atomicMax(&box32[9 * g + 3 + k], float_to_ordered(hi[k]));
-                atomicMax(&box32[9 * g + 6 + k], float_to_ordered(sm[k]));
+        __syncthreads();
+        for (int g = 0; g < m; ++g) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const float4 c = s_g[g][k];
+                float lo = INFINITY, hi = -INFINITY;
+#pragma unroll
+                for (int r = 0; r < kBoxPer; ++r) {
+                    const float q = dot32(x[r], y[r], z[r], c.x, c.y, c.z);
+                    lo = fminf(lo, q), hi = fmaxf(hi, q);
+                }
+                lo = warp_min(lo), hi = warp_max(hi);
+                if (lane == 0) {
+                    s_r[g][k][warp] = lo;
+                    s_r[g][3 + k][warp] = hi;
+                }
             }
+        }
+        __syncthreads();
+        if (per_warp) {
+            for (int t = threadIdx.x; t < 6 * kBoxWarps * m; t += kBoxThreads) {
+                const int g = t / (6 * kBoxWarps), q = t / 6 % kBoxWarps, k = t % 6;
+                range[((g0 + g) * chunks + chunk) * 6 * kBoxWarps + 6 * q + k] = s_r[g][k][q];
+            }
+            continue;
+        }
+        for (int t = threadIdx.x; t < 6 * m; t += kBoxThreads) {
+            const int g = t / 6, k = t % 6;
+            float v = s_r[g][k][0];
+            for (int q = 1; q < kBoxWarps; ++q) v = k < 3 ? fminf(v, s_r[g][k][q]) : fmaxf(v, s_r[g][k][q]);
+            range[((g0 + g) * chunks + chunk) * 6 + k] = v;
+        }
+    }
+}
+
+// (h, l) before (h2, l2) of values h + l with |l| at most half a unit of h
+__device__ __forceinline__ bool below2(float h, float l, float h2, float l2) { return h < h2 || (h == h2 && l < l2); }
+
+// h + l and h2 + l2 as one such pair
+__device__ __forceinline__ void join2(float& h, float& l, float a)
+{
+    const float x = __fadd_rn(l, a), t = __fadd_rn(h, x), u = __fsub_rn(t, h);
+    l = __fadd_rn(__fsub_rn(h, __fsub_rn(t, u)), __fsub_rn(x, u));
+    h = t;
 }
 
 __global__ void __launch_bounds__(kBoxThreads)
-k_box_pass64(const float* __restrict__ V, int64_t nV, const double* __restrict__ G /*[nf][9]*/,
-             const int* __restrict__ box32 /*[nf][9]*/, long long* __restrict__ box /*[nf][6]*/)
+k_box_exact(const float* __restrict__ V, int64_t nV, const double* __restrict__ G, const float* __restrict__ range,
+            const float* __restrict__ amax, int64_t chunks, int64_t groups, int run,
+            long long* __restrict__ box /*[nf][6], ordered*/)
 {
-    const int g = blockIdx.y;
-    double gd[9];
-    float gm[9];
+    __shared__ int s_ext[9];                       // ordered: lo, hi, |x| maxima
+    __shared__ long long s_box[6];
+    __shared__ int s_n;
+    __shared__ int s_group[kBoxThreads];           // groups of `run` vertices: index * 8 + columns
+    const int64_t g = blockIdx.x;
+    const int t = threadIdx.x;
+    if (t < 9) s_ext[t] = t < 3 ? 0x7FFFFFFF : (t < 6 ? (int)0x80000000 : 0);
+    if (t < 6) s_box[t] = t < 3 ? 0x7FFFFFFFFFFFFFFFLL : (long long)0x8000000000000000ULL;
+    __syncthreads();
+    const float* mine = range + g * groups * 6;
+    float e[9] = {INFINITY, INFINITY, INFINITY, -INFINITY, -INFINITY, -INFINITY, 0.0f, 0.0f, 0.0f};
+    for (int64_t c = t; c < groups; c += kBoxThreads)
+        for (int k = 0; k < 3; ++k) {
+            e[k] = fminf(e[k], mine[6 * c + k]);
+            e[3 + k] = fmaxf(e[3 + k], mine[6 * c + 3 + k]);
+        }
+    for (int64_t c = t; c < 3 * chunks; c += kBoxThreads) {
+        const float v = amax[c];
+        e[6] = fmaxf(e[6], c % 3 == 0 ? v : 0.0f);
+        e[7] = fmaxf(e[7], c % 3 == 1 ? v : 0.0f);
+        e[8] = fmaxf(e[8], c % 3 == 2 ? v : 0.0f);
+    }
     for (int k = 0; k < 9; ++k) {
-        gd[k] = G[9 * g + k];
-        gm[k] = __double2float_rn(gd[k]);
+        const float w = k < 3 ? warp_min(e[k]) : warp_max(e[k]);
+        if ((t & 31) == 0) {
+            if (k < 3) atomicMin(&s_ext[k], float_to_ordered(w));
+            else atomicMax(&s_ext[k], float_to_ordered(w));
+        }
     }
-    float tlo[3], thi[3];
+    __syncthreads();
+    __shared__ double s_gd[9];
+    __shared__ float s_gh[9], s_gl[9];             // the frame in two fp32 terms
+    __shared__ float2 s_two[6][kBoxWarps];
+    if (t < 9) {
+        const double d = G[9 * g + t];
+        s_gd[t] = d;
+        s_gh[t] = __double2float_rn(d);
+        s_gl[t] = __double2float_rn(d - (double)s_gh[t]);
+    }
+    __syncthreads();
+    float gm[9], tlo[3], thi[3], w2[3];
+    for (int k = 0; k < 9; ++k) gm[k] = s_gh[k];
     for (int k = 0; k < 3; ++k) {
-        const float w = ordered_to_float(box32[9 * g + 6 + k]) * 1.9073486328125e-06f;   // 2^-19
-        tlo[k] = __fadd_rn(ordered_to_float(box32[9 * g + k]), w);
-        thi[k] = __fsub_rn(ordered_to_float(box32[9 * g + 3 + k]), w);
+        const float S = ordered_to_float(s_ext[6]) * fabsf(gm[k]) + ordered_to_float(s_ext[7]) * fabsf(gm[3 + k]) +
+                        ordered_to_float(s_ext[8]) * fabsf(gm[6 + k]);
+        const float w = 1.9073486328125e-06f * S;   // 2^-19
+        tlo[k] = ordered_to_float(s_ext[k]) + w;
+        thi[k] = ordered_to_float(s_ext[3 + k]) - w;
+        w2[k] = 2e-12f * S + 1e-35f;
     }
-    double lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
-    const int64_t v0 = (int64_t)blockIdx.x * kBoxChunk;
-    const int64_t v1 = min64(v0 + kBoxChunk, nV);
-    for (int64_t v = v0 + threadIdx.x; v < v1; v += blockDim.x) {
-        const float x = V[3 * v], y = V[3 * v + 1], z = V[3 * v + 2];
-        for (int k = 0; k < 3; ++k) {
-            const float q32 = dot32(x, y, z, gm[k], gm[3 + k], gm[6 + k]);
-            if (q32 <= tlo[k] || q32 >= thi[k]) {
-                double q = __dadd_rn(__dmul_rn((double)x, gd[k]), __dmul_rn((double)y, gd[3 + k]));
-                q = __dadd_rn(q, __dmul_rn((double)z, gd[6 + k]));
-                lo[k] = fmin(lo[k], q);
-                hi[k] = fmax(hi[k], q);
+    const auto two = [&](float x, float y, float z, int k, float& h, float& l) {
+        dot2(x, gm[k], y, gm[3 + k], z, gm[6 + k], h, l);
+        join2(h, l, x * s_gl[k] + y * s_gl[3 + k] + z * s_gl[6 + k]);
+    };
+    // first the extremes in two-term fp32 (error under 5e-13 S), then FP64 of
+    // the vertices within 2e-12 S of them: the turning axis keeps a flat side
+    // at its extreme in every step, thousands of vertices within W
+    float2 least[3], most[3];                      // (h, l); after the first round the thresholds
+    for (int k = 0; k < 3; ++k) {
+        least[k] = make_float2(INFINITY, 0.0f);
+        most[k] = make_float2(-INFINITY, 0.0f);
+    }
+    long long lo[3], hi[3];
+    for (int k = 0; k < 3; ++k) {
+        lo[k] = 0x7FFFFFFFFFFFFFFFLL;
+        hi[k] = (long long)0x8000000000000000ULL;
+    }
+    for (int round = 0; round < 2; ++round) {
+        for (int64_t c0 = 0; c0 < groups; c0 += kBoxThreads) {
+            __syncthreads();
+            if (t == 0) s_n = 0;
+            __syncthreads();
+            const int64_t c = c0 + t;
+            int cols = 0;
+            if (c < groups)
+                for (int k = 0; k < 3; ++k) cols |= !(mine[6 * c + k] > tlo[k] && mine[6 * c + 3 + k] < thi[k]) ? 1 << k : 0;
+            if (cols) s_group[atomicAdd(&s_n, 1)] = t * 8 + cols;
+            __syncthreads();
+            // a warp takes a run of 256 vertices, all its loads first
+            const int parts = run / kBoxRun;
+            for (int q = t >> 5; q < s_n * parts; q += kBoxWarps) {
+                const int e = s_group[q / parts];
+                const int64_t v0 = (c0 + (e >> 3)) * run + (q % parts) * kBoxRun + (t & 31);
+                float x[kBoxPer], y[kBoxPer], z[kBoxPer];
+#pragma unroll
+                for (int r = 0; r < kBoxPer; ++r) {
+                    const int64_t v = min64(v0 + 32 * r, nV - 1);
+                    x[r] = V[3 * v], y[r] = V[3 * v + 1], z[r] = V[3 * v + 2];
+                }
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    if (!((e >> k) & 1)) continue;
+#pragma unroll
+                    for (int r = 0; r < kBoxPer; ++r) {
+                        const float q32 = dot32(x[r], y[r], z[r], gm[k], gm[3 + k], gm[6 + k]);
+                        if (q32 > tlo[k] && q32 < thi[k]) continue;
+                        float h, l;
+                        two(x[r], y[r], z[r], k, h, l);
+                        if (round == 0) {
+                            if (below2(h, l, least[k].x, least[k].y)) least[k] = make_float2(h, l);
+                            if (below2(most[k].x, most[k].y, h, l)) most[k] = make_float2(h, l);
+                        } else if (!(below2(least[k].x, least[k].y, h, l) && below2(h, l, most[k].x, most[k].y))) {
+                            double d = __dadd_rn(__dmul_rn(widen(x[r]), s_gd[k]), __dmul_rn(widen(y[r]), s_gd[3 + k]));
+                            d = __dadd_rn(d, __dmul_rn(widen(z[r]), s_gd[6 + k]));
+                            lo[k] = min(lo[k], (long long)double_to_ordered(d));
+                            hi[k] = max(hi[k], (long long)double_to_ordered(d));
+                        }
+                    }
+                }
             }
         }
+        if (round == 1) break;
+        for (int k = 0; k < 6; ++k) {
+            float2 v = k < 3 ? least[k % 3] : most[k % 3];
+            for (int off = 16; off; off >>= 1) {
+                const float h = __shfl_xor_sync(0xFFFFFFFFu, v.x, off), l = __shfl_xor_sync(0xFFFFFFFFu, v.y, off);
+                if (k < 3 ? below2(h, l, v.x, v.y) : below2(v.x, v.y, h, l)) v = make_float2(h, l);
+            }
+            if ((t & 31) == 0) s_two[k][t >> 5] = v;
+        }
+        __syncthreads();
+        for (int k = 0; k < 6; ++k) {
+            float2 v = s_two[k][0];
+            for (int q = 1; q < kBoxWarps; ++q) {
+                const float2 o = s_two[k][q];
+                if (k < 3 ? below2(o.x, o.y, v.x, v.y) : below2(v.x, v.y, o.x, o.y)) v = o;
+            }
+            join2(v.x, v.y, k < 3 ? w2[k % 3] : -w2[k % 3]);
+            if (k < 3) least[k % 3] = v;
+            else most[k % 3] = v;
+        }
     }
-    for (int off = 16; off; off >>= 1)
-        for (int k = 0; k < 3; ++k) {
-            lo[k] = fmin(lo[k], __shfl_xor_sync(0xFFFFFFFFu, lo[k], off));
-            hi[k] = fmax(hi[k], __shfl_xor_sync(0xFFFFFFFFu, hi[k], off));
+    for (int k = 0; k < 3; ++k)
+        if (lo[k] <= hi[k]) {
+            atomicMin(&s_box[k], lo[k]);
+            atomicMax(&s_box[3 + k], hi[k]);
         }
-    if ((threadIdx.x & 31) == 0)
-        for (int k = 0; k < 3; ++k) {
-            if (lo[k] <= hi[k]) atomicMin(&box[6 * g + k], double_to_ordered(lo[k]));
-            if (lo[k] <= hi[k]) atomicMax(&box[6 * g + 3 + k], double_to_ordered(hi[k]));
-        }
+    __syncthreads();
+    if (t < 6) box[6 * g + t] = s_box[t];
 }
 
 // ---------------------------------------------------------------------------
@@ -516,22 +689,31 @@ rc_status rc_frame_candidates(rc_bvh h, const rc_params* p, rc_frames* out, void
     const int nf = (int)(G.size() / 9);
     const int64_t chunks = std::max<int64_t>(1, (h->nV + kBoxChunk - 1) / kBoxChunk);
     if (chunks > 0x7FFFFFFF) return set_error(RC_E_UNSUPPORTED, "too many vertices");
+    // ranges per warp's run of vertices (108 bytes a vertex and 1,152 frames)
+    // or, for a large part, per block: an edge that turns past an extreme
+    // touches every block of a part meshed in slabs, but few of the runs
+    const bool per_warp = h->nV <= kBoxFine;
+    const int64_t groups = per_warp ? chunks * kBoxWarps : chunks;
     double* dG = nullptr;
     long long* dbox = nullptr;
-    int* dbox32 = nullptr;
+    float* drange = nullptr;               // and the chunks' |x| maxima behind it
     FrameScratch sf{s};
     RC_CUDA(cudaMallocAsync(&dG, sizeof(double) * G.size(), s));
     sf.p[0] = dG;
     RC_CUDA(cudaMallocAsync(&dbox, sizeof(long long) * 6 * nf, s));
     sf.p[1] = dbox;
-    RC_CUDA(cudaMallocAsync(&dbox32, sizeof(int) * 9 * nf, s));
-    sf.p[2] = dbox32;
+    RC_CUDA(cudaMallocAsync(&drange, sizeof(float) * (6 * (size_t)groups * nf + 3 * chunks), s));
+    sf.p[2] = drange;
+    float* damax = drange + 6 * (size_t)groups * nf;
     RC_CUDA(cudaMemcpyAsync(dG, G.data(), sizeof(double) * G.size(), cudaMemcpyHostToDevice, s));
-    k_box_init<<<(9 * nf + 255) / 256, 256, 0, s>>>(dbox, dbox32, nf);
+    // slices of the frames: about eight blocks per SM, whole batches
+    const int64_t want = (8 * (int64_t)device_sms() + chunks - 1) / chunks;
+    const int batches = (nf + kBoxBatch - 1) / kBoxBatch;
+    const int slice = kBoxBatch * (int)((batches + std::min<int64_t>(want, batches) - 1) / std::min<int64_t>(want, batches));
+    k_box_ranges<<<dim3((unsigned)chunks, (unsigned)((nf + slice - 1) / slice)), kBoxThreads, 0, s>>>(h->V, h->nV, dG, nf, slice,
+                                                                                                     per_warp, drange, damax);
     RC_LAUNCHED();
-    k_box_pass32<<<dim3((unsigned)chunks, (unsigned)nf), kBoxThreads, 0, s>>>(h->V, h->nV, dG, dbox32);
-    RC_LAUNCHED();
-    k_box_pass64<<<dim3((unsigned)chunks, (unsigned)nf), kBoxThreads, 0, s>>>(h->V, h->nV, dG, dbox32, dbox);
+    k_box_exact<<<nf, kBoxThreads, 0, s>>>(h->V, h->nV, dG, drange, damax, chunks, groups, per_warp ? kBoxRun : kBoxChunk, dbox);
     RC_LAUNCHED();
     std::vector<long long> box(6 * (size_t)nf);
     RC_CUDA(cudaMemcpyAsync(box.data(), dbox, sizeof(long long) * 6 * nf, cudaMemcpyDeviceToHost, s));
@@ -581,7 +763,7 @@ rc_status rc_frame_candidates(rc_bvh h, const rc_params* p, rc_frames* out, void
     // volumes of the fp32 candidate frames (as the casts use them)
     FrameDev* fds = nullptr;
     RC_CUDA(cudaMallocAsync(&fds, sizeof(FrameDev) * out->k, s));
-    for (int c = 0; c < out->k && st == RC_OK; ++c) st = frame_setup_f(h, out->frame[c], fds + c, s);
+    st = frame_setups(h, out->frame, nullptr, out->k, fds, s);
     std::vector<FrameDev> hf(out->k);
     if (st == RC_OK)
         st = cudaMemcpyAsync(hf.data(), fds, sizeof(FrameDev) * out->k, cudaMemcpyDeviceToHost, s) == cudaSuccess
@@ -639,11 +821,9 @@ rc_status rc_frame_select(rc_bvh h, const float* d_P, const float* d_N, const in
             st = set_error(RC_E_CUDA, "memset failed");
             break;
         }
-        for (int c = 0; c < K && st == RC_OK; ++c) {
-            // each turned frame's axis rays walk the tree with boxes in its coordinates
-            if (n > 0) st = make_frame_tree(h, io->frame[c], p, &ftrees[c], s);
-            if (st == RC_OK) st = frame_setup_f(h, io->frame[c], fds + c, s, ftrees[c]);
-        }
+        // each turned frame's axis rays walk the tree with boxes in its coordinates
+        for (int c = 0; c < K && st == RC_OK && n > 0; ++c) st = make_frame_tree(h, io->frame[c], p, &ftrees[c], s);
+        if (st == RC_OK) st = frame_setups(h, io->frame, ftrees.data(), K, fds, s);
         if (st != RC_OK) break;
         if (n > 0) {
             st = launch_orthogonal_frames(h, d_P, d_N, n, p, fds, K, mask, trav, (unsigned long long*)d_counters, s);

@@ -78,10 +78,12 @@ constexpr int kAllTris = -2;       // wide-node child made of all triangles (par
 constexpr int kLeafChild = -3;     // wide-node child that is a leaf (its triangles are in its code)
 
 // machining frame on the device (Section 3.2)
-struct FrameArgs { float f[9]; const float4* tree; double sc_c[3]; double sc_r; };
+constexpr int kMaxFrames = 6;      // frames set up by one launch
+struct FrameArgs { float f[kMaxFrames][9]; const float4* tree[kMaxFrames]; double sc_c[3]; double sc_r; };
 struct FrameDev {
     float axes[18];     // +X', -X', +Y', -Y', +Z', -Z' (fp32)
-    float pad[2];
+    unsigned done;      // blocks of k_frame_box that have added their part
+    unsigned pad;
     double frame[9];    // row-major frame, FP64
     double fbox[6];     // frame-coordinate bounding box of the vertices (lo xyz, hi xyz)
     long long box[6];   // ordered-integer accumulators for fbox
@@ -116,6 +118,8 @@ struct BatchPart {
 // (nullptr: the world tree)
 rc_status frame_setup(rc_bvh h, const rc_params* p, FrameDev* d, cudaStream_t s, const float4* tree = nullptr);
 rc_status frame_setup_f(rc_bvh h, const float* f9, FrameDev* d, cudaStream_t s, const float4* tree = nullptr);
+rc_status frame_setups(rc_bvh h, const float (*f9)[9], const float4* const* trees, int nf, FrameDev* d, cudaStream_t s);
+int device_sms();                  // SMs of the current device
 // the 4-wide tree of h with its child boxes in the coordinates of frame f9
 // (ftree: as many nodes as h's 4-wide tree)
 rc_status frame_tree(rc_bvh h, const float f9[9], float4* ftree, cudaStream_t s);

@@ -127,7 +127,7 @@ __device__ __noinline__ DirSums exact_sums(const uint32_t* __restrict__ bits, fl
 //     at most W / 2 terms per half, then the halves and five shuffles.
 //   - Two directions per instruction (f32x2), from a table in shared memory
 //     whose entries are the pairs of words 2 p and 2 p + 1.
-// 300k points x 1000 directions, 70% visible: 729 -> 431 us.
+// 300k points x 1000 directions, 70% visible: 729 -> 467 us.
 // conc_mode 1 needs the sums themselves and takes the exact path per point.
 constexpr int kVarThreads = 256, kVarBlocks = 4;   // 3, 5 and 6 blocks per SM measured 6 to 9% slower
 constexpr int kVarTableWords = 96;     // most words of the shared table (36 KB); beyond, the table is read from L1
@@ -409,11 +409,21 @@ __global__ void k_fixture(const float* __restrict__ V, const int32_t* __restrict
                           const float* __restrict__ fnorm, int64_t T, const double* __restrict__ frame,
                           const double* __restrict__ fbox, uint8_t* fixture)
 {
-    int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    // the frame's constants once per block: formed by every thread, their
+    // FP64 took 16 us for 203k faces where the rest takes 8
+    __shared__ double s_tol;
+    __shared__ float s_f[9], s_b[6];
+    if (threadIdx.x < 9) s_f[threadIdx.x] = (float)frame[threadIdx.x];
+    if (threadIdx.x < 6) s_b[threadIdx.x] = (float)fbox[threadIdx.x];
+    if (threadIdx.x == 0) {
+        const double d0 = __dsub_rn(fbox[3], fbox[0]), d1 = __dsub_rn(fbox[4], fbox[1]), d2 = __dsub_rn(fbox[5], fbox[2]);
+        const double diag = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(d0, d0), __dmul_rn(d1, d1)), __dmul_rn(d2, d2)));
+        s_tol = __dmul_rn(1e-6, diag);
+    }
+    __syncthreads();
+    const int64_t f = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (f >= T) return;
-    const double d0 = __dsub_rn(fbox[3], fbox[0]), d1 = __dsub_rn(fbox[4], fbox[1]), d2 = __dsub_rn(fbox[5], fbox[2]);
-    const double diag = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(d0, d0), __dmul_rn(d1, d1)), __dmul_rn(d2, d2)));
-    const double tol = __dmul_rn(1e-6, diag);
+    const double tol = s_tol;
     const double lim = 1.0 - 1e-6;
     // fp32 pre-check.  The frame entries are fp32 values, so the fp32 frame
     // coordinate q of a vertex (three rounded operations) is within 3 u s of
@@ -425,8 +435,8 @@ __global__ void k_fixture(const float* __restrict__ V, const int32_t* __restrict
     const float tolf = (float)tol;
     bool fx = false;
     for (int k = 0; k < 3; ++k) {
-        const float f0 = (float)frame[k], f1 = (float)frame[3 + k], f2 = (float)frame[6 + k];
-        const float blo = (float)fbox[k], bhi = (float)fbox[3 + k];
+        const float f0 = s_f[k], f1 = s_f[3 + k], f2 = s_f[6 + k];
+        const float blo = s_b[k], bhi = s_b[3 + k];
         bool near_lo = true, near_hi = true;
         for (int a = 0; a < 3; ++a) {
             const int64_t v = F[3 * f + a];
