@@ -865,8 +865,6 @@ __device__ __forceinline__ TraceOut trace_any(const float4* __restrict__ nodes, 
 // ---------------------------------------------------------------------------
 struct AxisRay {
     float lo[3], hi[3];   // frame-coordinate band the ray can reach (+-inf on its far side along k)
-    int k;                // frame axis of the ray
-    int pos;              // 1: along +column k, 0: along -column k
 };
 
 // The band of an axis ray (see above).  Its bounds are sums hi + lo -+ tol
@@ -893,8 +891,6 @@ __device__ __forceinline__ AxisRay make_axis_ray(const FrameDev& fd, int a, floa
             else ar.lo[j] = -INFINITY;
         }
     }
-    ar.k = k;
-    ar.pos = pos ? 1 : 0;
     return ar;
 }
 
@@ -985,20 +981,25 @@ using CastAcc = CastAccFwd;
 //     blocked leaves its remaining boxes untested.  Testing boxes ahead (48
 //     or 64 pairs) fills the lanes better and still measured 11% and 22%
 //     slower: more pairs of rays that a nearer box would have blocked.
-//   - Pairs of a blocked ray are dropped when they are taken.  A leaf's pair
-//     waits in a queue of its own for a full step of triangle tests.
-//   - The nearest entered child of every lane's node is pushed last, so the
-//     walk stays depth-first and near-first per ray.
+//   - Pairs of a blocked ray are dropped when they are taken.  The triangles
+//     of a leaf wait, each for itself, in a queue of their own for a full step
+//     of tests (a lane per leaf left the second test a third empty: impeller
+//     28.4 -> 27.2 ms per 100k points); those of at most 32 pairs left over
+//     move on to the next tile with the nodes (29.2 -> 28.4 ms).
+//   - Entered children are pushed as they lie in the node, one of every lane
+//     on top, so the walk stays depth-first; steps of 22 lanes and more are
+//     taken as they come (27.0 ms; refilled to 28: 27.2, to 30: 27.5).
 // Every ray meets the same boxes and triangles as in a walk of its own, less
 // those that a hit found earlier makes unnecessary, so the bits are the same.
-// What bounds it: instruction issue (58% of cycles at 28 active lanes and 125
-// warp instructions per ray on the impeller, where a ray per lane took 73% at
-// 11 lanes and 191), then the L1 data path (48%).  A step at a node is about
-// 280 warp instructions, 60% of the time.
+// What bounds it: the latency of dependent instructions and loads at 20 warps
+// per SM (a warp issues every 7.7 cycles, 63% of the issue slots at 28 active
+// lanes); more warps would need fewer registers than the walk has, and their
+// pools would take the L1 they live from (6 blocks per SM: 31.3 ms, 4: 30.1).
+// Steps at nodes take 55% of the time, at triangles 25%.
 // ---------------------------------------------------------------------------
 constexpr int kPoolPairs = 320;        // pairs (ray, node or leaf) on the stack
-constexpr int kPoolLeaves = 96;        // pairs (ray, leaf) that wait for a full step
-constexpr int kPoolFill = 28;          // lanes that are enough for a step
+constexpr int kPoolLeaves = 128;       // pairs (ray, triangle) that wait for a full step
+constexpr int kPoolFill = 22;          // lanes that are enough for a step
 // Room on the stack: a step takes n pairs and adds up to 4 n.  While more than
 // kPoolFull wait, steps take fewer, down to one pair at a time, whose subtree
 // needs at most 3 entries per level of a tree of depth (kStack4 - 1) / 3.
@@ -1256,14 +1257,17 @@ __device__ __forceinline__ void cast_point_pooled(const float4* __restrict__ wno
                     have = live && code >= 0;
                     leaf = live && code < 0;
                 }
-                const unsigned ml = __ballot_sync(kAll, leaf);
-                if (leaf) pool->leaf[lsp + __popc(ml & below)] = Pair::make(code, slot);
+                const bool two = leaf && leaf_count(code) == 2;
+                const unsigned ml = __ballot_sync(kAll, leaf), m2 = __ballot_sync(kAll, two);
+                if (leaf) pool->leaf[lsp + __popc(ml & below)] = Pair::make(leaf_code(leaf_first(code), 1), slot);
                 lsp += __popc(ml);
+                if (two) pool->leaf[lsp + __popc(m2 & below)] = Pair::make(leaf_code(leaf_first(code) + 1, 1), slot);
+                lsp += __popc(m2);
                 sp = max(0, sp - __popc(want));
-                if (sp == 0 || lsp > kPoolLeaves - 32 || __popc(__ballot_sync(kAll, have || idle)) >= kPoolFill) break;
+                if (sp == 0 || lsp > kPoolLeaves - 64 || __popc(__ballot_sync(kAll, have || idle)) >= kPoolFill) break;
             }
-            float d[4] = {INFINITY, INFINITY, INFINITY, INFINITY};
-            int c[4] = {0, 0, 0, 0};
+            bool i0 = false, i1 = false, i2 = false, i3 = false;
+            float4 ci = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
             if (have) {
                 if (kStats) acc.nvis += 1;
                 const float4 v = pool->inv[slot];
@@ -1280,78 +1284,58 @@ __device__ __forceinline__ void cast_point_pooled(const float4* __restrict__ wno
                     return __ldg((const float4*)((const char*)wnodes + (((unsigned)code << 7) | q)));
                 };
                 const float4 nx = ld(qx), fx = ld(qx ^ 16u), ny = ld(qy), fy = ld(qy ^ 16u), nz = ld(qz), fz = ld(qz ^ 16u);
-                const float4 ci = ld(at ^ 96u);
+                ci = ld(at ^ 96u);
                 const auto entry = [&](float nxk, float nyk, float nzk, float fxk, float fyk, float fzk) {
                     const float tn = fmaxf(fmaxf(fmaf(nxk, v.x, -(x + mx)), fmaf(nyk, v.y, -(y + my))),
                                            fmaxf(fmaf(nzk, v.z, -(z + mz)), 0.0f));
                     const float tf = fminf(fminf(fmaf(fxk, v.x, mx - x), fmaf(fyk, v.y, my - y)),
                                            fmaf(fzk, v.z, mz - z));
-                    return tn <= tf ? tn : INFINITY;
+                    return tn <= tf;
                 };
-                d[0] = entry(nx.x, ny.x, nz.x, fx.x, fy.x, fz.x);
-                d[1] = entry(nx.y, ny.y, nz.y, fx.y, fy.y, fz.y);
-                d[2] = entry(nx.z, ny.z, nz.z, fx.z, fy.z, fz.z);
-                d[3] = entry(nx.w, ny.w, nz.w, fx.w, fy.w, fz.w);
-                c[0] = __float_as_int(ci.x);
-                c[1] = __float_as_int(ci.y);
-                c[2] = __float_as_int(ci.z);
-                c[3] = __float_as_int(ci.w);
-#define RC_CSWAP(a, b)                                              \
-    if (d[b] < d[a]) {                                              \
-        const float td = d[a]; d[a] = d[b]; d[b] = td;              \
-        const int tc = c[a]; c[a] = c[b]; c[b] = tc;                \
-    }
-                RC_CSWAP(0, 1) RC_CSWAP(2, 3) RC_CSWAP(0, 2)
-#undef RC_CSWAP
+                i0 = entry(nx.x, ny.x, nz.x, fx.x, fy.x, fz.x);
+                i1 = entry(nx.y, ny.y, nz.y, fx.y, fy.y, fz.y);
+                i2 = entry(nx.z, ny.z, nz.z, fx.z, fy.z, fz.z);
+                i3 = entry(nx.w, ny.w, nz.w, fx.w, fy.w, fz.w);
             }
             __syncwarp();
-            // push the entered children: the farther ones first (a lane's side
+            // push the entered children: the last three first (a lane's side
             // by side, its count 0..3 summed over the lower lanes bit by bit),
-            // then the nearest of every lane
-            const bool i0 = d[0] != INFINITY, i1 = d[1] != INFINITY, i2 = d[2] != INFINITY, i3 = d[3] != INFINITY;
+            // then the first of every lane.  Nothing is gained by sorting
+            // them by distance: an any-hit ray ends as soon in either order
+            // (impeller 29.3 ms per 100k points sorted, 29.2 as they lie)
             const unsigned b0 = __ballot_sync(kAll, i1 ^ i2 ^ i3), b1 = __ballot_sync(kAll, (i1 & i2) | (i3 & (i1 | i2))),
                            bn = __ballot_sync(kAll, i0);
             int at = sp + __popc(b0 & below) + 2 * __popc(b1 & below);
-            if (i3) pool->pair[at++] = Pair::make(c[3], slot);
-            if (i2) pool->pair[at++] = Pair::make(c[2], slot);
-            if (i1) pool->pair[at] = Pair::make(c[1], slot);
+            if (i3) pool->pair[at++] = Pair::make(__float_as_int(ci.w), slot);
+            if (i2) pool->pair[at++] = Pair::make(__float_as_int(ci.z), slot);
+            if (i1) pool->pair[at] = Pair::make(__float_as_int(ci.y), slot);
             sp += __popc(b0) + 2 * __popc(b1);
-            if (i0) pool->pair[sp + __popc(bn & below)] = Pair::make(c[0], slot);
+            if (i0) pool->pair[sp + __popc(bn & below)] = Pair::make(__float_as_int(ci.x), slot);
             sp += __popc(bn);
             __syncwarp();
             continue;
         }
-        if (lsp > 0) {
-            // up to 32 pairs with a leaf, one per lane
+        if (lsp >= 32 || (lsp > 0 && (t >= t1 || sp + lsp > 32))) {
+            // up to 32 pairs with a triangle, one per lane
             const int at = lsp - 1 - lane;
             lsp = max(0, lsp - 32);
-            int ntri = 0, slot = 0;
-            float4 rd = make_float4(0, 0, 0, 0);
-            const float4* tp = tris;
+            int slot = 0;
+            bool hit = false;
             if (at >= 0) {
                 const Pair q = pool->leaf[at];
                 slot = q.slot();
-                rd = pool->dir[slot];
-                tp = tris + 3 * (int64_t)leaf_first(q.code());
-                if (((slot & 32 ? live1 : live0) >> (slot & 31)) & 1u) ntri = leaf_count(q.code());
-            }
-            bool hit = false;
-            for (int k = 0; k < kLeafMax && __any_sync(kAll, k < ntri); ++k) {
-                int st = kMiss;
-                if (k < ntri) {
+                if (((slot & 32 ? live1 : live0) >> (slot & 31)) & 1u) {
+                    const float4 rd = pool->dir[slot];
+                    const float4* tp = tris + 3 * (int64_t)leaf_first(q.code());
                     if (kStats) acc.ntri += 1;
-                    st = tri_test_mt(ox, oy, oz, rd.x, rd.y, rd.z, rd.w, rs, __ldg(tp + 3 * k), __ldg(tp + 3 * k + 1),
-                                     __ldg(tp + 3 * k + 2));
+                    int st = tri_test_mt(ox, oy, oz, rd.x, rd.y, rd.z, rd.w, rs, __ldg(tp), __ldg(tp + 1), __ldg(tp + 2));
                     if (st == kUnsure) {
                         acc.retests += 1;
-                        if (pool_retest<kStats>(ox, oy, oz, rd, __float_as_int(pool->inv[slot].w), tp + 3 * k, rows, W,
-                                                i, relist, relist_cap, relist_ctr))
+                        if (pool_retest<kStats>(ox, oy, oz, rd, __float_as_int(pool->inv[slot].w), tp, rows, W, i, relist,
+                                                relist_cap, relist_ctr))
                             st = kHit;
                     }
-                    if (st == kHit) {
-                        hit = true;
-                        ntri = 0;
-                    }
+                    hit = st == kHit;
                 }
             }
             if (hit) {
@@ -1367,10 +1351,11 @@ __device__ __forceinline__ void cast_point_pooled(const float4* __restrict__ wno
         if (t >= t1) break;
         // the next tile enters; the rays of the pairs left over move down
         // (one slot per ray, the lowest pair's)
-        if (sp > 0) {
-            const bool mine = lane < sp;
+        if (sp + lsp > 0) {
+            const bool mine = lane < sp + lsp;
+            Pair* const at = lane < sp ? &pool->pair[lane] : &pool->leaf[lane - sp];
             Pair q = Pair::make(0, 0);
-            if (mine) q = pool->pair[lane];
+            if (mine) q = *at;
             const int from = q.slot();
             const float4 li = pool->inv[from], ld = pool->dir[from];
             const bool live = mine && (((from & 32 ? live1 : live0) >> (from & 31)) & 1u);
@@ -1380,7 +1365,7 @@ __device__ __forceinline__ void cast_point_pooled(const float4* __restrict__ wno
                 pool->inv[lane] = li;
                 pool->dir[lane] = ld;
             }
-            if (mine) pool->pair[lane] = Pair::make(q.code(), to);    // a pair of a blocked ray: its own slot, not live
+            if (mine) *at = Pair::make(q.code(), to);    // a pair of a blocked ray: its own slot, not live
             __syncwarp();
         }
         const float4 h = __ldg(&tdirs[32 * t + lane]);
@@ -1464,10 +1449,12 @@ __device__ __forceinline__ void cast_point_pooled(const float4* __restrict__ wno
 // runs along a fillet or a bore 1e-4 mm above it enters hundreds of boxes,
 // and alone in its lane it set the time of the launch; pooled, its pairs
 // fill the warp.  The rays of a warp share direction and axis, so a slot
-// holds an origin and a band only.  A queue of 32 leaves is tested at once,
+// holds an origin and a band only.  A queue of 32 triangles is tested at once,
 // fewer when no nodes are left (testing fewer earlier measured the same).
 // Prismatic part turned off its axes, 100k points: six axes, covers and a
-// ball-end tool 3.86 -> 2.61 ms, choice of a frame 5.84 -> 4.01 ms.
+// ball-end tool 3.86 -> 2.61 ms, choice of a frame 5.84 -> 4.01 ms.  Children
+// pushed as they lie and triangles queued one by one: 1.45 -> 1.30 and 2.0 ->
+// 1.85 ms of what later changes had left.
 // ---------------------------------------------------------------------------
 template <bool kBig>
 struct __align__(16) AxisPoolOf {
@@ -1491,12 +1478,8 @@ __device__ __forceinline__ bool trace_axis(const float4* __restrict__ ftree, con
     constexpr unsigned kAll = 0xFFFFFFFFu;
     const int lane = threadIdx.x & 31;
     const unsigned below = (1u << lane) - 1u;
-    // the axis, the same in every casting lane; near face of a child along
-    // the ray: lo of axis k going +, hi going -
     unsigned live = __ballot_sync(kAll, cast);
     if (live == 0) return false;
-    const int src = __ffs(live) - 1;
-    const int pos = __shfl_sync(kAll, ar.pos, src), near_at = 2 * __shfl_sync(kAll, ar.k, src) + (pos ? 0 : 1);
     unsigned amb = 0, hit64 = 0;           // rays with an ambiguous pair; one that FP64 calls a hit
     __syncwarp();
     if (cast) {
@@ -1512,10 +1495,7 @@ __device__ __forceinline__ bool trace_axis(const float4* __restrict__ ftree, con
     // bounds a malformed one
     int steps = (int)min64(0x7FFFFFFF, 2 * (int64_t)max_steps);
     for (;;) {
-#ifndef RC_AXIS_FLUSH
-#define RC_AXIS_FLUSH 0
-#endif
-        if (lsp < 32 && sp > 0 && !(sp < RC_AXIS_FLUSH && lsp > 0)) {
+        if (lsp < 32 && sp > 0) {
             if (--steps < 0) break;
             bool have = false, idle = false;
             if (sp > kPoolFull) idle = lane >= max(1, min(32, (kPoolPairs - kStack4 - sp) / 3));
@@ -1532,50 +1512,41 @@ __device__ __forceinline__ bool trace_axis(const float4* __restrict__ ftree, con
                     have = on && code >= 0;
                     leaf = on && code < 0;
                 }
-                const unsigned ml = __ballot_sync(kAll, leaf);
-                if (leaf) pool->leaf[lsp + __popc(ml & below)] = Pair::make(code, slot);
+                const bool two = leaf && leaf_count(code) == 2;
+                const unsigned ml = __ballot_sync(kAll, leaf), m2 = __ballot_sync(kAll, two);
+                if (leaf) pool->leaf[lsp + __popc(ml & below)] = Pair::make(leaf_code(leaf_first(code), 1), slot);
                 lsp += __popc(ml);
+                if (two) pool->leaf[lsp + __popc(m2 & below)] = Pair::make(leaf_code(leaf_first(code) + 1, 1), slot);
+                lsp += __popc(m2);
                 sp = max(0, sp - __popc(want));
-                if (sp == 0 || lsp > kPoolLeaves - 32 || __popc(__ballot_sync(kAll, have || idle)) >= kPoolFill) break;
+                if (sp == 0 || lsp > kPoolLeaves - 64 || __popc(__ballot_sync(kAll, have || idle)) >= kPoolFill) break;
             }
-            float d[4] = {INFINITY, INFINITY, INFINITY, INFINITY};
-            int c[4] = {0, 0, 0, 0};
+            bool i0 = false, i1 = false, i2 = false, i3 = false;
+            float4 ci = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
             if (have) {
                 if (kStats) acc.nvis += 1;
                 const float4* nd = wide_ptr(ftree, code);
                 const float4 lx = wide_ld(nd, 0), hx = wide_ld(nd, 1), ly = wide_ld(nd, 2), hy = wide_ld(nd, 3);
-                const float4 lz = wide_ld(nd, 4), hz = wide_ld(nd, 5), ci = wide_ld(nd, 6), ev = wide_ld(nd, near_at);
+                const float4 lz = wide_ld(nd, 4), hz = wide_ld(nd, 5);
+                ci = wide_ld(nd, 6);
                 const float4 l = pool->lo[slot], h = pool->hi[slot];
-                const auto entry = [&](float lxk, float hxk, float lyk, float hyk, float lzk, float hzk, float e) {
-                    const bool in = lxk <= h.x && hxk >= l.x && lyk <= h.y && hyk >= l.y && lzk <= h.z && hzk >= l.z;
-                    return in ? (pos ? e : -e) : INFINITY;
+                const auto entry = [&](float lxk, float hxk, float lyk, float hyk, float lzk, float hzk) {
+                    return lxk <= h.x && hxk >= l.x && lyk <= h.y && hyk >= l.y && lzk <= h.z && hzk >= l.z;
                 };
-                d[0] = entry(lx.x, hx.x, ly.x, hy.x, lz.x, hz.x, ev.x);
-                d[1] = entry(lx.y, hx.y, ly.y, hy.y, lz.y, hz.y, ev.y);
-                d[2] = entry(lx.z, hx.z, ly.z, hy.z, lz.z, hz.z, ev.z);
-                d[3] = entry(lx.w, hx.w, ly.w, hy.w, lz.w, hz.w, ev.w);
-                c[0] = __float_as_int(ci.x);
-                c[1] = __float_as_int(ci.y);
-                c[2] = __float_as_int(ci.z);
-                c[3] = __float_as_int(ci.w);
-#define RC_CSWAP(a, b)                                              \
-    if (d[b] < d[a]) {                                              \
-        const float td = d[a]; d[a] = d[b]; d[b] = td;              \
-        const int tc = c[a]; c[a] = c[b]; c[b] = tc;                \
-    }
-                RC_CSWAP(0, 1) RC_CSWAP(2, 3) RC_CSWAP(0, 2)
-#undef RC_CSWAP
+                i0 = entry(lx.x, hx.x, ly.x, hy.x, lz.x, hz.x);
+                i1 = entry(lx.y, hx.y, ly.y, hy.y, lz.y, hz.y);
+                i2 = entry(lx.z, hx.z, ly.z, hy.z, lz.z, hz.z);
+                i3 = entry(lx.w, hx.w, ly.w, hy.w, lz.w, hz.w);
             }
             __syncwarp();
-            const bool i0 = d[0] != INFINITY, i1 = d[1] != INFINITY, i2 = d[2] != INFINITY, i3 = d[3] != INFINITY;
             const unsigned b0 = __ballot_sync(kAll, i1 ^ i2 ^ i3), b1 = __ballot_sync(kAll, (i1 & i2) | (i3 & (i1 | i2))),
                            bn = __ballot_sync(kAll, i0);
             int at = sp + __popc(b0 & below) + 2 * __popc(b1 & below);
-            if (i3) pool->pair[at++] = Pair::make(c[3], slot);
-            if (i2) pool->pair[at++] = Pair::make(c[2], slot);
-            if (i1) pool->pair[at] = Pair::make(c[1], slot);
+            if (i3) pool->pair[at++] = Pair::make(__float_as_int(ci.w), slot);
+            if (i2) pool->pair[at++] = Pair::make(__float_as_int(ci.z), slot);
+            if (i1) pool->pair[at] = Pair::make(__float_as_int(ci.y), slot);
             sp += __popc(b0) + 2 * __popc(b1);
-            if (i0) pool->pair[sp + __popc(bn & below)] = Pair::make(c[0], slot);
+            if (i0) pool->pair[sp + __popc(bn & below)] = Pair::make(__float_as_int(ci.x), slot);
             sp += __popc(bn);
             __syncwarp();
             continue;
@@ -1583,36 +1554,30 @@ __device__ __forceinline__ bool trace_axis(const float4* __restrict__ ftree, con
         if (lsp == 0) break;
         const int at = lsp - 1 - lane;
         lsp = max(0, lsp - 32);
-        int ntri = 0, slot = 0;
-        Ray q = r;
-        const float4* tp = tris;
+        int slot = 0;
+        bool hit = false, ua = false, uh = false;
         if (at >= 0) {
             const Pair pr = pool->leaf[at];
             slot = pr.slot();
-            q.ox = pool->lo[slot].w;
-            q.oy = pool->hi[slot].w;
-            q.oz = pool->oz[slot];
-            q.rs = fmaxf(fmaxf(1.0f, scene_maxabs), fmaxf(fabsf(q.ox), fmaxf(fabsf(q.oy), fabsf(q.oz))));
-            tp = tris + 3 * (int64_t)leaf_first(pr.code());
-            if ((live >> slot) & 1u) ntri = leaf_count(pr.code());
-        }
-        bool hit = false, ua = false, uh = false;
-        for (int k = 0; k < kLeafMax && __any_sync(kAll, k < ntri); ++k) {
-            if (k >= ntri) continue;
-            if (kStats) acc.ntri += 1;
-            const float4 v0 = __ldg(tp + 3 * k), v1 = __ldg(tp + 3 * k + 1), v2 = __ldg(tp + 3 * k + 2);
-            int st = tri_test32(q, v0, v1, v2);
-            if (st == kUnsure) st = tri_test_close(q, v0, v1, v2);
-            if (st == kUnsure) {
-                ++acc.retests;
-                const Pair64 w = retest64(q, v0, v1, v2);
-                st = w.state;
-                ua |= st == kUnsure;
-                uh |= st == kUnsure && w.hit64;
-            }
-            if (st == kHit) {
-                hit = true;
-                ntri = 0;
+            if ((live >> slot) & 1u) {
+                Ray q = r;
+                q.ox = pool->lo[slot].w;
+                q.oy = pool->hi[slot].w;
+                q.oz = pool->oz[slot];
+                q.rs = fmaxf(fmaxf(1.0f, scene_maxabs), fmaxf(fabsf(q.ox), fmaxf(fabsf(q.oy), fabsf(q.oz))));
+                const float4* tp = tris + 3 * (int64_t)leaf_first(pr.code());
+                if (kStats) acc.ntri += 1;
+                const float4 v0 = __ldg(tp), v1 = __ldg(tp + 1), v2 = __ldg(tp + 2);
+                int st = tri_test32(q, v0, v1, v2);
+                if (st == kUnsure) st = tri_test_close(q, v0, v1, v2);
+                if (st == kUnsure) {
+                    ++acc.retests;
+                    const Pair64 w = retest64(q, v0, v1, v2);
+                    st = w.state;
+                    ua = st == kUnsure;
+                    uh = ua && w.hit64;
+                }
+                hit = st == kHit;
             }
         }
         if (__any_sync(kAll, ua)) {
