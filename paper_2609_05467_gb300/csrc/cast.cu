@@ -2411,10 +2411,6 @@ rc_status launch_hemisphere(rc_bvh h, const float* P, const float* N, int64_t n,
     const int threads = 128;
     const int per_sm = p->blocks_per_sm > 0 ? p->blocks_per_sm : RC_HEMI_MIN_BLOCKS;
     int64_t blocks = (int64_t)sm_count() * per_sm;
-    const int64_t need = (n * 32 + threads - 1) / threads;
-    if (blocks > need || p->launch_mode == 1) blocks = need;
-    if (blocks < 1) blocks = 1;
-    if (blocks > 0x7FFFFFFF) return set_error(RC_E_UNSUPPORTED, "too many points for one launch");
     if (p->launch_mode == 1) work = nullptr;
     const bool wide = use_wide(p);
     const int kind = cast_kind(p, h->T);
@@ -2423,17 +2419,22 @@ rc_status launch_hemisphere(rc_bvh h, const float* P, const float* N, int64_t n,
     {
         // the last points (RC_TAIL_POINTS per resident warp) are cast in parts;
         // with a grid sized to the work (one item per warp) the parts are the
-        // highest blocks, which the block scheduler starts last
+        // highest blocks, which the block scheduler starts last.  Few points
+        // go out in more parts, down to a tile each, until there are two per
+        // resident warp, although each part finds its frontier anew (37
+        // points x 2048 directions in 4, 16, 32 and 64 parts: 365, 187, 137
+        // and 117 us; 200 points in 4, 15, 30: 367, 207, 192; 1,000 x 1024
+        // in 4, 6: 275, 268; from 1,500 points on four parts fill the
+        // chip).  Not for a grid sized to the work, which shares the GPU.
         const int W = (p->n_dirs + 31) / 32;
         const int64_t resident_warps = (int64_t)sm_count() * per_sm * (threads / 32);
         int splits = std::min(RC_TAIL_SPLITS, W);
+        if (work && n > 0) splits = (int)std::max<int64_t>(splits, std::min<int64_t>(2 * resident_warps / n, W));
         int64_t n_split = splits > 1 ? std::min<int64_t>(n, RC_TAIL_POINTS * resident_warps) : 0;
         if (n_split == 0) splits = 1;
-        if (!work) {
-            const int64_t items = (n - n_split) + n_split * splits;
-            blocks = std::max<int64_t>(1, (items * 32 + threads - 1) / threads);
-            if (blocks > 0x7FFFFFFF) return set_error(RC_E_UNSUPPORTED, "too many points for one launch");
-        }
+        const int64_t need = std::max<int64_t>(1, (((n - n_split) + n_split * splits) * 32 + threads - 1) / threads);
+        if (!work && need > 0x7FFFFFFF) return set_error(RC_E_UNSUPPORTED, "too many points for one launch");
+        if (!work || blocks > need) blocks = need;
         if (n_split > 0) {
             k_zero_split<<<(unsigned)((n_split * W + 255) / 256), 256, 0, s>>>(order, n - n_split, n, W, bits, count);
             RC_LAUNCHED();

@@ -131,3 +131,20 @@ def test_batch_of_mixed_parts_equals_single_casts():
         assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
         bvh.close()
     rc.rc_batch_destroy(b)
+
+
+@pytest.mark.parametrize("n,dirs", [(1, 33), (1, 2048), (5, 257), (37, 1000), (200, 2048), (1500, 96), (1600, 96)])
+def test_few_points_in_parts_equal_the_same_points_among_many(n, dirs):
+    """Few points are cast in parts of a tile or more: their rows and counts are those they get in a large set."""
+    import paper_2609_05467_gb300 as rc
+    V, F = _soup(3000, 1.0, n)
+    rng = np.random.default_rng(dirs)
+    P = rng.uniform(0, 10, (8000, 3)).astype(np.float32)
+    N = rng.normal(size=(8000, 3))
+    N = (N / np.linalg.norm(N, axis=1, keepdims=True)).astype(np.float32)
+    bvh = rc.Bvh(*gpu_mesh(V, F))
+    p = rc.rc_params_default(n_dirs=dirs)
+    many, few = gpu_cast(rc, bvh.h, P, N, p), gpu_cast(rc, bvh.h, P[:n], N[:n], p)
+    assert np.array_equal(many[0][:n], few[0]) and np.array_equal(many[1][:n], few[1])
+    assert few[2][0] == n * dirs
+    bvh.close()
