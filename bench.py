@@ -507,8 +507,8 @@ def roofline(rc, args, name, dev, stream, ps, cast_s, rays, nodes_per_ray, tris_
         "peak_source": "unit counts and clocks: %d SMs x 128 FP32 lanes x 2 flop x %.0f MHz"
                        % (props.multi_processor_count, sm_max),
         "kernel": "k_hemisphere", "kernel_ms": 1e3 * cast_s,
-        "binding": "instruction issue of a divergent walk whose dependent fetch -> test -> stack chain is "
-                   "latency-bound; no bandwidth binds (see levels)",
+        "binding": "latency of dependent instructions and loads of the pooled walk at 20 warps per SM; no bandwidth "
+                   "binds (see levels)",
         "algorithmic": {"ops_per_ray": ops_per_ray, "bytes_per_ray": bytes_per_ray, "nodes_per_ray": nodes_per_ray,
                         "tris_per_ray": tris_per_ray, "node_bytes": node_bytes,
                         "tree": "4-wide" if ps.tree_width != 2 else "binary",
