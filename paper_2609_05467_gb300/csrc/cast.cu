@@ -529,22 +529,40 @@ struct Frontier {
 // n . (v - o) < 0 for the three vertices, in FP64: the differences of fp32
 // values are exact there and the products and sums round far below the
 // margin taken (4e-15 of the sum of the terms' magnitudes)
-__device__ __forceinline__ bool below_tangent(float4 v, float ox, float oy, float oz, float nx, float ny, float nz)
+__device__ __noinline__ bool below_tangent64(float x, float y, float z, float ox, float oy, float oz, float nx, float ny, float nz)
 {
-    const double a = (double)v.x - ox, b = (double)v.y - oy, c = (double)v.z - oz;
+    const double a = (double)x - ox, b = (double)y - oy, c = (double)z - oz;
     const double s = __dadd_rn(__dadd_rn(__dmul_rn((double)nx, a), __dmul_rn((double)ny, b)), __dmul_rn((double)nz, c));
     const double m = fabs((double)nx * a) + fabs((double)ny * b) + fabs((double)nz * c);
     return s < -4e-15 * m;
+}
+
+// the same, decided in fp32 where the sign is clear (each difference, product
+// and sum rounds once: under 4u of the sum of the terms' magnitudes, 8u taken)
+__device__ __forceinline__ bool below_tangent(float4 v, float ox, float oy, float oz, float nx, float ny, float nz)
+{
+    const float a = (v.x - ox) * nx, b = (v.y - oy) * ny, c = (v.z - oz) * nz;
+    const float s = a + b + c, e = 8.0f * 5.9604644775390625e-8f * (fabsf(a) + fabsf(b) + fabsf(c)) + 1e-36f;
+    if (fabsf(s) > e && e < 1e30f) return s < 0.0f;
+    return below_tangent64(v.x, v.y, v.z, ox, oy, oz, nx, ny, nz);
 }
 
 // Shortcuts that skip what lies below a point's tangent plane need every
 // direction of the set above it.  With |n|^2 = 1 + delta the basis tilts by
 // about |delta|, so d.n >= z_min - 3 |delta| - 1e-6 with z_min = 1/(2N) >=
 // 1/(64 W) (W = ceil(N/32)); a normal further from unit length takes none.
-__device__ __forceinline__ bool tangent_shortcuts_ok(float nx, float ny, float nz, int W)
+// In fp32 where the comparison is clear by 1e-6 (rounding: 3u nn and less).
+__device__ __noinline__ bool tangent_shortcuts_ok64(float nx, float ny, float nz, int W)
 {
     const double nn = (double)nx * nx + (double)ny * ny + (double)nz * nz;
     return fabs(nn - 1.0) <= 0.25 * (1.0 / (64.0 * W) - 2e-6);
+}
+
+__device__ __forceinline__ bool tangent_shortcuts_ok(float nx, float ny, float nz, int W)
+{
+    const float off = fabsf(nx * nx + ny * ny + nz * nz - 1.0f) - (__fdividef(0.25f, 64.0f * (float)W) - 5e-7f);
+    if (fabsf(off) > 1e-6f && off < 1.0f) return off < 0.0f;
+    return tangent_shortcuts_ok64(nx, ny, nz, W);
 }
 
 // A box wholly below the tangent plane through o: the largest n.(x - o) over

@@ -148,3 +148,26 @@ def test_few_points_in_parts_equal_the_same_points_among_many(n, dirs):
     assert np.array_equal(many[0][:n], few[0]) and np.array_equal(many[1][:n], few[1])
     assert few[2][0] == n * dirs
     bvh.close()
+
+
+@pytest.mark.parametrize("dirs", [33, 600, 2048])
+def test_normals_at_the_gate_of_the_tangent_shortcuts(dirs):
+    """Normals whose squared length differs from one by the bound of the tangent shortcuts, a little less and a little more:
+    bits equal the binary walk's and the oracle's, also for points on the surface and on its vertices."""
+    import paper_2609_05467_gb300 as rc
+    V, F = synth.icosphere(10.0, 2)
+    V = np.concatenate([V, 0.6 * V]).astype(np.float32)
+    F = np.concatenate([F, F[:, ::-1] + len(V) // 2]).astype(np.int32)
+    gate = 0.25 * (1.0 / (64.0 * ((dirs + 31) // 32)) - 2e-6)
+    P, N, _, _ = oracle.sample_centroid(V, F)
+    rng = np.random.default_rng(dirs)
+    pick = rng.choice(len(P), 120, replace=False)
+    P, N = P[pick], N[pick].astype(np.float64)
+    P[::3] = V[F[pick[::3], 0]]                              # on a vertex: planes through the origin's neighbourhood
+    d = gate * rng.choice([-1, 1], 120) * (1.0 + rng.choice([-1e-2, -1e-4, 0.0, 1e-4, 1e-2], 120))
+    N = (N * np.sqrt(1.0 + d)[:, None]).astype(np.float32)
+    bvh = rc.Bvh(*gpu_mesh(V, F))
+    g = _both(bvh.h, P, N, dirs)
+    ob, oa, oc = oracle.Mesh(V, F).hemisphere(P, N, dirs)
+    compare_bits(g[0], g[1], ob, oa, oc, dirs)
+    bvh.close()
