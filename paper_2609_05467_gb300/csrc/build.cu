@@ -7,11 +7,13 @@
 //   morton      : 48-bit Morton code of each face-box centre (16 bits per axis)
 //   radix sort  : 6 passes of 8-bit LSD (histogram / scan / stable scatter)
 //   karras      : binary radix tree over the sorted codes (Karras, HPG 2012)
-//   refit       : bottom-up boxes with arrival counters
-//   pack        : BVH2 nodes holding both child boxes (64 B), leaves of up
-//                 to kLeafMax consecutive triangles, triangle records 48 B
-//   wide        : top-down collapse into 4-wide nodes (128 B): the top
-//                 levels one launch each, the subtrees below depth-first
+//   refit       : triangle records (48 B), boxes bottom-up and BVH2 nodes
+//                 holding both child boxes (64 B, leaves of up to kLeafMax
+//                 consecutive triangles) in one launch: within a block in
+//                 shared memory, across blocks by arrival counters
+//   wide        : top-down collapse into 4-wide nodes (128 B): six levels in
+//                 one block, further ones a launch each, the subtrees below
+//                 depth-first
 //   area cdf    : 2^32-quantised face areas, inclusive int64 prefix
 #include <math.h>
 #include <stdio.h>

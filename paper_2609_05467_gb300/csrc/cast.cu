@@ -1,8 +1,9 @@
 // cast.cu -- any-hit occlusion traversal (Section 3.1 hemispherical cast,
 // Section 3.2 orthogonal cast).
 //
-// Each ray/triangle pair is first decided in FP32 with the watertight test
-// of Woop, Benthin and Wald (JCGT 2013) together with a forward error bound
+// Each ray/triangle pair is first decided in FP32: by signed volumes in the
+// pooled hemispherical walk (tri_test_mt), elsewhere with the watertight test
+// of Woop, Benthin and Wald (JCGT 2013), together with a forward error bound
 // on its edge functions U, V, W, on det = U+V+W and on the unscaled
 // plane-crossing value T' = U*az + V*bz + W*cz (see tri_test32).  The FP32
 // outcome is accepted only when it is certain -- a clear hit outside the
