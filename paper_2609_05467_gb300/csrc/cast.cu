@@ -1380,6 +1380,7 @@ __device__ __forceinline__ void cast_point_pooled(const float4* __restrict__ wno
             const bool live = mine && (((from & 32 ? live1 : live0) >> (from & 31)) & 1u);
             const int to = __ffs(__match_any_sync(kAll, live ? __float_as_int(li.w) : -1 - lane)) - 1;
             live0 = __ballot_sync(kAll, live && to == lane);
+            __syncwarp();                  // every slot is read before one is written
             if (live && to == lane) {
                 pool->inv[lane] = li;
                 pool->dir[lane] = ld;
