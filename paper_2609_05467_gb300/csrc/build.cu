@@ -780,8 +780,8 @@ __device__ __forceinline__ bool gather_tri(const float* __restrict__ V, int64_t 
 // first one's box and both heights, and goes on.  A node whose leaves all
 // belong to one block (255 of 256 do) meets in shared memory, at the place of
 // its split (the last leaf of its left subtree, which no other node has).
-// The others meet in global memory: a fence, an exchange and a read back, a
-// microsecond or two per level; that chain bounds a small tree, and the boxes'
+// The others meet in global memory: a fence, an exchange, a fence and a read
+// back, a microsecond or two per level; that chain bounds a small tree, and the boxes'
 // traffic a large one.  kPack: the packed binary nodes are written on the way
 // (both children's boxes are at hand), and `sc` receives the tree's depth and
 // box at the root; otherwise every node's box goes to nbox.  The arrival word
@@ -817,7 +817,7 @@ __device__ __forceinline__ void climb(ClimbShared& sm, bool leaf, int64_t T, int
     int height = 0;
     if (!kPack) put_box(nbox, cur, lo, hi);
     // every chain ends at the root; the cap only guards against a malformed
-    // tree (the build then reports the depth it reached)
+    // tree (the depth recorded is then one that the build rejects)
     int32_t p = parent[cur];
     for (int steps = 0; p >= 0 && steps <= kMaxWalk; ++steps) {
         const int32_t a = child[2 * p], b = child[2 * p + 1], r0 = range[2 * p], r1 = range[2 * p + 1];
@@ -845,6 +845,7 @@ __device__ __forceinline__ void climb(ClimbShared& sm, bool leaf, int64_t T, int
             __threadfence();
             const int other = atomicExch(&visits[p], height + 1);
             if (other == 0) return;
+            __threadfence();                            // the sibling's box is read after its arrival
             const int64_t sib = left ? b : a;
             for (int c = 0; c < 3; ++c) {
                 slo[c] = __ldcg(&nbox[6 * sib + c]);
@@ -876,8 +877,8 @@ __device__ __forceinline__ void climb(ClimbShared& sm, bool leaf, int64_t T, int
         last = r1;
         p = parent[p];
     }
-    if (kPack && p < 0) {
-        sc->max_depth = height;
+    if (kPack) {
+        sc->max_depth = p < 0 ? height : kMaxWalk;
         for (int c = 0; c < 3; ++c) {
             sc->lo[c] = lo[c];
             sc->hi[c] = hi[c];
