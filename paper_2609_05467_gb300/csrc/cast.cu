@@ -1019,11 +1019,21 @@ using CastAcc = CastAccFwd;
 constexpr int kPoolPairs = 320;        // pairs (ray, node or leaf) on the stack
 constexpr int kPoolLeaves = 128;       // pairs (ray, triangle) that wait for a full step
 constexpr int kPoolFill = 22;          // lanes that are enough for a step
-// Room on the stack: a step takes n pairs and adds up to 4 n.  While more than
-// kPoolFull wait, steps take fewer, down to one pair at a time, whose subtree
-// needs at most 3 entries per level of a tree of depth (kStack4 - 1) / 3.
-constexpr int kPoolFull = kPoolPairs - kStack4 - 96;
-static_assert(kPoolFull >= 64, "a box's rays on top of what waits");
+// Room on the stack: a step takes n <= 32 pairs and adds up to 4 n.  Before a
+// step that may find no room the lowest kPoolMove pairs move to the lanes'
+// local memory; they come back when fewer than 32 wait (axis rays: none).
+// Taking fewer pairs a step instead, down to one, starved parts whose boxes
+// overlap: 16,384 diagonal needles, 1,024 points x 256 directions 259 ms, now
+// 62 (a ray per lane: 150), their 3,072 axis rays 54.8 ms, now 10.0 (18.2).
+// All pairs together: what a step adds lies on top, and what lies above a pair
+// that waits descends from pairs added with it.  So at most one step's pairs
+// wait per level of the tree, 128 for each of (kStack4 - 1) / 3 levels, on top
+// of a box's rays and what was left before them.
+constexpr int kPoolFull = kPoolPairs - 96;
+constexpr int kPoolMove = 128;         // four a lane
+constexpr int kPoolStore = 128;        // pairs a lane can keep aside
+static_assert(kPoolFull >= 64 && kPoolMove <= kPoolFull, "a box's rays on top of what waits");
+static_assert(32 * kPoolStore >= 63 + 128 * ((kStack4 - 1) / 3), "every pair of a walk has a place");
 
 // A pair: a code (node >= 0, leaf < 0) and the slot of its ray.  32 bits hold
 // codes of 26 bits, that is 2^25 nodes and 2^24 triangles; parts beyond that
@@ -1056,6 +1066,30 @@ struct __align__(16) PoolOf {
     uint8_t met[kFrontEntries];    // the frontier boxes that the current tile can meet
 };
 static_assert(kPoolPairs >= kFrontQueue, "the stack also serves as the frontier's queue");
+
+// The lowest kPoolMove of the stack's sp pairs go to the lanes' stores (each
+// place is read and written by one lane: no barrier in between), and back.
+// The warp calls both; a barrier before and after.
+template <class Pair>
+__device__ __forceinline__ void pool_aside(Pair* pair, int& sp, Pair* store, int& stored)
+{
+    const int lane = threadIdx.x & 31;
+    for (int k = 0; k < kPoolMove / 32; ++k) store[stored + k] = pair[32 * k + lane];
+    stored += kPoolMove / 32;
+    for (int q = kPoolMove + lane; q < sp; q += 32) pair[q - kPoolMove] = pair[q];
+    sp -= kPoolMove;
+    __syncwarp();
+}
+template <class Pair>
+__device__ __forceinline__ void pool_back(Pair* pair, int& sp, Pair* store, int& stored)
+{
+    const int lane = threadIdx.x & 31;
+    stored -= kPoolMove / 32;
+    if (lane < sp) pair[kPoolMove + lane] = pair[lane];
+    for (int k = 0; k < kPoolMove / 32; ++k) pair[32 * k + lane] = store[stored + k];
+    sp += kPoolMove;
+    __syncwarp();
+}
 
 // bit rows of a warp: visible so far, met an ambiguous pair, met an ambiguous
 // pair that FP64 calls a hit, and (instrumented cast) re-tested in FP64
@@ -1224,11 +1258,19 @@ __device__ __forceinline__ void cast_point_pooled(const float4* __restrict__ wno
     unsigned live0 = 0, live1 = 0;         // slots 0..31 and 32..63 whose rays are not known to be blocked
     int t = t0;                            // next tile
     int boxes = 0;                         // of pool->met still to be tested
-    // on a well-formed tree a ray meets each node at most once; the cap only
-    // bounds a malformed one
-    int steps = (int)min64(0x7FFFFFFF, 2 * (int64_t)(t1 - t0 + 1) * max_steps);
+    Pair store[kPoolStore];                // pairs set aside (pool_aside)
+    int stored = 0;                        // of store, the same in every lane
+    // On a well-formed tree a ray meets each node and leaf at most once, and a
+    // step takes at least one pair: at most 64 rays have pairs between two
+    // entries of tiles.  The cap only bounds a malformed tree.
+    const int most = (int)min64(0x7FFFFFFF, 64 * (int64_t)max_steps);
+    int steps = most;
     for (;;) {
-        if (lsp < 32 && sp < 32 && boxes > 0) {
+        if (lsp < 32 && sp < 32 && (boxes > 0 || stored > 0)) {
+            if (stored > 0) {
+                pool_back(pool->pair, sp, store, stored);
+                continue;
+            }
             // the tile's rays against its frontier boxes, nearest first (the
             // deepest), until a step's worth of pairs waits
             if (live1 == 0) {
@@ -1261,14 +1303,14 @@ __device__ __forceinline__ void cast_point_pooled(const float4* __restrict__ wno
             // per lane; pairs with a leaf move to the leaf queue, pairs of
             // blocked rays are dropped, and lanes left without look again
             if (--steps < 0) break;
-            bool have = false, idle = false;
-            if (sp > kPoolFull) idle = lane >= max(1, min(32, (kPoolPairs - kStack4 - sp) / 3));
+            if (sp > kPoolFull) pool_aside(pool->pair, sp, store, stored);
+            bool have = false;
             int code = 0, slot = 0;
             for (;;) {
-                const unsigned want = __ballot_sync(kAll, !(have || idle));
+                const unsigned want = __ballot_sync(kAll, !have);
                 const int at = sp - 1 - __popc(want & below);
                 bool leaf = false;
-                if (!(have || idle) && at >= 0) {
+                if (!have && at >= 0) {
                     const Pair q = pool->pair[at];
                     slot = q.slot();
                     code = q.code();
@@ -1283,7 +1325,7 @@ __device__ __forceinline__ void cast_point_pooled(const float4* __restrict__ wno
                 if (two) pool->leaf[lsp + __popc(m2 & below)] = Pair::make(leaf_code(leaf_first(code) + 1, 1), slot);
                 lsp += __popc(m2);
                 sp = max(0, sp - __popc(want));
-                if (sp == 0 || lsp > kPoolLeaves - 64 || __popc(__ballot_sync(kAll, have || idle)) >= kPoolFill) break;
+                if (sp == 0 || lsp > kPoolLeaves - 64 || __popc(__ballot_sync(kAll, have)) >= kPoolFill) break;
             }
             bool i0 = false, i1 = false, i2 = false, i3 = false;
             float4 ci = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
@@ -1368,6 +1410,7 @@ __device__ __forceinline__ void cast_point_pooled(const float4* __restrict__ wno
             continue;
         }
         if (t >= t1) break;
+        steps = most;
         // the next tile enters; the rays of the pairs left over move down
         // (one slot per ray, the lowest pair's)
         if (sp + lsp > 0) {
@@ -1438,7 +1481,16 @@ __device__ __forceinline__ void cast_point_pooled(const float4* __restrict__ wno
         }
         __syncwarp();
     }
-    if (steps < 0) acc.overflow += lane == 0;
+    if (steps < 0) {
+        // rays that are not decided count as blocked (those of later tiles have no bit yet)
+        acc.overflow += lane == 0;
+        for (int q = 0; q < 2; ++q)
+            if (((q ? live1 : live0) >> lane) & 1u) {
+                const int j = __float_as_int(pool->inv[32 * q + lane].w);
+                atomicAnd(&vis[j >> 5], ~(1u << (j & 31)));
+            }
+        __syncwarp();
+    }
     // visible, less the rays that only an FP64-ambiguous pair blocks
     int cnt = 0;
     for (int w = lane; w < W; w += 32) {
@@ -1510,21 +1562,23 @@ __device__ __forceinline__ bool trace_axis(const float4* __restrict__ ftree, con
         acc.rays += 1;
     }
     int sp = __popc(live), lsp = 0;
+    Pair store[kPoolStore];                // pairs set aside (pool_aside)
+    int stored = 0;
     __syncwarp();
-    // on a well-formed tree a ray meets each node at most once; the cap only
-    // bounds a malformed one
-    int steps = (int)min64(0x7FFFFFFF, 2 * (int64_t)max_steps);
+    // on a well-formed tree each of 32 rays meets a node or leaf at most once,
+    // and a step takes at least one pair; the cap only bounds a malformed tree
+    int steps = (int)min64(0x7FFFFFFF, 32 * (int64_t)max_steps);
     for (;;) {
         if (lsp < 32 && sp > 0) {
             if (--steps < 0) break;
-            bool have = false, idle = false;
-            if (sp > kPoolFull) idle = lane >= max(1, min(32, (kPoolPairs - kStack4 - sp) / 3));
+            if (sp > kPoolFull) pool_aside(pool->pair, sp, store, stored);
+            bool have = false;
             int code = 0, slot = 0;
             for (;;) {
-                const unsigned want = __ballot_sync(kAll, !(have || idle));
+                const unsigned want = __ballot_sync(kAll, !have);
                 const int at = sp - 1 - __popc(want & below);
                 bool leaf = false;
-                if (!(have || idle) && at >= 0) {
+                if (!have && at >= 0) {
                     const Pair q = pool->pair[at];
                     slot = q.slot();
                     code = q.code();
@@ -1539,7 +1593,7 @@ __device__ __forceinline__ bool trace_axis(const float4* __restrict__ ftree, con
                 if (two) pool->leaf[lsp + __popc(m2 & below)] = Pair::make(leaf_code(leaf_first(code) + 1, 1), slot);
                 lsp += __popc(m2);
                 sp = max(0, sp - __popc(want));
-                if (sp == 0 || lsp > kPoolLeaves - 64 || __popc(__ballot_sync(kAll, have || idle)) >= kPoolFill) break;
+                if (sp == 0 || lsp > kPoolLeaves - 64 || __popc(__ballot_sync(kAll, have)) >= kPoolFill) break;
             }
             bool i0 = false, i1 = false, i2 = false, i3 = false;
             float4 ci = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
@@ -1569,6 +1623,10 @@ __device__ __forceinline__ bool trace_axis(const float4* __restrict__ ftree, con
             if (i0) pool->pair[sp + __popc(bn & below)] = Pair::make(__float_as_int(ci.x), slot);
             sp += __popc(bn);
             __syncwarp();
+            continue;
+        }
+        if (lsp < 32 && stored > 0) {
+            pool_back(pool->pair, sp, store, stored);
             continue;
         }
         if (lsp == 0) break;
@@ -1607,7 +1665,10 @@ __device__ __forceinline__ bool trace_axis(const float4* __restrict__ ftree, con
         live &= ~__reduce_or_sync(kAll, hit ? 1u << slot : 0u);
         __syncwarp();
     }
-    if (steps < 0) acc.overflow += lane == 0;
+    if (steps < 0) {
+        acc.overflow += lane == 0;
+        live = 0;                              // rays that are not decided count as blocked
+    }
     const bool open = (live >> lane) & 1u;
     if (open && ((amb >> lane) & 1u)) ++acc.amb;
     return cast && !(open && !((hit64 >> lane) & 1u));
