@@ -21,7 +21,7 @@ rc_status build_bvh(rc_bvh h, cudaStream_t s);
 rc_status refit_bvh(rc_bvh h, cudaStream_t s);
 rc_status sample_points(rc_bvh h, int64_t n, const rc_params* p, float* P, float* N, int32_t* face,
                         double* weight, cudaStream_t s);
-rc_status launch_hemisphere(rc_bvh h, const float* P, const float* N, int64_t n, const rc_params* p,
+rc_status launch_hemisphere(rc_bvh h, const float* P, const float* N, int64_t n, const float4* tdirs, const rc_params* p,
                             uint32_t* bits, int32_t* count, unsigned long long* counters, bool stats,
                             cudaStream_t s, long long* relist = nullptr, long long relist_cap = 0);
 rc_status launch_orthogonal(rc_bvh h, const float* P, const float* N, int64_t n, const rc_params* p,
@@ -417,12 +417,9 @@ rc_status rc_hemisphere_cast(rc_bvh h, const float* d_P, const float* d_N, int64
     if (d_counters) RC_CUDA(cudaMemsetAsync(d_counters, 0, sizeof(int64_t) * (stats ? 8 : 4), s));
     if (n == 0) return RC_OK;
     if (!d_P || !d_N || !d_bits || !d_count) return set_error(RC_E_ARG, "array pointer is NULL");
-    const float4 *dirs = nullptr, *tdirs = nullptr;
-    if ((st = device_dirs(p->n_dirs, &dirs, &tdirs)) != RC_OK) return st;
-    h->dirs = dirs;
-    h->tdirs = p->tile_mode == 1 ? dirs : tdirs;
-    h->dirs_n = p->n_dirs;
-    return launch_hemisphere(h, d_P, d_N, n, p, d_bits, d_count, (unsigned long long*)d_counters, stats, s);
+    const float4* tdirs = nullptr;
+    if ((st = device_dirs_for_cast(p, &tdirs)) != RC_OK) return st;
+    return launch_hemisphere(h, d_P, d_N, n, tdirs, p, d_bits, d_count, (unsigned long long*)d_counters, stats, s);
 }
 
 rc_status rc_hemisphere_cast_retests(rc_bvh h, const float* d_P, const float* d_N, int64_t n, const rc_params* p,
@@ -441,12 +438,9 @@ rc_status rc_hemisphere_cast_retests(rc_bvh h, const float* d_P, const float* d_
     RC_CUDA(cudaMemsetAsync(d_counters, 0, sizeof(int64_t) * 8, s));
     if (n == 0) return RC_OK;
     if (!d_P || !d_N || !d_bits || !d_count) return set_error(RC_E_ARG, "array pointer is NULL");
-    const float4 *dirs = nullptr, *tdirs = nullptr;
-    if ((st = device_dirs(p->n_dirs, &dirs, &tdirs)) != RC_OK) return st;
-    h->dirs = dirs;
-    h->tdirs = p->tile_mode == 1 ? dirs : tdirs;
-    h->dirs_n = p->n_dirs;
-    return launch_hemisphere(h, d_P, d_N, n, p, d_bits, d_count, (unsigned long long*)d_counters, true, s,
+    const float4* tdirs = nullptr;
+    if ((st = device_dirs_for_cast(p, &tdirs)) != RC_OK) return st;
+    return launch_hemisphere(h, d_P, d_N, n, tdirs, p, d_bits, d_count, (unsigned long long*)d_counters, true, s,
                              (long long*)d_list, cap);
 }
 

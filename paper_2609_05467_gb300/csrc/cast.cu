@@ -2471,7 +2471,7 @@ struct LaunchScratch {
     }
 };
 
-rc_status launch_hemisphere(rc_bvh h, const float* P, const float* N, int64_t n, const rc_params* p,
+rc_status launch_hemisphere(rc_bvh h, const float* P, const float* N, int64_t n, const float4* tdirs, const rc_params* p,
                             uint32_t* bits, int32_t* count, unsigned long long* counters, bool stats,
                             cudaStream_t s, long long* relist, long long relist_cap)
 {
@@ -2524,7 +2524,7 @@ rc_status launch_hemisphere(rc_bvh h, const float* P, const float* N, int64_t n,
             if (smem > 48 * 1024)
                 RC_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
             kernel<<<(unsigned)blocks, threads, smem, s>>>(tree, h->tris, max_steps(h), h->scene_maxabs, P, N, n, order,
-                                                           h->tdirs, p->n_dirs, p->origin_offset, bits, count, counters,
+                                                           tdirs, p->n_dirs, p->origin_offset, bits, count, counters,
                                                            work, n - n_split, splits, relist, relist_cap);
             return RC_OK;
         };
