@@ -17,7 +17,7 @@ namespace rc {
 rc_status point_order(rc_bvh h, const float* P, int64_t n, int32_t* order, cudaStream_t s);
 rc_status launch_batch(const BatchPart* d_parts, int n_parts, long long n_items, int ppi, const float4* tdirs,
                        const rc_params* p, int64_t max_tris, unsigned long long* work, cudaStream_t s);
-rc_status prepare_batch_kernel(int n_dirs);
+rc_status prepare_batch_kernel();
 rc_status device_dirs_for_cast(const rc_params* p, const float4** tdirs);
 rc_status check_params_public(const rc_params* p);
 bool use_wide(const rc_params* p);
@@ -195,7 +195,7 @@ static rc_status prepare(rc_batch b, cudaStream_t s)
     const float4* tdirs = nullptr;
     rc_status st = device_dirs_for_cast(&b->p, &tdirs);
     if (st != RC_OK) return st;
-    st = prepare_batch_kernel(b->p.n_dirs);
+    st = prepare_batch_kernel();
     if (st != RC_OK) return st;
     // capture on the batch's private stream; nothing runs during capture
     const float4* canon = nullptr;

@@ -1765,6 +1765,16 @@ __host__ __device__ __forceinline__ size_t cast_smem(int warps, int W, int kind,
     return warps * pool_bytes(kind) + (size_t)warps * W * cast_rows(kind, stats) * sizeof(uint32_t);
 }
 
+// Let a kernel have the shared memory of the most directions.  The limit
+// belongs to the kernel, not to a launch, and casts of other threads may have
+// other direction counts: it is always set to the same value.
+template <class Kernel>
+static cudaError_t allow_cast_smem(Kernel kernel, int warps, int kind, bool stats)
+{
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)cast_smem(warps, kMaxDirs / 32, kind, stats));
+}
+
 template <bool kStats, int kKind>
 __device__ __forceinline__ void cast_point(const float4* __restrict__ nodes, const float4* __restrict__ tris,
                                            int max_steps, float scene_maxabs, const float* __restrict__ P,
@@ -2521,8 +2531,7 @@ rc_status launch_hemisphere(rc_bvh h, const float* P, const float* N, int64_t n,
             RC_LAUNCHED();
         }
         const auto run = [&](auto kernel) -> rc_status {
-            if (smem > 48 * 1024)
-                RC_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            if (smem > 48 * 1024) RC_CUDA(allow_cast_smem(kernel, threads / 32, kind, stats));
             kernel<<<(unsigned)blocks, threads, smem, s>>>(tree, h->tris, max_steps(h), h->scene_maxabs, P, N, n, order,
                                                            tdirs, p->n_dirs, p->origin_offset, bits, count, counters,
                                                            work, n - n_split, splits, relist, relist_cap);
@@ -2810,17 +2819,11 @@ rc_status launch_batch(const BatchPart* d_parts, int n_parts, long long n_items,
     return RC_OK;
 }
 
-rc_status prepare_batch_kernel(int n_dirs)
+rc_status prepare_batch_kernel()
 {
-    const int W = (n_dirs + 31) / 32;
-    const auto allow = [&](auto kernel, int kind) {
-        const size_t smem = cast_smem(4, W, kind, false);
-        return smem > 48 * 1024 ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-                                : cudaSuccess;
-    };
-    RC_CUDA(allow(k_batch<false, kBinary>, kBinary));
-    RC_CUDA(allow(k_batch<false, kWide4>, kWide4));
-    RC_CUDA(allow(k_batch<false, kWide4Big>, kWide4Big));
+    RC_CUDA(allow_cast_smem(k_batch<false, kBinary>, 4, kBinary, false));
+    RC_CUDA(allow_cast_smem(k_batch<false, kWide4>, 4, kWide4, false));
+    RC_CUDA(allow_cast_smem(k_batch<false, kWide4Big>, 4, kWide4Big, false));
     return RC_OK;
 }
 
