@@ -381,7 +381,7 @@ k_dir_hist(const uint32_t* __restrict__ bits, int64_t n, int W, int n_dirs, cons
         if (equal) {
 #pragma unroll 8
             for (int q = 0; q < m; ++q) cnt += (__ldg(row + (int64_t)q * W) >> lane) & 1u;
-            s = __dmul_rn((double)cnt, first);
+            if (cnt) s = __dmul_rn((double)cnt, first);      // (an infinite weight times no point is no weight)
         } else {
             int q = 0;
 #pragma unroll 4
