@@ -128,15 +128,37 @@ __device__ __noinline__ DirSums exact_sums(const uint32_t* __restrict__ bits, fl
 //   - Two directions per instruction (f32x2), from a table in shared memory
 //     whose entries are the pairs of words 2 p and 2 p + 1.
 // 300k points x 1000 directions, 70% visible: 729 -> 467 us.
-// conc_mode 1 needs the sums themselves and takes the exact path per point.
+// conc_mode 1 (kSums) needs the exact sums themselves and no counts by axis: it
+// takes them in the one pass, two directions per instruction as well (300k
+// points x 1000 directions 532 us, 20k x 8192, whose table is read from L1,
+// 374; the fp32 pass and then exact_sums 1151 and 705).
 constexpr int kVarThreads = 256, kVarBlocks = 4;   // 3, 5 and 6 blocks per SM measured 6 to 9% slower
 constexpr int kVarTableWords = 96;     // most words of the shared table (36 KB); beyond, the table is read from L1
 
-template <bool kTable>
+// fixed40_split of the two values of x where they are visible, added to the
+// sums hi and lo, each with the bits of C on top (kFixedC a value, modulo
+// 2^32: taken off once per sum)
+constexpr unsigned kFixedC = 0x4B400000u;
+__device__ __forceinline__ void add_fixed40(f2 x, bool v0, bool v1, unsigned& hi, unsigned& lo)
+{
+    const float C = 12582912.0f;                             // the float of bits kFixedC
+    const f2 k18 = pack2(262144.0f, 262144.0f), k22 = pack2(4194304.0f, 4194304.0f), c = pack2(C, C), neg = pack2(-1.0f, -1.0f);
+    float x0, x1;
+    unpack2(x, x0, x1);
+    const f2 y = pack2(v0 ? x0 : 0.0f, v1 ? x1 : 0.0f);      // zero adds zero to both
+    const f2 a = fma2(y, k18, c), r = fma2(y, k18, fma2(a, neg, c)), l = fma2(r, k22, c);
+    float a0, a1, l0, l1;
+    unpack2(a, a0, a1);
+    unpack2(l, l0, l1);
+    hi += __float_as_uint(a0) + __float_as_uint(a1);
+    lo += __float_as_uint(l0) + __float_as_uint(l1);
+}
+
+template <bool kTable, bool kSums>
 __global__ void __launch_bounds__(kVarThreads, kVarBlocks)
 k_variability(const uint32_t* __restrict__ bits, const float* __restrict__ Nrm,
               const double* __restrict__ weight, int64_t n,
-              const float4* __restrict__ dirs, int n_dirs, int conc_mode, int G, float* acc, int8_t* dom,
+              const float4* __restrict__ dirs, int n_dirs, int G, float* acc, int8_t* dom,
               float* conc, unsigned long long* sums, double* wpart)
 {
     constexpr unsigned kAll = 0xFFFFFFFFu;
@@ -164,7 +186,7 @@ k_variability(const uint32_t* __restrict__ bits, const float* __restrict__ Nrm,
     for (int64_t g = (int64_t)blockIdx.x * (kVarThreads >> 5) + (threadIdx.x >> 5); g * G < n; g += nw) {
         const int m = (int)min64(G, n - g * G);
         int my_cnt = 0, my_axis = 0, my_dm = -1;   // point `lane` of the group: visible rays, those along dm, dm
-        long long my_M = 0;                        // |M_dm| (conc_mode 1)
+        long long my_M = 0;                        // |M_dm| (kSums)
         for (int q = 0; q < m; ++q) {
             const int64_t i = g * G + q;
             const float nx = Nrm[3 * i], ny = Nrm[3 * i + 1], nz = Nrm[3 * i + 2];
@@ -173,14 +195,18 @@ k_variability(const uint32_t* __restrict__ bits, const float* __restrict__ Nrm,
             const f2 bx = pack2(b.t2x, b.t2x), by = pack2(b.t2y, b.t2y), bz = pack2(b.t2z, b.t2z);
             const f2 cx = pack2(nx, nx), cy = pack2(ny, ny), cz = pack2(nz, nz);
             f2 sx = 0, sy = 0, sz = 0;
+            long long M0 = 0, M1 = 0, M2 = 0;
             int a1 = 0, a2 = 0, cnt = 0;
             for (int w0 = 0; w0 < W; w0 += 32) {
                 const int wn = min(32, W - w0);
                 const uint32_t mine = lane < wn ? __ldg(&bits[i * W + w0 + lane]) : 0u;
                 cnt += __popc(mine);
+                unsigned h0 = 0, h1 = 0, h2 = 0, l0 = 0, l1 = 0, l2 = 0;   // as in exact_sums
+                unsigned off = 0;
                 for (int dw = 0; dw < wn; dw += 2) {
                     const uint32_t u0 = __shfl_sync(kAll, mine, dw), u1 = __shfl_sync(kAll, mine, dw + 1);
                     if ((u0 | u1) == 0u) continue;
+                    if (kSums) off -= 2 * kFixedC;
                     f2 hx, hy, hz;
                     if (kTable) {
                         const float2* t = s_dirs + 16 * (w0 + dw) + lane;
@@ -199,6 +225,12 @@ k_variability(const uint32_t* __restrict__ bits, const float* __restrict__ Nrm,
                     const f2 dy = add2(add2(mul2(ay, hx, mz), mul2(by, hy, mz)), mul2(cy, hz, mz));
                     const f2 dz = add2(add2(mul2(az, hx, mz), mul2(bz, hy, mz)), mul2(cz, hz, mz));
                     const bool v0 = (u0 >> lane) & 1u, v1 = (u1 >> lane) & 1u;
+                    if (kSums) {
+                        add_fixed40(dx, v0, v1, h0, l0);
+                        add_fixed40(dy, v0, v1, h1, l1);
+                        add_fixed40(dz, v0, v1, h2, l2);
+                        continue;
+                    }
                     const f2 on = pack2(v0 ? 1.0f : 0.0f, v1 ? 1.0f : 0.0f);
                     sx = fma2(on, dx, sx);
                     sy = fma2(on, dy, sy);
@@ -207,41 +239,62 @@ k_variability(const uint32_t* __restrict__ bits, const float* __restrict__ Nrm,
                     unpack2(dx, x0, x1);
                     unpack2(dy, y0, y1);
                     unpack2(dz, z0, z1);
-                    const bool l0 = fabsf(z0) > fmaxf(fabsf(x0), fabsf(y0)), l1 = fabsf(z1) > fmaxf(fabsf(x1), fabsf(y1));
-                    a2 += v0 && l0;
-                    a2 += v1 && l1;
-                    a1 += v0 && !l0 && fabsf(y0) > fabsf(x0);
-                    a1 += v1 && !l1 && fabsf(y1) > fabsf(x1);
+                    const bool z0m = fabsf(z0) > fmaxf(fabsf(x0), fabsf(y0)), z1m = fabsf(z1) > fmaxf(fabsf(x1), fabsf(y1));
+                    a2 += v0 && z0m;
+                    a2 += v1 && z1m;
+                    a1 += v0 && !z0m && fabsf(y0) > fabsf(x0);
+                    a1 += v1 && !z1m && fabsf(y1) > fabsf(x1);
+                }
+                if (kSums) {
+                    M0 += (long long)(int)(h0 + off) * 4194304LL + (int)(l0 + off);
+                    M1 += (long long)(int)(h1 + off) * 4194304LL + (int)(l1 + off);
+                    M2 += (long long)(int)(h2 + off) * 4194304LL + (int)(l2 + off);
                 }
             }
             cnt = __reduce_add_sync(kAll, cnt);
-            a1 = __reduce_add_sync(kAll, a1);
-            a2 = __reduce_add_sync(kAll, a2);
             if (cnt == 0) continue;                // the lane's initial values
-            float S[3], t;
-            unpack2(sx, S[0], t);
-            S[0] += t;
-            unpack2(sy, S[1], t);
-            S[1] += t;
-            unpack2(sz, S[2], t);
-            S[2] += t;
-            for (int off = 16; off; off >>= 1) {
-                S[0] += __shfl_xor_sync(kAll, S[0], off);
-                S[1] += __shfl_xor_sync(kAll, S[1], off);
-                S[2] += __shfl_xor_sync(kAll, S[2], off);
+            int dm = 0;
+            bool clear = false;
+            if (!kSums) {
+                a1 = __reduce_add_sync(kAll, a1);
+                a2 = __reduce_add_sync(kAll, a2);
+                float S[3], t;
+                unpack2(sx, S[0], t);
+                S[0] += t;
+                unpack2(sy, S[1], t);
+                S[1] += t;
+                unpack2(sz, S[2], t);
+                S[2] += t;
+                for (int off = 16; off; off >>= 1) {
+                    S[0] += __shfl_xor_sync(kAll, S[0], off);
+                    S[1] += __shfl_xor_sync(kAll, S[1], off);
+                    S[2] += __shfl_xor_sync(kAll, S[2], off);
+                }
+                const float B = fmaxf(fabsf(b.t1x) + fabsf(b.t2x) + fabsf(nx),
+                                      fmaxf(fabsf(b.t1y) + fabsf(b.t2y) + fabsf(ny), fabsf(b.t1z) + fabsf(b.t2z) + fabsf(nz)));
+                const float err = 6.3e-8f * B * (float)cnt * (float)(W / 2 + 8);
+                const float A0 = fabsf(S[0]), A1 = fabsf(S[1]), A2 = fabsf(S[2]);
+                dm = A1 > A0 ? 1 : 0;
+                if (A2 > fmaxf(A0, A1)) dm = 2;
+                const float first = fmaxf(A0, fmaxf(A1, A2)), second = fmaxf(fminf(A0, A1), fminf(fmaxf(A0, A1), A2));
+                clear = first - second > 2.0f * err;
             }
-            const float B = fmaxf(fabsf(b.t1x) + fabsf(b.t2x) + fabsf(nx),
-                                  fmaxf(fabsf(b.t1y) + fabsf(b.t2y) + fabsf(ny), fabsf(b.t1z) + fabsf(b.t2z) + fabsf(nz)));
-            const float err = 6.3e-8f * B * (float)cnt * (float)(W / 2 + 8);
-            const float A0 = fabsf(S[0]), A1 = fabsf(S[1]), A2 = fabsf(S[2]);
-            int dm = A1 > A0 ? 1 : 0;
-            if (A2 > fmaxf(A0, A1)) dm = 2;
-            const float first = fmaxf(A0, fmaxf(A1, A2)), second = fmaxf(fminf(A0, A1), fminf(fmaxf(A0, A1), A2));
             long long M = 0;
-            if (conc_mode != 0 || !(first - second > 2.0f * err)) {
-                const DirSums e = exact_sums(bits, nx, ny, nz, i, W, dirs);
-                const long long M0 = e.M[0] < 0 ? -e.M[0] : e.M[0], M1 = e.M[1] < 0 ? -e.M[1] : e.M[1],
-                                M2 = e.M[2] < 0 ? -e.M[2] : e.M[2];
+            if (!clear) {
+                DirSums e;
+                if (kSums) {
+                    for (int off = 16; off; off >>= 1) {
+                        M0 += __shfl_xor_sync(kAll, M0, off);
+                        M1 += __shfl_xor_sync(kAll, M1, off);
+                        M2 += __shfl_xor_sync(kAll, M2, off);
+                    }
+                    e = DirSums{{M0, M1, M2}};
+                } else {
+                    e = exact_sums(bits, nx, ny, nz, i, W, dirs);
+                }
+                M0 = e.M[0] < 0 ? -e.M[0] : e.M[0];
+                M1 = e.M[1] < 0 ? -e.M[1] : e.M[1];
+                M2 = e.M[2] < 0 ? -e.M[2] : e.M[2];
                 dm = M1 > M0 ? 1 : 0;
                 M = M1 > M0 ? M1 : M0;
                 if (M2 > M) {
@@ -260,7 +313,7 @@ k_variability(const uint32_t* __restrict__ bits, const float* __restrict__ Nrm,
             const int64_t i = g * G + lane;
             double cc = 0.0;
             if (my_cnt > 0) {
-                if (conc_mode == 0)
+                if (!kSums)
                     cc = __ddiv_rn((double)my_axis, (double)my_cnt);
                 else
                     cc = __ddiv_rn(__ll2double_rn(my_M), __dmul_rn(1099511627776.0, (double)my_cnt));
@@ -512,12 +565,11 @@ rc_status launch_variability(const uint32_t* bits, const float* N, const double*
         const int64_t groups = (n + G - 1) / G;
         int64_t blocks = std::min<int64_t>((groups + kVarThreads / 32 - 1) / (kVarThreads / 32), (int64_t)sm * kVarBlocks);
         if (blocks > kVarMaxBlocks) blocks = kVarMaxBlocks;
-        if (W <= kVarTableWords)
-            k_variability<true><<<(unsigned)blocks, kVarThreads, (size_t)((W + 1) / 2) * 32 * 3 * sizeof(float2), s>>>(
-                bits, N, weight, n, dirs, nd, p->conc_mode, G, acc, dom, conc, sums, wpart);
-        else
-            k_variability<false><<<(unsigned)blocks, kVarThreads, 0, s>>>(bits, N, weight, n, dirs, nd, p->conc_mode, G,
-                                                                         acc, dom, conc, sums, wpart);
+        const bool table = W <= kVarTableWords;
+        const auto kernel = p->conc_mode == 0 ? (table ? k_variability<true, false> : k_variability<false, false>)
+                                              : (table ? k_variability<true, true> : k_variability<false, true>);
+        kernel<<<(unsigned)blocks, kVarThreads, table ? (size_t)((W + 1) / 2) * 32 * 3 * sizeof(float2) : 0, s>>>(
+            bits, N, weight, n, dirs, nd, G, acc, dom, conc, sums, wpart);
         RC_LAUNCHED();
         if (weight) {
             k_wsum_finish<<<1, 32, 0, s>>>(wpart, (int)blocks, wsum);
