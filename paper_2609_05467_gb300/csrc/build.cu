@@ -1652,8 +1652,9 @@ __device__ __forceinline__ void frame_bounds(float x, float y, float z, float a,
     float h, l;
     dot2(x, a, y, b, z, c, h, l);
     const float e = 2e-13f * (fabsf(x * a) + fabsf(y * b) + fabsf(z * c)) + 1e-36f;
-    lo = fminf(lo, __fadd_rd(h, __fsub_rd(l, e)));
-    hi = fmaxf(hi, __fadd_ru(h, __fadd_ru(l, e)));
+    const bool in = fabsf(h) < INFINITY;           // else beyond fp32's range: no bound
+    lo = fminf(lo, in ? __fadd_rd(h, __fsub_rd(l, e)) : -INFINITY);
+    hi = fmaxf(hi, in ? __fadd_ru(h, __fadd_ru(l, e)) : INFINITY);
 }
 
 // leaf boxes in frame coordinates and all boxes above them.  The bounds are

@@ -887,24 +887,29 @@ struct AxisRay {
 };
 
 // The band of an axis ray (see above).  Its bounds are sums hi + lo -+ tol
-// rounded outward; everything in tol is rounded up by its spare factors.
+// rounded outward; everything in tol is rounded up by its spare factors.  A
+// coordinate beyond fp32's range has no band, and a length whose square is
+// beyond it is bounded by the sum of its components.
 __device__ __forceinline__ AxisRay make_axis_ray(const FrameDev& fd, int a, float ox, float oy, float oz, float rs)
 {
     AxisRay ar;
     const int k = a >> 1;
     const bool pos = (a & 1) == 0;
     const float ex = ox - fd.c32[0], ey = oy - fd.c32[1], ez = oz - fd.c32[2];
-    const float reach = (sqrtf(ex * ex + ey * ey + ez * ez) + fd.r32 + 1e-6f * rs) * fd.rlen[k] + 1e-6f;
+    const float ee = ex * ex + ey * ey + ez * ez;
+    const float len = ee < INFINITY ? sqrtf(ee) : fabsf(ex) + fabsf(ey) + fabsf(ez);
+    const float reach = (len + fd.r32 + 1e-6f * rs) * fd.rlen[k] + 1e-6f;
     for (int j = 0; j < 3; ++j) {
         const float f0 = fd.axes[6 * j], f1 = fd.axes[6 * j + 1], f2 = fd.axes[6 * j + 2];   // column j
         float hi, lo;
         dot2(ox, f0, oy, f1, oz, f2, hi, lo);
         const float qs = fabsf(ox * f0) + fabsf(oy * f1) + fabsf(oz * f2);
         float tol = 1.01e-9f * rs + 2e-13f * (qs + 4.0f * rs + 1.0f);
-        if (j != k) tol += reach * (fd.gram_up[3 * j + k] + 1e-15f);
+        if (j != k) tol += reach * fd.gram_up[3 * j + k];
         tol *= 1.001f;
-        ar.lo[j] = __fadd_rd(hi, __fsub_rd(lo, tol));
-        ar.hi[j] = __fadd_ru(hi, __fadd_ru(lo, tol));
+        const bool in = fabsf(hi) < INFINITY;
+        ar.lo[j] = in ? __fadd_rd(hi, __fsub_rd(lo, tol)) : -INFINITY;
+        ar.hi[j] = in ? __fadd_ru(hi, __fadd_ru(lo, tol)) : INFINITY;
         if (j == k) {
             if (pos) ar.hi[j] = INFINITY;
             else ar.lo[j] = -INFINITY;
@@ -2603,11 +2608,15 @@ __global__ void k_frame_init(const __grid_constant__ FrameArgs a, FrameDev* fram
     const float* f = a.f[blockIdx.x];
     FrameDev* d = frames + blockIdx.x;
     if (t < 9) {
-        const double gram = __dadd_rn(__dadd_rn(__dmul_rn((double)f[j], (double)f[k]), __dmul_rn((double)f[3 + j], (double)f[3 + k])),
-                                      __dmul_rn((double)f[6 + j], (double)f[6 + k]));
+        const auto product = [&](int a, int b) {
+            return __dadd_rn(__dadd_rn(__dmul_rn((double)f[a], (double)f[b]), __dmul_rn((double)f[3 + a], (double)f[3 + b])),
+                             __dmul_rn((double)f[6 + a], (double)f[6 + b]));
+        };
+        const double gram = product(j, k);
         d->frame[t] = (double)f[t];
         d->gram[t] = gram;
-        d->gram_up[t] = __double2float_ru(fabs(gram));
+        // its rounding, 1e-15 of the columns' lengths at most, is on top
+        d->gram_up[t] = __double2float_ru(fabs(gram) + 1e-15 * sqrt(product(j, j)) * sqrt(product(k, k)));
         if (j == k) d->rlen[j] = __double2float_ru(1.01 / sqrt(gram));
     }
     if (t < 18) d->axes[t] = (t / 3) & 1 ? -f[3 * k + t / 6] : f[3 * k + t / 6];
