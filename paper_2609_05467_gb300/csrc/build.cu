@@ -1216,7 +1216,7 @@ __device__ __forceinline__ long long quantise_area(double area, double amax, dou
 // their own had taken 45 us for 1.93M faces, the scan of 1,024-value blocks
 // with a barrier per doubling 25; together now 51)
 __global__ void __launch_bounds__(kScanThreads)
-k_scan_block(long long* x, int64_t n, const double* __restrict__ farea, const DevScalars* sc, long long* bsum)
+k_scan_block(long long* x, int64_t n, const double* __restrict__ farea, const DevScalars* sc, long long* bsum, long long* total)
 {
     __shared__ long long wsum[32];
     __shared__ double s_scale;
@@ -1263,7 +1263,10 @@ k_scan_block(long long* x, int64_t n, const double* __restrict__ farea, const De
         run += v[k];
         if (i0 + k < n) x[i0 + k] = run;
     }
-    if (threadIdx.x == kScanThreads - 1) bsum[blockIdx.x] = run;
+    if (threadIdx.x == kScanThreads - 1) {
+        bsum[blockIdx.x] = run;
+        if (gridDim.x == 1) *total = run;          // the last level: one block holds the sum of everything
+    }
 }
 
 __global__ void __launch_bounds__(kScanThreads)
@@ -1276,8 +1279,8 @@ k_scan_add(long long* x, int64_t n, const long long* bsum_incl)
         if (i0 + k < n) x[i0 + k] += add;
 }
 
-// inclusive scan of x, or of the quantised areas into x
-static rc_status scan_inclusive(long long* x, int64_t n, const double* farea, const DevScalars* sc, cudaStream_t s)
+// inclusive scan of x, or of the quantised areas into x; *total (device) = the sum
+static rc_status scan_inclusive(long long* x, int64_t n, const double* farea, const DevScalars* sc, long long* total, cudaStream_t s)
 {
     if (n <= 0) return RC_OK;
     const int64_t nb = (n + kScanBlock - 1) / kScanBlock;
@@ -1285,10 +1288,10 @@ static rc_status scan_inclusive(long long* x, int64_t n, const double* farea, co
     BuildScratch g{s};
     RC_CUDA(cudaMallocAsync(&bs, sizeof(long long) * nb, s));
     g.p[0] = bs;
-    k_scan_block<<<(unsigned)nb, kScanThreads, 0, s>>>(x, n, farea, sc, bs);
+    k_scan_block<<<(unsigned)nb, kScanThreads, 0, s>>>(x, n, farea, sc, bs, total);
     RC_LAUNCHED();
     if (nb > 1) {
-        rc_status st = scan_inclusive(bs, nb, nullptr, nullptr, s);
+        rc_status st = scan_inclusive(bs, nb, nullptr, nullptr, total, s);
         if (st != RC_OK) return st;
         k_scan_add<<<(unsigned)nb, kScanThreads, 0, s>>>(x, n, bs);
         RC_LAUNCHED();
@@ -1306,14 +1309,18 @@ __device__ __forceinline__ double uniform01(unsigned long long seed, long long i
     return __dmul_rn(__ull2double_rn(r >> 11), 1.0 / 9007199254740992.0);
 }
 
+// total = cdf[T - 1], which the build has read back: the search need not wait
+// for it.  kMany: conversions by integers, which spare the FP64 pipe but are a
+// longer chain; they pay from about 128 points an SM on (203k triangles: 37
+// points 6.5 us without and 7.4 with, 20,000 8.6 and 8.0, a million 93 and 76).
+template <bool kMany>
 __global__ void k_sample_area(const float* __restrict__ V, const int32_t* __restrict__ F, int64_t T,
-                              const long long* __restrict__ cdf, const float* __restrict__ fnorm, int64_t n, unsigned long long seed,
+                              const long long* __restrict__ cdf, long long total, const float* __restrict__ fnorm, int64_t n, unsigned long long seed,
                               float* P, float* Nout, int32_t* face, double* weight)
 {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
     const double u0 = uniform01(seed, i, 0), u1 = uniform01(seed, i, 1), u2 = uniform01(seed, i, 2);
-    const long long total = cdf[T - 1];
     const long long target = (long long)floor(__dmul_rn(u0, __ll2double_rn(total)));
     int64_t lo = 0, hi = T - 1;
     while (lo < hi) {
@@ -1326,12 +1333,11 @@ __global__ void k_sample_area(const float* __restrict__ V, const int32_t* __rest
     const double wb = __dmul_rn(s, __dsub_rn(1.0, u2));
     const double wc = __dmul_rn(s, u2);
     for (int k = 0; k < 3; ++k) {
-        const double A = widen(V[3 * (int64_t)F[3 * f + 0] + k]);
-        const double B = widen(V[3 * (int64_t)F[3 * f + 1] + k]);
-        const double C = widen(V[3 * (int64_t)F[3 * f + 2] + k]);
+        const float a = V[3 * (int64_t)F[3 * f + 0] + k], b = V[3 * (int64_t)F[3 * f + 1] + k], c = V[3 * (int64_t)F[3 * f + 2] + k];
+        const double A = kMany ? widen(a) : (double)a, B = kMany ? widen(b) : (double)b, C = kMany ? widen(c) : (double)c;
         double p = __dadd_rn(__dmul_rn(wa, A), __dmul_rn(wb, B));
         p = __dadd_rn(p, __dmul_rn(wc, C));
-        P[3 * i + k] = narrow(p);
+        P[3 * i + k] = kMany ? narrow(p) : __double2float_rn(p);
         Nout[3 * i + k] = fnorm[3 * f + k];
     }
     face[i] = (int32_t)f;
@@ -1482,7 +1488,7 @@ static rc_status face_data(rc_bvh h, float* tbox, cudaStream_t s)
     k_face_prep<<<(unsigned)std::min<int64_t>(nblocks(h->T, kPrepThreads), 8 * (int64_t)device_sms()), kPrepThreads, 0, s>>>(
         h->V, h->nV, h->F, h->T, h->fnorm, h->farea, tbox, h->sc);
     RC_LAUNCHED();
-    return scan_inclusive(h->cdf, h->T, h->farea, h->sc, s);
+    return scan_inclusive(h->cdf, h->T, h->farea, h->sc, &h->sc->total, s);
 }
 
 // mesh validity and scene bounds from the scalars already read back
@@ -1873,8 +1879,9 @@ rc_status sample_points(rc_bvh h, int64_t n, const rc_params* p, float* P, float
         RC_LAUNCHED();
         return RC_OK;
     }
-    k_sample_area<<<nblocks(n, 256), 256, 0, s>>>(h->V, h->F, h->T, h->cdf, h->fnorm, n, p->seed,
-                                                  P, N, face, weight);
+    const auto kernel = n > 128 * (int64_t)device_sms() ? k_sample_area<true> : k_sample_area<false>;
+    kernel<<<nblocks(n, 256), 256, 0, s>>>(h->V, h->F, h->T, h->cdf, h->host_sc.total, h->fnorm, n, p->seed, P, N, face,
+                                           weight);
     RC_LAUNCHED();
     return RC_OK;
 }

@@ -63,6 +63,7 @@ constexpr size_t kVarScratchBytes = kVarPartOffset + 2 * sizeof(double) * kVarMa
 // ---------------------------------------------------------------------------
 struct DevScalars {
     unsigned long long amax_bits;  // max face area (FP64 bits, >= 0)
+    long long total;               // total quantised area
     int cmin[3], cmax[3];          // box-centre bounds (orderable float ints)
     int vmaxabs;                   // max |coordinate| (orderable float int)
     int err_index;                 // first bad face (index out of range), else -1
