@@ -224,11 +224,11 @@ __device__ __noinline__ int tri_test_close(const Ray& r, const float4 v0, const 
 // sign decision (used for rays that only ambiguous pairs decide).
 struct Pair64 { int state; bool hit64; };
 
-// kQuick ends early, after a third of the work, for most pairs; the cast of
-// hemisphere rays, which calls it 5 times in 10,000, takes the form that costs
-// its kernel fewer registers (2% of the impeller's time).
+// kQuick ends early, after a third of the work, for most pairs; the casts of
+// hemisphere rays, which call it 5 times in 10,000, take the form that costs
+// their kernels fewer registers (2% of the impeller's time).
 template <bool kQuick>
-__device__ __noinline__ Pair64 retest64(float ox, float oy, float oz, float dx, float dy, float dz, const float4 v0,
+__device__ __forceinline__ Pair64 retest64_of(float ox, float oy, float oz, float dx, float dy, float dz, const float4 v0,
                                         const float4 v1, const float4 v2)
 {
     const double o[3] = {ox, oy, oz}, d[3] = {dx, dy, dz};
@@ -314,9 +314,19 @@ __device__ __noinline__ Pair64 retest64(float ox, float oy, float oz, float dx, 
     return res;
 }
 
-__device__ __forceinline__ Pair64 retest64(const Ray& r, const float4 v0, const float4 v1, const float4 v2)
+template <bool kQuick>
+__device__ __noinline__ Pair64 retest64(float ox, float oy, float oz, float dx, float dy, float dz, const float4 v0,
+                                        const float4 v1, const float4 v2)
 {
-    return retest64<true>(r.ox, r.oy, r.oz, r.dx, r.dy, r.dz, v0, v1, v2);
+    return retest64_of<kQuick>(ox, oy, oz, dx, dy, dz, v0, v1, v2);
+}
+
+// of a ray by itself in its lane: passed by reference (its six values in
+// registers cost the walk around the call more spills: binary walk, housing,
+// 20k points x 1024 directions, 2.45 ms, 2.70 by value and quick)
+__device__ __noinline__ Pair64 retest64(const Ray& r, const float4 v0, const float4 v1, const float4 v2)
+{
+    return retest64_of<false>(r.ox, r.oy, r.oz, r.dx, r.dy, r.dz, v0, v1, v2);
 }
 
 // Conservative slab test of both children of a packed node.
@@ -975,6 +985,9 @@ __device__ __forceinline__ bool eligible(float nx, float ny, float nz, float dx,
 #endif
 #ifndef RC_AXIS_MIN_BLOCKS
 #define RC_AXIS_MIN_BLOCKS 5
+#endif
+#ifndef RC_BATCH_MIN_BLOCKS
+#define RC_BATCH_MIN_BLOCKS 5
 #endif
 #ifndef RC_TAIL_SPLITS
 #define RC_TAIL_SPLITS 4
@@ -1655,7 +1668,7 @@ __device__ __forceinline__ bool trace_axis(const float4* __restrict__ ftree, con
                 if (st == kUnsure) st = tri_test_close(q, v0, v1, v2);
                 if (st == kUnsure) {
                     ++acc.retests;
-                    const Pair64 w = retest64(q, v0, v1, v2);
+                    const Pair64 w = retest64<true>(q.ox, q.oy, q.oz, q.dx, q.dy, q.dz, v0, v1, v2);
                     st = w.state;
                     ua = st == kUnsure;
                     uh = ua && w.hit64;
@@ -1749,6 +1762,12 @@ __device__ __forceinline__ void cast_point_binary(const float4* __restrict__ nod
 // tree, pooled on the 4-wide one (with 64-bit pairs on the largest parts).
 enum { kBinary = 0, kWide4 = 1, kWide4Big = 2 };
 
+// Resident blocks per SM of the hemispherical cast.  The binary walk keeps no
+// pool, and what it waits for are loads of its own, one ray a lane: more warps
+// hide them (housing, 20k points x 1024 directions: 2.45 ms with 7, 2.50 and
+// 2.66 with 6 and 5, 2.60 with 8).
+constexpr int hemi_blocks(int kind) { return kind == kBinary ? 7 : RC_HEMI_MIN_BLOCKS; }
+
 // dynamic shared memory of the axis casts (four warps)
 __host__ __device__ __forceinline__ constexpr size_t axis_smem(int kind)
 {
@@ -1801,7 +1820,7 @@ __device__ __forceinline__ void cast_point(const float4* __restrict__ nodes, con
 }
 
 template <bool kStats, int kKind>
-__global__ void __launch_bounds__(128, RC_HEMI_MIN_BLOCKS)
+__global__ void __launch_bounds__(128, hemi_blocks(kKind))
 k_hemisphere(const float4* __restrict__ nodes, const float4* __restrict__ tris, int max_steps, float scene_maxabs,
              const float* __restrict__ P, const float* __restrict__ Nrm, int64_t n,
              const int32_t* __restrict__ order, const float4* __restrict__ tdirs, int n_dirs, double eps,
@@ -2147,10 +2166,6 @@ __device__ __forceinline__ void flush_part_counters(unsigned long long* c, CastA
     warp_add_counters(c, a.rays, a.amb, a.retests, a.overflow);
     a = CastAcc();
 }
-
-#ifndef RC_BATCH_MIN_BLOCKS
-#define RC_BATCH_MIN_BLOCKS 5
-#endif
 
 template <bool kStats, int kKind>
 __global__ void __launch_bounds__(128, RC_BATCH_MIN_BLOCKS)
@@ -2505,11 +2520,11 @@ rc_status launch_hemisphere(rc_bvh h, const float* P, const float* N, int64_t n,
         if (st != RC_OK) return st;
     }
     const int threads = 128;
-    const int per_sm = p->blocks_per_sm > 0 ? p->blocks_per_sm : RC_HEMI_MIN_BLOCKS;
+    const int kind = cast_kind(p, h->T);
+    const int per_sm = p->blocks_per_sm > 0 ? p->blocks_per_sm : hemi_blocks(kind);
     int64_t blocks = (int64_t)sm_count() * per_sm;
     if (p->launch_mode == 1) work = nullptr;
     const bool wide = use_wide(p);
-    const int kind = cast_kind(p, h->T);
     const size_t smem = cast_smem(threads / 32, (p->n_dirs + 31) / 32, kind, stats);
     const float4* tree = wide ? h->wnodes : h->nodes;
     {
@@ -2706,12 +2721,12 @@ rc_status launch_orthogonal_frames_into(rc_bvh h, const float* P, const float* N
     RC_CUDA(cudaMemsetAsync(mbits, 0, sizeof(uint32_t) * (mw + 2), s));
     unsigned long long* work = (unsigned long long*)(mbits + mw);
     const int64_t items = (int64_t)nf * 6 * ((n + 31) / 32);
+    const int kind = cast_kind(p, h->T);
     const int64_t cap = (int64_t)sm_count() * RC_AXIS_MIN_BLOCKS;
     int64_t blocks = (items + 3) / 4;
     if (blocks > cap && p->launch_mode == 0) blocks = cap;
     if (p->launch_mode == 1) work = nullptr;
     const float4* tree = use_wide(p) ? h->wnodes : h->nodes;
-    const int kind = cast_kind(p, h->T);
     const auto run = [&](auto kernel) {
         kernel<<<(unsigned)blocks, 128, axis_smem(kind), s>>>(tree, h->tris, max_steps(h), h->scene_maxabs, P, N, n, order,
                                                              fds, nf, p->origin_offset, p->parallel_tol, mbits, travel,
@@ -2787,10 +2802,10 @@ rc_status launch_tool_cast(rc_bvh h, const float* P, const float* N, int64_t n, 
     if (st == RC_OK && order) st = point_order(h, P, n, order, s);
     if (st == RC_OK) {
         int64_t blocks = (6 * ((n + 31) / 32) + 3) / 4;
+        const int kind = cast_kind(p, h->T);
         const int64_t cap = (int64_t)sm_count() * RC_AXIS_MIN_BLOCKS;
         if (blocks > cap) blocks = cap;
         unsigned long long* work = (unsigned long long*)(mbits + mw);
-        const int kind = cast_kind(p, h->T);
         const auto kernel = kind == kWide4 ? k_tool_cast_axis<kWide4> : kind == kBinary ? k_tool_cast_axis<kBinary>
                                                                                       : k_tool_cast_axis<kWide4Big>;
         kernel<<<(unsigned)blocks, 128, axis_smem(kind), s>>>(use_wide(p) ? h->wnodes : h->nodes, h->tris, max_steps(h),
