@@ -1986,11 +1986,12 @@ constexpr int kUpdateQueue = 64;       // rays that wait, per warp
 // left the slab test of the rays decides as before; a tile alone filled 5 to
 // 10 lanes of a walk.  Near points are handed out a few tiles at a time, and
 // first: whole, with a thousand rays each, they were a tail of half the time.
-// The margin of the cones covers the slab test's
-// rounding (4e-7 of a distance) and normals off unit length (tilt 3 delta,
-// delta <= 0.004 / W).  Bound by the walks.  Edit of one blade, 1.93M
-// triangles, 200k points x 1024 directions: 1776 -> 730 us with the two
-// kernels beside it.
+// A tile of a point on a moved face is 32 rays already and walks as it is
+// (everything moved, 20k points x 512 directions: 1.53 ms, by way of the queue
+// 1.58).  The margin of the cones covers the slab test's rounding (4e-7 of a
+// distance) and normals off unit length (tilt 3 delta, delta <= 0.004 / W).
+// Bound by the walks.  Edit of one blade, 1.93M triangles, 200k points x 1024
+// directions: 1776 -> 730 us with the two kernels beside it.
 template <bool kWide>
 __global__ void __launch_bounds__(128, RC_UPDATE_MIN_BLOCKS)
 k_hemisphere_update(const float4* __restrict__ nodes, const float4* __restrict__ tris, int max_steps,
@@ -2031,29 +2032,19 @@ k_hemisphere_update(const float4* __restrict__ nodes, const float4* __restrict__
     unsigned todo = 0;                     // of tiles [t0 - 32, t0): those left
     float bx = 0.0f, by = 0.0f, bz = 0.0f, ca = 0.0f, sa = 0.0f;   // the box's cone in the point's basis
     for (;;) {
+        float4 o, d;                       // the ray to walk: from the queue, or of a tile that is cast in full
+        bool walk = false;
         if (qn >= 32 || (qn > 0 && !more)) {
             const int m = min(32, qn);
             qn -= m;
-            if (lane < m) {
-                const float4 o = ray_o[qn + lane], d = ray_d[qn + lane];
-                const int j = __float_as_int(d.w) & 0xFFFF;
-                Ray r;
-                setup_ray(r, o.x, o.y, o.z, d.x, d.y, d.z, scene_maxabs);
-                const TraceOut tr = trace_any<false, kWide>(nodes, tris, r, max_steps);
-                acc.retests += tr.retests;
-                acc.overflow += tr.overflow;
-                acc.amb += (tr.flags >> 1) & 1;
-                acc.rays += 1;
-                const int64_t at = (int64_t)__float_as_uint(o.w) | (int64_t)(__float_as_uint(d.w) >> 16) << 32;
-                uint32_t* row = bits + at * W + (j >> 5);
-                if ((tr.flags & 1) == 0) atomicOr(row, 1u << (j & 31));
-                else atomicAnd(row, ~(1u << (j & 31)));
+            walk = lane < m;
+            if (walk) {
+                o = ray_o[qn + lane];
+                d = ray_d[qn + lane];
             }
-            __syncwarp();
-            continue;
-        }
-        if (!more) break;
-        if (todo == 0) {
+        } else if (!more) {
+            break;
+        } else if (todo == 0) {
             if (t0 >= t1) {
                 // the next item
                 unsigned long long k = 0;
@@ -2107,27 +2098,49 @@ k_hemisphere_update(const float4* __restrict__ nodes, const float4* __restrict__
             todo = __ballot_sync(kAll, in);
             t0 += 32;
             continue;
+        } else {
+            const int t = t0 - 32 + __ffs(todo) - 1;
+            todo &= todo - 1;
+            const float4 h = __ldg(&tdirs[32 * t + lane]);
+            const float4 cx = onb[0], cy = onb[1], cz = onb[2];
+            const Onb b = {cx.x, cy.x, cz.x, cx.y, cy.y, cz.y};
+            float dx, dy, dz;
+            local_to_world(b, cx.z, cy.z, cz.z, h.x, h.y, h.z, dx, dy, dz);
+            bool on = __float_as_int(h.w) >= 0;
+            if (!full && on) {
+                Ray r;
+                setup_ray(r, cx.w, cy.w, cz.w, dx, dy, dz, scene_maxabs);
+                on = ray_enters_box(r, blo, bhi);       // otherwise it keeps its old bit
+            }
+            o = make_float4(cx.w, cy.w, cz.w, __uint_as_float((unsigned)i));
+            d = make_float4(dx, dy, dz, __int_as_float(__float_as_int(h.w) | (int)(i >> 32) << 16));   // j < 65536
+            if (!full) {
+                const unsigned m = __ballot_sync(kAll, on);
+                if (on) {
+                    const int at = qn + __popc(m & below);
+                    ray_o[at] = o;
+                    ray_d[at] = d;
+                }
+                qn += __popc(m);
+                __syncwarp();
+                continue;
+            }
+            walk = on;
         }
-        const int t = t0 - 32 + __ffs(todo) - 1;
-        todo &= todo - 1;
-        const float4 h = __ldg(&tdirs[32 * t + lane]);
-        const float4 cx = onb[0], cy = onb[1], cz = onb[2];
-        const Onb b = {cx.x, cy.x, cz.x, cx.y, cy.y, cz.y};
-        float dx, dy, dz;
-        local_to_world(b, cx.z, cy.z, cz.z, h.x, h.y, h.z, dx, dy, dz);
-        bool on = __float_as_int(h.w) >= 0;
-        if (!full && on) {
+        if (walk) {
+            const int j = __float_as_int(d.w) & 0xFFFF;
             Ray r;
-            setup_ray(r, cx.w, cy.w, cz.w, dx, dy, dz, scene_maxabs);
-            on = ray_enters_box(r, blo, bhi);           // otherwise it keeps its old bit
+            setup_ray(r, o.x, o.y, o.z, d.x, d.y, d.z, scene_maxabs);
+            const TraceOut tr = trace_any<false, kWide>(nodes, tris, r, max_steps);
+            acc.retests += tr.retests;
+            acc.overflow += tr.overflow;
+            acc.amb += (tr.flags >> 1) & 1;
+            acc.rays += 1;
+            const int64_t at = (int64_t)__float_as_uint(o.w) | (int64_t)(__float_as_uint(d.w) >> 16) << 32;
+            uint32_t* row = bits + at * W + (j >> 5);
+            if ((tr.flags & 1) == 0) atomicOr(row, 1u << (j & 31));
+            else atomicAnd(row, ~(1u << (j & 31)));
         }
-        const unsigned m = __ballot_sync(kAll, on);
-        if (on) {
-            const int at = qn + __popc(m & below);
-            ray_o[at] = make_float4(cx.w, cy.w, cz.w, __uint_as_float((unsigned)i));
-            ray_d[at] = make_float4(dx, dy, dz, __int_as_float(__float_as_int(h.w) | (int)(i >> 32) << 16));   // j < 65536
-        }
-        qn += __popc(m);
         __syncwarp();
     }
     warp_add_counters(counters, acc.rays, acc.amb, acc.retests, acc.overflow);
