@@ -92,7 +92,7 @@ static std::vector<int32_t> tile_order(int32_t N, const float* h)
         const double z = 1.0 - ((double)j + 0.5) / (double)N;
         const double s = sqrt(std::max(0.0, 1.0 - z * z));
         int32_t m = (int32_t)llround(s * sqrt(2.0 * M_PI * (double)N / (32.0 * kTileAspect)));
-        m = std::max(1, std::min(m, ntiles - t));
+        m = std::max(1, std::min({m, ntiles - t, (int32_t)kMaxBand}));
         key.clear();
         for (int32_t k = j; k < j + 32 * m; ++k) {
             const double phi = atan2((double)h[3 * k + 1], (double)h[3 * k]);

@@ -973,10 +973,12 @@ __device__ __forceinline__ bool eligible(float nx, float ny, float nz, float dx,
 // warp's shared-memory row, which is written out in canonical order once the
 // point is done.
 // ---------------------------------------------------------------------------
-// 5 blocks of 4 warps: 96 registers without spills, and the 32 KB a block
-// keeps in shared memory leave L1 about 90 KB.  4 and 6 blocks measured 32.5
-// and 34.4 ms against 31.1 on the impeller (100k points x 2048), 5.99 and
-// 6.08 against 5.85 on the housing (100k x 1024).
+// 5 blocks of 4 warps of the pooled walk: 96 registers with some 100 bytes of
+// spills, and the 25 KB of pools and 12 bytes per warp and word of directions
+// that a block keeps in shared memory leave L1 85 KB at 2,048 directions.  4
+// and 6 blocks measured 30.1 and 31.3 ms against 27.0 on the impeller (100k
+// points x 2048).  Five fit an SM up to 13,300 directions, three up to 34,112,
+// and beyond that a point is cast in segments (kSegTiles), five again.
 #ifndef RC_HEMI_MIN_BLOCKS
 #define RC_HEMI_MIN_BLOCKS 5
 #endif
@@ -1113,6 +1115,17 @@ __device__ __forceinline__ void pool_back(Pair* pair, int& sp, Pair* store, int&
 // pair that FP64 calls a hit, and (instrumented cast) re-tested in FP64
 __host__ __device__ __forceinline__ constexpr int pool_rows(bool stats) { return stats ? 4 : 3; }
 
+// A point of more than kWholeWords words of directions is cast in segments of
+// kSegTiles tiles, whose rows hold the words that the segment's tiles reach:
+// a band of the tile order has as many tiles as words, the same ones, and at
+// most kMaxBand.  Up to kWholeWords three blocks with whole rows fit an SM;
+// with 65,536 directions it was one (6,000 points of the housing 51.4 ms, now
+// 21.1; 49,152 directions, 500 points, 3.07 and 2.67).  Segments from the
+// words on at which five blocks fit no more would gain nothing: their kernel
+// spills more (10,000 x 32,768: 19.6 ms whole, 20.2; 20,000 x 16,384: 15.3 and
+// 15.8), and so would one kernel for both (4,096 directions 10% slower).
+constexpr int kSegTiles = 256, kSegWords = kSegTiles + 2 * kMaxBand, kWholeWords = 1066;
+
 // FP32 decision of one pair by signed volumes (Moeller and Trumbore 1997),
 // with a forward error bound; kHit and kMiss only when certain, as
 // tri_test32.  With s = A - o, e1 = B - A, e2 = C - A, p = d x e2 and
@@ -1213,42 +1226,43 @@ __device__ __forceinline__ TileAxis tile_axis(float x)
 // tp) that FP32 left open; true for a clear hit.  Not inlined: it is rare.
 template <bool kStats>
 __device__ __noinline__ bool pool_retest(float ox, float oy, float oz, const float4 d, int j, const float4* tp,
-                                         uint32_t* rows, int W, int64_t i, long long* relist, long long relist_cap,
+                                         uint32_t* rows, int R, int64_t i, long long* relist, long long relist_cap,
                                          unsigned long long* relist_ctr)
 {
     const Pair64 q = retest64<false>(ox, oy, oz, d.x, d.y, d.z, tp[0], tp[1], tp[2]);
     const uint32_t b = 1u << (j & 31);
-    if (kStats && relist && !(atomicOr(&rows[3 * W + (j >> 5)], b) & b)) {
+    if (kStats && relist && !(atomicOr(&rows[3 * R + (j >> 5)], b) & b)) {
         const unsigned long long at = atomicAdd(relist_ctr, 1ULL);
         if (at < (unsigned long long)relist_cap) relist[at] = (long long)i * 65536 + j;
     }
     if (q.state == kUnsure) {
-        atomicOr(&rows[W + (j >> 5)], b);
-        if (q.hit64) atomicOr(&rows[2 * W + (j >> 5)], b);
+        atomicOr(&rows[R + (j >> 5)], b);
+        if (q.hit64) atomicOr(&rows[2 * R + (j >> 5)], b);
     }
     return q.state == kHit;
 }
 
 // cast_point on the 4-wide tree (same arguments; pool and rows: the warp's
 // shared memory)
-template <bool kStats, bool kBig>
+template <bool kStats, bool kBig, bool kSeg>
 __device__ __forceinline__ void cast_point_pooled(const float4* __restrict__ wnodes, const float4* __restrict__ tris,
                                                   int max_steps, float scene_maxabs, const float* __restrict__ P,
                                                   const float* __restrict__ Nrm, int64_t i,
                                                   const float4* __restrict__ tdirs, int W, double eps,
                                                   PoolOf<kBig>* pool, uint32_t* rows, uint32_t* __restrict__ bits,
                                                   int32_t* __restrict__ count, CastAcc& acc, int t0, int t1,
-                                                  long long* relist, long long relist_cap,
+                                                  bool whole, long long* relist, long long relist_cap,
                                                   unsigned long long* relist_ctr)
 {
     using Pair = PairOf<kBig>;
     constexpr unsigned kAll = 0xFFFFFFFFu;
     const int lane = threadIdx.x & 31;
     const unsigned below = (1u << lane) - 1u;
-    const bool whole = t1 < 0;
-    if (whole) t1 = W;
+    // the rows hold words [w0, w1), R words apart, and start at word w0
+    const int R = kSeg ? kSegWords : W, w0 = kSeg ? max(0, t0 - kMaxBand) : 0, w1 = kSeg ? min(W, t1 + kMaxBand) : W;
+    for (int w = lane; w < pool_rows(kStats) * R; w += 32) rows[w] = 0u;
+    rows -= w0;
     uint32_t* vis = rows;
-    for (int w = lane; w < pool_rows(kStats) * W; w += 32) rows[w] = 0u;
     Frontier* f = &pool->front;
     float ox, oy, oz;
     {
@@ -1410,7 +1424,7 @@ __device__ __forceinline__ void cast_point_pooled(const float4* __restrict__ wno
                     int st = tri_test_mt(ox, oy, oz, rd.x, rd.y, rd.z, rd.w, rs, __ldg(tp), __ldg(tp + 1), __ldg(tp + 2));
                     if (st == kUnsure) {
                         acc.retests += 1;
-                        if (pool_retest<kStats>(ox, oy, oz, rd, __float_as_int(pool->inv[slot].w), tp, rows, W, i, relist,
+                        if (pool_retest<kStats>(ox, oy, oz, rd, __float_as_int(pool->inv[slot].w), tp, rows, R, i, relist,
                                                 relist_cap, relist_ctr))
                             st = kHit;
                     }
@@ -1468,7 +1482,7 @@ __device__ __forceinline__ void cast_point_pooled(const float4* __restrict__ wno
                                  f->tri[3 * k + 2]);
             if (st == kUnsure) {
                 acc.retests += 1;
-                if (pool_retest<kStats>(ox, oy, oz, rd, jt, &f->tri[3 * k], rows, W, i, relist, relist_cap, relist_ctr))
+                if (pool_retest<kStats>(ox, oy, oz, rd, jt, &f->tri[3 * k], rows, R, i, relist, relist_cap, relist_ctr))
                     st = kHit;
             }
             open = st != kHit;
@@ -1511,10 +1525,10 @@ __device__ __forceinline__ void cast_point_pooled(const float4* __restrict__ wno
     }
     // visible, less the rays that only an FP64-ambiguous pair blocks
     int cnt = 0;
-    for (int w = lane; w < W; w += 32) {
+    for (int w = w0 + lane; w < w1; w += 32) {
         const uint32_t v = vis[w];
-        acc.amb += __popc(v & rows[W + w]);
-        const uint32_t r = v & ~rows[2 * W + w];
+        acc.amb += __popc(v & rows[R + w]);
+        const uint32_t r = v & ~rows[2 * R + w];
         cnt += __popc(r);
         if (whole)
             bits[i * W + w] = r;
@@ -1760,7 +1774,9 @@ __device__ __forceinline__ void cast_point_binary(const float4* __restrict__ nod
 
 // One point by one warp, by the tree's kind: a ray per lane on the binary
 // tree, pooled on the 4-wide one (with 64-bit pairs on the largest parts).
-enum { kBinary = 0, kWide4 = 1, kWide4Big = 2 };
+enum { kBinary = 0, kWide4 = 1, kWide4Big = 2, kWide4Seg = 3, kWide4BigSeg = 4 };   // Seg: in segments (point casts)
+__host__ __device__ constexpr bool is_big(int kind) { return kind == kWide4Big || kind == kWide4BigSeg; }
+__host__ __device__ constexpr bool is_seg(int kind) { return kind >= kWide4Seg; }
 
 // Resident blocks per SM of the hemispherical cast.  The binary walk keeps no
 // pool, and what it waits for are loads of its own, one ray a lane: more warps
@@ -1775,18 +1791,18 @@ __host__ __device__ __forceinline__ constexpr size_t axis_smem(int kind)
 }
 
 // Dynamic shared memory of the point casts: each warp's pool (4-wide tree),
-// then each warp's bit rows of W words.
-__host__ __device__ __forceinline__ constexpr int cast_rows(int kind, bool stats)
+// then each warp's bit rows of W words (of a segment's: kSegWords).
+__host__ __device__ __forceinline__ constexpr int cast_words(int kind, int W, bool stats)
 {
-    return kind == kBinary ? 1 : pool_rows(stats);
+    return kind == kBinary ? W : pool_rows(stats) * (is_seg(kind) ? kSegWords : W);
 }
 __host__ __device__ __forceinline__ constexpr size_t pool_bytes(int kind)
 {
-    return kind == kBinary ? 0 : kind == kWide4 ? sizeof(PoolOf<false>) : sizeof(PoolOf<true>);
+    return kind == kBinary ? 0 : is_big(kind) ? sizeof(PoolOf<true>) : sizeof(PoolOf<false>);
 }
 __host__ __device__ __forceinline__ size_t cast_smem(int warps, int W, int kind, bool stats)
 {
-    return warps * pool_bytes(kind) + (size_t)warps * W * cast_rows(kind, stats) * sizeof(uint32_t);
+    return warps * (pool_bytes(kind) + cast_words(kind, W, stats) * sizeof(uint32_t));
 }
 
 // Let a kernel have the shared memory of the most directions.  The limit
@@ -1796,7 +1812,7 @@ template <class Kernel>
 static cudaError_t allow_cast_smem(Kernel kernel, int warps, int kind, bool stats)
 {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)cast_smem(warps, kMaxDirs / 32, kind, stats));
+                                (int)cast_smem(warps, kind == kWide4 || kind == kWide4Big ? kWholeWords : kMaxDirs / 32, kind, stats));
 }
 
 template <bool kStats, int kKind>
@@ -1809,14 +1825,29 @@ __device__ __forceinline__ void cast_point(const float4* __restrict__ nodes, con
                                            long long relist_cap = 0, unsigned long long* relist_ctr = nullptr)
 {
     const int warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
-    uint32_t* rows = (uint32_t*)(smem + warps * pool_bytes(kKind)) + warp * W * cast_rows(kKind, kStats);
-    if (kKind == kBinary)
+    uint32_t* rows = (uint32_t*)(smem + warps * pool_bytes(kKind)) + warp * cast_words(kKind, W, kStats);
+    if (kKind == kBinary) {
         cast_point_binary<kStats>(nodes, tris, max_steps, scene_maxabs, P, Nrm, i, tdirs, W, eps, rows, bits, count,
                                   acc, t0, t1, relist, relist_cap, relist_ctr);
-    else
-        cast_point_pooled<kStats, kKind == kWide4Big>(nodes, tris, max_steps, scene_maxabs, P, Nrm, i, tdirs, W, eps,
-                                                      (PoolOf<kKind == kWide4Big>*)smem + warp, rows, bits, count, acc,
-                                                      t0, t1, relist, relist_cap, relist_ctr);
+        return;
+    }
+    const bool whole = t1 < 0;
+    if (whole) t1 = W;
+    auto* pool = (PoolOf<is_big(kKind)>*)smem + warp;
+    if (!is_seg(kKind)) {
+        cast_point_pooled<kStats, is_big(kKind), false>(nodes, tris, max_steps, scene_maxabs, P, Nrm, i, tdirs, W, eps, pool,
+                                                        rows, bits, count, acc, t0, t1, whole, relist, relist_cap, relist_ctr);
+        return;
+    }
+    if (whole) {                           // the segments add to the point's row and count
+        for (int w = threadIdx.x & 31; w < W; w += 32) bits[i * W + w] = 0u;
+        if ((threadIdx.x & 31) == 0) count[i] = 0;
+        __syncwarp();
+    }
+    for (; t0 < t1; t0 += kSegTiles)
+        cast_point_pooled<kStats, is_big(kKind), true>(nodes, tris, max_steps, scene_maxabs, P, Nrm, i, tdirs, W, eps, pool,
+                                                       rows, bits, count, acc, t0, min(t1, t0 + kSegTiles), false, relist,
+                                                       relist_cap, relist_ctr);
 }
 
 template <bool kStats, int kKind>
@@ -2488,6 +2519,13 @@ static int cast_kind(const rc_params* p, int64_t max_tris)
     return !use_wide(p) ? kBinary : max_tris <= kPairTris ? kWide4 : kWide4Big;
 }
 
+// and, with more directions than a point's rows should hold, in segments
+static int point_kind(const rc_params* p, int64_t max_tris)
+{
+    const int kind = cast_kind(p, max_tris);
+    return kind == kBinary || (p->n_dirs + 31) / 32 <= kWholeWords ? kind : kind == kWide4 ? kWide4Seg : kWide4BigSeg;
+}
+
 static int g_sm_count = 0;
 
 static int sm_count()
@@ -2533,7 +2571,7 @@ rc_status launch_hemisphere(rc_bvh h, const float* P, const float* N, int64_t n,
         if (st != RC_OK) return st;
     }
     const int threads = 128;
-    const int kind = cast_kind(p, h->T);
+    const int kind = point_kind(p, h->T);
     const int per_sm = p->blocks_per_sm > 0 ? p->blocks_per_sm : hemi_blocks(kind);
     int64_t blocks = (int64_t)sm_count() * per_sm;
     if (p->launch_mode == 1) work = nullptr;
@@ -2570,10 +2608,13 @@ rc_status launch_hemisphere(rc_bvh h, const float* P, const float* N, int64_t n,
                                                            work, n - n_split, splits, relist, relist_cap);
             return RC_OK;
         };
+        const auto pick = [&](auto with, auto without) { return run(stats ? with : without); };
         rc_status st = RC_OK;
-        if (kind == kWide4) st = stats ? run(k_hemisphere<true, kWide4>) : run(k_hemisphere<false, kWide4>);
-        else if (kind == kBinary) st = stats ? run(k_hemisphere<true, kBinary>) : run(k_hemisphere<false, kBinary>);
-        else st = stats ? run(k_hemisphere<true, kWide4Big>) : run(k_hemisphere<false, kWide4Big>);
+        if (kind == kWide4) st = pick(k_hemisphere<true, kWide4>, k_hemisphere<false, kWide4>);
+        else if (kind == kBinary) st = pick(k_hemisphere<true, kBinary>, k_hemisphere<false, kBinary>);
+        else if (kind == kWide4Big) st = pick(k_hemisphere<true, kWide4Big>, k_hemisphere<false, kWide4Big>);
+        else if (kind == kWide4Seg) st = pick(k_hemisphere<true, kWide4Seg>, k_hemisphere<false, kWide4Seg>);
+        else st = pick(k_hemisphere<true, kWide4BigSeg>, k_hemisphere<false, kWide4BigSeg>);
         if (st != RC_OK) return st;
     }
     RC_LAUNCHED();
@@ -2841,15 +2882,18 @@ rc_status launch_batch(const BatchPart* d_parts, int n_parts, long long n_items,
                        const rc_params* p, int64_t max_tris, unsigned long long* work, cudaStream_t s)
 {
     const int threads = 128;
-    const int kind = cast_kind(p, max_tris);
+    const int kind = point_kind(p, max_tris);
     const size_t smem = cast_smem(threads / 32, (p->n_dirs + 31) / 32, kind, false);
     const int per_sm = p->blocks_per_sm > 0 ? p->blocks_per_sm : RC_BATCH_MIN_BLOCKS;
     int64_t blocks = (int64_t)sm_count() * per_sm;
     const int64_t need = (n_items * 32 + threads - 1) / threads;
     if (blocks > need) blocks = need;
     if (blocks < 1) blocks = 1;
-    const auto kernel = kind == kWide4 ? k_batch<false, kWide4> : kind == kBinary ? k_batch<false, kBinary>
-                                                                                   : k_batch<false, kWide4Big>;
+    const auto kernel = kind == kWide4      ? k_batch<false, kWide4>
+                        : kind == kBinary   ? k_batch<false, kBinary>
+                        : kind == kWide4Big ? k_batch<false, kWide4Big>
+                        : kind == kWide4Seg ? k_batch<false, kWide4Seg>
+                                            : k_batch<false, kWide4BigSeg>;
     kernel<<<(unsigned)blocks, threads, smem, s>>>(d_parts, n_parts, n_items, ppi, tdirs, p->n_dirs, p->origin_offset,
                                                    work);
     RC_LAUNCHED();
@@ -2861,6 +2905,8 @@ rc_status prepare_batch_kernel()
     RC_CUDA(allow_cast_smem(k_batch<false, kBinary>, 4, kBinary, false));
     RC_CUDA(allow_cast_smem(k_batch<false, kWide4>, 4, kWide4, false));
     RC_CUDA(allow_cast_smem(k_batch<false, kWide4Big>, 4, kWide4Big, false));
+    RC_CUDA(allow_cast_smem(k_batch<false, kWide4Seg>, 4, kWide4Seg, false));
+    RC_CUDA(allow_cast_smem(k_batch<false, kWide4BigSeg>, 4, kWide4BigSeg, false));
     return RC_OK;
 }
 

@@ -48,6 +48,7 @@ constexpr int kStack = 64;         // binary traversal stack entries (>= max tre
 constexpr int kStack4 = 96;        // 4-wide traversal stack entries (>= 3 * wide depth + 1)
 constexpr double kTau = 1e-9;      // relative ambiguity band of the occlusion test
 constexpr int kMaxDirs = 65536;
+constexpr int kMaxBand = 80;       // most tiles of a band of the tile order (66 at kMaxDirs directions)
 
 // scratch of the variability reduction: kVarSums int64 sums, then the two
 // FP64 weighted sums, then the per-block FP64 partials (two rows of
