@@ -489,7 +489,9 @@ def roofline(rc, args, name, dev, stream, ps, cast_s, rays, nodes_per_ray, tris_
     except (OSError, KeyError, ValueError):
         sm_max = 2070.0
     fp32_peak = props.multi_processor_count * 128 * 2 * sm_max * 1e6 / 1e12
-    ops_per_ray = 18.0 * (4.0 if ps.tree_width != 2 else 2.0) * nodes_per_ray + 35.0 * tris_per_ray
+    wide = ps.tree_width != 2
+    tri_ops = 49.0 if wide else 35.0
+    ops_per_ray = 18.0 * (4.0 if wide else 2.0) * nodes_per_ray + tri_ops * tris_per_ray
     fp32_ach = ops_per_ray * rays / cast_s / 1e12
     hbm_peak, peak_src = peaks()
     alg_bytes = bytes_per_ray * rays
@@ -512,8 +514,9 @@ def roofline(rc, args, name, dev, stream, ps, cast_s, rays, nodes_per_ray, tris_
         "algorithmic": {"ops_per_ray": ops_per_ray, "bytes_per_ray": bytes_per_ray, "nodes_per_ray": nodes_per_ray,
                         "tris_per_ray": tris_per_ray, "node_bytes": node_bytes,
                         "tree": "4-wide" if ps.tree_width != 2 else "binary",
-                        "ops_source": "18 per box test (6 FMA counted as 2 each, 5 min/max, 1 compare), 35 per "
-                                      "triangle test (watertight formulas); counts from the instrumented walk"},
+                        "ops_source": "18 per box test (6 FMA counted as 2 each, 5 min/max, 1 compare), %d per "
+                                      "triangle test (%s); counts from the instrumented walk"
+                                      % (tri_ops, "signed volumes" if wide else "watertight formulas")},
         "hbm": {"achieved": hbm_ach, "peak": hbm_peak, "unit": "GB/s", "frac": hbm_ach / hbm_peak,
                 "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs)" if peak_src == "measured" else peak_src,
                 "note": "algorithmic bytes per second; served mostly by L1 and L2, so this can exceed 1"},

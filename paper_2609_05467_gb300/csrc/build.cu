@@ -1647,7 +1647,7 @@ static rc_status build_wide(rc_bvh h, const float* tbox, cudaStream_t s)
 // The 4-wide tree with its child boxes in the coordinates of a machining
 // frame (rows of M = the frame's columns): the same nodes, codes and
 // triangles; each box is the bounding box of the frame coordinates of its
-// triangles' vertices, evaluated in FP64 and rounded outward to fp32.  The
+// triangles' vertices, evaluated in two-term fp32 sums and rounded outward.  The
 // axis walk of the orthogonal cast tests these boxes (its rays run along a
 // frame axis) and still tests triangles in world coordinates.
 // ---------------------------------------------------------------------------

@@ -419,10 +419,6 @@ __device__ __forceinline__ TraceOut trace(const float4* __restrict__ nodes, cons
     return out;
 }
 
-// Any-hit walk of the 4-wide tree: the same ray, box and triangle decisions
-// as trace(); per node the four child boxes are tested together, the
-// nearest hit child is visited next and the others are pushed (the default
-// walk orders them only partly, the while-while walk fully, far-to-near).
 // Per-ray constants of the 4-wide slab test.  A slab distance is one FMA,
 // t = b * i - o * i, with the near / far bound of each axis picked by the
 // load address (the node stores lo and hi of an axis in adjacent float4s).
@@ -516,7 +512,8 @@ __device__ __forceinline__ int slab4(const float4* __restrict__ wnodes, int w, c
 // plane is dropped, because a hemisphere ray leaves that plane (d.n > 0 for
 // every direction of the set, N <= 65536, when n is of unit length to within
 // the rounding of an fp32 normal) and meets no point of it at t > 0; that
-// exact FP64 test runs once per point.  For the same reason a frontier box
+// test runs once per point, in fp32 where its sign is clear and in FP64
+// otherwise.  For the same reason a frontier box
 // wholly below the plane is dropped, and so is a frontier leaf whose
 // triangles all lie below it (conservative fp32 tests).  Large boxes then
 // make way for their children's while there is room (see build_frontier),
@@ -629,7 +626,7 @@ __device__ __noinline__ void build_frontier(const float4* __restrict__ wnodes, c
         // a box below the tangent plane holds no hit of any ray of the point
         if (out && drop && box_below_tangent(lx, hx, ly, hy, lz, hz, ox, oy, oz, nx, ny, nz)) out = false;
         // leaves: a triangle of one that contains o becomes a local triangle
-        // unless it lies below the plane (FP64); one that does not is dropped
+        // unless it lies below the plane; one that does not is dropped
         // when all its triangles do (fp32)
         const int first = leaf_first(code), cnt = box && code < 0 && (in || (out && drop)) ? leaf_count(code) : 0;
         bool above = !(out && drop && code < 0);
@@ -803,16 +800,18 @@ __device__ __noinline__ void build_frontier(const float4* __restrict__ wnodes, c
     __syncwarp();
 }
 
-// Any-hit walk of the subtree at wide node `start` (0: the whole tree) by one
-// lane, with its stack in local memory.
+// Any-hit walk of the 4-wide tree by one lane, with its stack in local memory:
+// the same ray, box and triangle decisions as trace(); per node the four child
+// boxes are tested together, the nearest hit child is visited next and the
+// others are pushed partly ordered.
 template <bool kStats>
 __device__ __forceinline__ TraceOut trace4(const float4* __restrict__ wnodes, const float4* __restrict__ tris,
-                                           const Ray& r, int max_steps, int start = 0)
+                                           const Ray& r, int max_steps)
 {
     TraceOut out = {0, 0, 0, 0, 0};
     int stack[kStack4];
     int sp = 0;
-    int cur = start;
+    int cur = 0;
     bool amb = false, ambhit = false;
     const SlabRay sr = make_slab_ray(r, r.rs);
     for (int steps = 0;; ++steps) {
@@ -1073,7 +1072,7 @@ struct PairOf<true> {
     __device__ __forceinline__ int slot() const { return s; }
 };
 constexpr int64_t kPairTris = 1 << 24;     // most triangles of 32-bit pairs (leaves of 2, nodes fewer)
-static_assert(kLeafBits == 1, "a leaf code of 2^24 triangles has 26 bits with its sign");
+static_assert(kLeafMax == 2, "a leaf code of 2^24 triangles has 26 bits with its sign; a leaf adds two pairs at most");
 
 template <bool kBig>
 struct __align__(16) PoolOf {
@@ -2683,7 +2682,6 @@ __global__ void k_frame_init(const __grid_constant__ FrameArgs a, FrameDev* fram
         };
         const double gram = product(j, k);
         d->frame[t] = (double)f[t];
-        d->gram[t] = gram;
         // its rounding, 1e-15 of the columns' lengths at most, is on top
         d->gram_up[t] = __double2float_ru(fabs(gram) + 1e-15 * sqrt(product(j, j)) * sqrt(product(k, k)));
         if (j == k) d->rlen[j] = __double2float_ru(1.01 / sqrt(gram));
@@ -2691,12 +2689,10 @@ __global__ void k_frame_init(const __grid_constant__ FrameArgs a, FrameDev* fram
     if (t < 18) d->axes[t] = (t / 3) & 1 ? -f[3 * k + t / 6] : f[3 * k + t / 6];
     if (t < 6) d->box[t] = t < 3 ? 0x7FFFFFFFFFFFFFFFLL : (long long)0x8000000000000000ULL;
     if (t < 3) {
-        d->sc_c[t] = a.sc_c[t];
         d->c32[t] = __double2float_rn(a.sc_c[t]);
     }
     if (t == 0) {
         d->tree = a.tree[blockIdx.x];
-        d->sc_r = a.sc_r;
         d->r32 = __double2float_ru(a.sc_r);
         d->done = 0;
     }

@@ -35,15 +35,10 @@ void count_launch(int k = 1);
 // ---------------------------------------------------------------------------
 // constants
 // ---------------------------------------------------------------------------
-#ifndef RC_LEAF_MAX
-#define RC_LEAF_MAX 2
-#endif
-constexpr int kLeafMax = RC_LEAF_MAX;   // triangles per packed leaf (1..8)
-constexpr int kLeafBits = kLeafMax <= 2 ? 1 : 3;   // leaf codes: -1 - (first << kLeafBits | count - 1)
-static_assert(kLeafMax <= 8, "a leaf code has at most three bits for its count");
-__host__ __device__ __forceinline__ int leaf_code(int first, int cnt) { return -1 - ((first << kLeafBits) | (cnt - 1)); }
-__host__ __device__ __forceinline__ int leaf_first(int code) { return (-1 - code) >> kLeafBits; }
-__host__ __device__ __forceinline__ int leaf_count(int code) { return ((-1 - code) & ((1 << kLeafBits) - 1)) + 1; }
+constexpr int kLeafMax = 2;        // triangles per packed leaf; codes: -1 - (first << 1 | count - 1)
+__host__ __device__ __forceinline__ int leaf_code(int first, int cnt) { return -1 - ((first << 1) | (cnt - 1)); }
+__host__ __device__ __forceinline__ int leaf_first(int code) { return (-1 - code) >> 1; }
+__host__ __device__ __forceinline__ int leaf_count(int code) { return ((-1 - code) & 1) + 1; }
 constexpr int kStack = 64;         // binary traversal stack entries (>= max tree depth)
 constexpr int kStack4 = 96;        // 4-wide traversal stack entries (>= 3 * wide depth + 1)
 constexpr double kTau = 1e-9;      // relative ambiguity band of the occlusion test
@@ -90,13 +85,12 @@ struct FrameDev {
     double fbox[6];     // frame-coordinate bounding box of the vertices (lo xyz, hi xyz)
     long long box[6];   // ordered-integer accumulators for fbox
     const float4* tree; // 4-wide tree with child boxes in frame coordinates (the world tree for the identity)
-    double gram[9];     // G = F^T F of the fp32 frame F (FP64): how far the axes are from orthonormal
-    double sc_c[3];     // centre of the part's bounding box (world)
-    double sc_r;        // half its diagonal
-    float gram_up[9];   // |G| rounded up, 1.01 / |column k|, and the centre and
-    float rlen[3];      //   half diagonal in fp32: the axis rays' bands are
-    float c32[3];       //   bounds, evaluated in fp32 (GB300 issues FP64 at
-    float r32;          //   1/64 of its fp32 rate)
+    // the axis rays' bands are bounds, evaluated in fp32 (GB300 issues FP64 at
+    // 1/64 of its fp32 rate)
+    float gram_up[9];   // |G| rounded up, G = F^T F of the fp32 frame F: how far the axes are from orthonormal
+    float rlen[3];      // 1.01 / |column k|
+    float c32[3];       // centre of the part's bounding box (world)
+    float r32;          // half its diagonal
 };
 
 // one part of a batched cast (device descriptor)
@@ -164,7 +158,7 @@ struct rc_bvh_s {
     int32_t* child = nullptr;      // [n_int][2] combined indices (leaf k -> n_int+k)
     int32_t* range = nullptr;      // [n_int][2] first,last sorted leaf
     int32_t* order = nullptr;      // [T] original face id of sorted slot
-    float* nbox = nullptr;         // [n_int + T][6] boxes (lo xyz, hi xyz)
+    float* nbox = nullptr;         // [n_int + T][6], scratch of the refit: only boxes that meet across its blocks are written
     int32_t* visits = nullptr;     // [n_int] refit arrival counters
     float* fnorm = nullptr;        // [T][3] fp32 unit normals
     double* farea = nullptr;       // [T] FP64 areas
