@@ -681,6 +681,16 @@ __global__ void k_ploc_scatter(const int* __restrict__ n_ptr, const int* __restr
     for (int c = 0; c < 6; ++c) cb_out[6 * (int64_t)pos + c] = cb_tmp[6 * (int64_t)i + c];
 }
 
+// An arrival: what the thread wrote before is seen by the one that arrives
+// second, and that one's reads come after.  (With a fence on either side of a
+// plain exchange a refit of 1.93M triangles took 630 us, so 603.)
+__device__ __forceinline__ int exchange_acq_rel(int32_t* p, int v)
+{
+    int old;
+    asm volatile("atom.acq_rel.gpu.global.exch.b32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
+    return old;
+}
+
 // subtree sizes (leaves, interior nodes) bottom-up with arrival counters;
 // sizes of raw interior id p at sz_leaf[p], sz_int[p]
 __global__ void k_ploc_sizes(int64_t T, int64_t n_int, const int32_t* __restrict__ parent_raw,
@@ -692,8 +702,7 @@ __global__ void k_ploc_sizes(int64_t T, int64_t n_int, const int32_t* __restrict
     int32_t p = parent_raw[n_int + k];
     for (int steps = 0; p >= 0; ++steps) {
         if (steps > kMaxWalk) { atomicExch(err, 1); return; }
-        __threadfence();
-        if (atomicAdd(&visits[p], 1) == 0) return;
+        if (exchange_acq_rel(&visits[p], 1) == 0) return;
         const int32_t a = child_raw[2 * p], b = child_raw[2 * p + 1];
         const int la = a >= n_int ? 1 : __ldcg(&sz_leaf[a]), lb = b >= n_int ? 1 : __ldcg(&sz_leaf[b]);
         const int ia = a >= n_int ? 0 : __ldcg(&sz_int[a]), ib = b >= n_int ? 0 : __ldcg(&sz_int[b]);
@@ -780,13 +789,13 @@ __device__ __forceinline__ bool gather_tri(const float* __restrict__ V, int64_t 
 // first one's box and both heights, and goes on.  A node whose leaves all
 // belong to one block (255 of 256 do) meets in shared memory, at the place of
 // its split (the last leaf of its left subtree, which no other node has).
-// The others meet in global memory: a fence, an exchange, a fence and a read
-// back, a microsecond or two per level; that chain bounds a small tree, and the boxes'
-// traffic a large one.  kPack: the packed binary nodes are written on the way
-// (both children's boxes are at hand), and `sc` receives the tree's depth and
-// box at the root; otherwise every node's box goes to nbox.  The arrival word
-// of a node holds 1 + the first arrival's height, so depth needs no walk of
-// its own.
+// The others meet in global memory: an exchange that orders both sides and a
+// read back, a microsecond or two per level; that chain bounds a small tree,
+// and the boxes' traffic a large one.  kPack: the packed binary nodes are
+// written on the way (both children's boxes are at hand), and `sc` receives the
+// tree's depth and box at the root; otherwise every node's box goes to nbox.
+// The arrival word of a node holds 1 + the first arrival's height, so depth
+// needs no walk of its own.
 constexpr int kClimb = 256;        // leaves (threads) per block
 struct ClimbShared {
     float box[2][6][kClimb];       // of the left and the right child, by split
@@ -842,10 +851,9 @@ __device__ __forceinline__ void climb(ClimbShared& sm, bool leaf, int64_t T, int
             height = max(height, *(volatile int*)&sm.height[1 - me][at]) + 1;
         } else {
             if (kPack) put_box(nbox, cur, lo, hi);      // (else it is there)
-            __threadfence();
-            const int other = atomicExch(&visits[p], height + 1);
+            // the box above is written before the arrival, the sibling's read after its own
+            const int other = exchange_acq_rel(&visits[p], height + 1);
             if (other == 0) return;
-            __threadfence();                            // the sibling's box is read after its arrival
             const int64_t sib = left ? b : a;
             for (int c = 0; c < 3; ++c) {
                 slo[c] = __ldcg(&nbox[6 * sib + c]);
