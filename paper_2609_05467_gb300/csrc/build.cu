@@ -1887,7 +1887,7 @@ rc_status sample_points(rc_bvh h, int64_t n, const rc_params* p, float* P, float
         RC_LAUNCHED();
         return RC_OK;
     }
-    const auto kernel = n > 128 * (int64_t)device_sms() ? k_sample_area<true> : k_sample_area<false>;
+    const auto kernel = n > 128 && n > 128 * (int64_t)device_sms() ? k_sample_area<true> : k_sample_area<false>;
     kernel<<<nblocks(n, 256), 256, 0, s>>>(h->V, h->F, h->T, h->cdf, h->host_sc.total, h->fnorm, n, p->seed, P, N, face,
                                            weight);
     RC_LAUNCHED();

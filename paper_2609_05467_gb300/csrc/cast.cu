@@ -1833,6 +1833,8 @@ __device__ __forceinline__ void cast_point(const float4* __restrict__ nodes, con
     const bool whole = t1 < 0;
     if (whole) t1 = W;
     auto* pool = (PoolOf<is_big(kKind)>*)smem + warp;
+    static_assert(4 * sizeof(PoolOf<is_big(kKind)>) >= kMaxDirs / 32 * sizeof(uint32_t),
+                  "the rows' place less a segment's first word lies in the block's shared memory still");
     if (!is_seg(kKind)) {
         cast_point_pooled<kStats, is_big(kKind), false>(nodes, tris, max_steps, scene_maxabs, P, Nrm, i, tdirs, W, eps, pool,
                                                         rows, bits, count, acc, t0, t1, whole, relist, relist_cap, relist_ctr);
