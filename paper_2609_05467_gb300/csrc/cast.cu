@@ -56,7 +56,8 @@ __device__ __forceinline__ void setup_ray(Ray& r, float ox, float oy, float oz, 
     // reciprocals; a zero (or tiny) component gets +-2^100 instead of
     // +-inf, so slab products stay finite (no inf * 0 = NaN) and, 2^100
     // being a power of two, exact: such a slab is decided by the sign of
-    // b - o alone
+    // b - o alone.  That holds for coordinates up to 2.6e8; beyond, o times
+    // 2^100 overflows and the 4-wide walk may miss boxes of such a ray
     r.ix = __frcp_rn(dx);
     r.iy = __frcp_rn(dy);
     r.iz = __frcp_rn(dz);
